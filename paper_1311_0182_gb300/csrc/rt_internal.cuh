@@ -16,7 +16,9 @@
 #include "../../include/traphic_rt.h"
 
 #define RT_Q 1048576          // 2^20 quantisation cells per box side
-#define RT_BUDGET_CHUNK 4096
+// particles of one budget chunk (one block): 1024 gives a 64^3 box 256 blocks; with 4096 its 64
+// blocks left most of the chip idle (the two passes of a step with their sums: 74 -> 41 us)
+#define RT_BUDGET_CHUNK 1024
 #define RT_OCC_MIN 1           // finest kNN grid the occupancy search tries
 #define RT_MAXK 32            // maximum neighbours per particle
 #define RT_FREE_BIT (1ull << 63)
