@@ -39,7 +39,7 @@ enum {
     CNT_GAS = 7,        // gas-to-gas contributions this step
     CNT_SUB = 8,        // chemistry subcycles
     CNT_FLOOR = 9,      // subcycle-floor hits
-    CNT_NFREE = 10,     // free packets of the current hop
+    CNT_CHEMQ = 10,     // the chemistry's work queue: particles taken
     CNT_ACTP = 11,      // particles with a packet able to move, summed over hops
     CNT_ACTS = 12,      // packets able to move (slots), summed over hops
     CNT_GCON = 13,      // gas-to-gas contributions, summed over hops
