@@ -7,6 +7,7 @@
 
 #include "rt_knn.cuh"
 
+// quantised positions, boxes and volumes of the particles (densities and atoms are in place)
 __global__ void k_quantise(DevPtrs P, const double *x, const double *y, const double *z) {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P.n) return;
@@ -30,6 +31,9 @@ __global__ void k_quantise(DevPtrs P, const double *x, const double *y, const do
     }
     P.pbox[i] = lo;
     P.qx[i] = q[0]; P.qy[i] = q[1]; P.qz[i] = q[2];
+    double V = P.NH[i] / P.nH[i] / P.vunit[lo];   // volume in the box's volume unit
+    if (P.fp32) ((float *)P.Vr)[i] = (float)V;
+    else ((double *)P.Vr)[i] = V;
 }
 
 __global__ void k_quantise_src(DevPtrs P, const double *x, const double *y, const double *z) {

@@ -349,24 +349,38 @@ __global__ void k_rebin(DevPtrs P) {
     P.act[cur][key] = no;   // clocks restart: every held packet can move again
 }
 
-// Recombination emission into the reception cones, counter reset, frozen n_HI.
+// the direction of a set opposite to direction b (both sets are symmetric about the origin)
+__device__ __forceinline__ int axis_opposite(int nax, int b) {
+    if (nax == 8) return 7 - b;
+    if (b >= 12 && b < 20) return 31 - b;   // the cube diagonals of the 32: 12 + (7 - (b - 12))
+    return b ^ 3;                           // vertex groups of four: both signs flip
+}
+
+// Recombination emission into the reception cones, deposit reset, frozen n_HI.  Bound by the
+// deposit words it clears and by FP64 (16 cycles of an SM per warp instruction): the words are
+// cleared key by key across the grid (coalesced, and only those the packet precision uses), the
+// rotated axes are computed for one of each opposite pair, and the particles' volumes, which a
+// step does not change, come from the upload.  512,000 particles, 9 bins, no emission: 246 ->
+// 41 us; the 64^3 HII region, 32 cones: 420 -> 203 us.
 template <typename Real, int NRC>
 __global__ void k_emit_rec(DevPtrs P) {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    for (long long key = i; key < P.n * P.nf; key += (long long)gridDim.x * blockDim.x) {
+        if (sizeof(Real) == 8) {
+            P.abs[key] = 0.0; P.absE[key] = 0.0; P.pass[key] = 0.0;
+        } else {
+            P.passf[key] = 0.0f;
+        }
+        P.fx_abs[key] = 0ull; P.fx_lo[key] = 0ull; P.fx_E[key] = 0ull;
+    }
     if (i >= P.n) return;
     int cur = (int)P.cnt[CNT_CUR];
     int b = P.pbox[i];
     double nm = P.norm[b];
-    for (int nu = 0; nu < P.nf; ++nu) {
-        long long key = i * P.nf + nu;
-        P.abs[key] = 0.0; P.absE[key] = 0.0; P.pass[key] = 0.0;
-        P.fx_abs[key] = 0ull; P.fx_lo[key] = 0ull; P.fx_E[key] = 0ull; P.passf[key] = 0.0f;
-    }
     double x = P.xHI[i], nH = P.nH[i], NH = P.NH[i];
     double nHI = __dmul_rn(x, nH);
     P.nHI[i] = nHI;
     ((Real *)P.nHIr)[i] = (Real)nHI;
-    ((Real *)P.Vr)[i] = (Real)(NH / nH / P.vunit[b]);   // volume in the box's volume unit
     double NHI = x * NH;
     ((Real *)P.dep_s)[i] = NHI > 0.0 ? (Real)(FX_ABS_SCALE * nm / NHI) : Real(0);
     ((Real *)P.depE_s)[i] = NHI > 0.0 ? (Real)(FX_E_SCALE * nm * P.eunit / (NHI * EV_ERG)) : Real(0);
@@ -383,21 +397,34 @@ __global__ void k_emit_rec(DevPtrs P) {
     // shared bin: each cone gains e sigma_rec of cross-section sum
     Real *SG = P.shared ? (Real *)P.slG[cur] + i * NRC : nullptr;
     Real eg = e * (Real)(P.sigma_rec / P.sunit);
-    const double *R = P.R + i * 9;
-    for (int bb = 0; bb < NRC; ++bb) {
-        double A[3];
-        rot_apply(R, c_axd[P.ax_rc] + 3 * bb, A);
+    double R[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) R[k] = P.R[i * 9 + k];
+    auto emit = [&](int bb, Real A0, Real A1, Real A2) {
         long long s = s0 + bb;
         if ((o >> bb) & 1) {
-            S.N[s] += e; S.X[s] += e * (Real)A[0]; S.Y[s] += e * (Real)A[1];
-            S.Z[s] += e * (Real)A[2]; S.E[s] += e * epsr;
+            S.N[s] += e; S.X[s] += e * A0; S.Y[s] += e * A1;
+            S.Z[s] += e * A2; S.E[s] += e * epsr;
             if (SG) SG[bb] += eg;
         } else {
-            S.N[s] = e; S.X[s] = e * (Real)A[0]; S.Y[s] = e * (Real)A[1];
-            S.Z[s] = e * (Real)A[2]; S.C[s] = Real(0); S.E[s] = e * epsr;
+            S.N[s] = e; S.X[s] = e * A0; S.Y[s] = e * A1;
+            S.Z[s] = e * A2; S.C[s] = Real(0); S.E[s] = e * epsr;
             if (SG) SG[bb] = eg;
         }
-        if (e > Real(0)) { o |= 1u << bb; a |= 1u << bb; }
+    };
+    for (int bb = 0; bb < NRC; ++bb) {
+        int ob = axis_opposite(NRC, bb);
+        if (ob < bb) continue;
+        double A[3];
+        rot_apply(R, c_axd[P.ax_rc] + 3 * bb, A);
+        Real A0 = (Real)A[0], A1 = (Real)A[1], A2 = (Real)A[2];
+        emit(bb, A0, A1, A2);
+        emit(ob, -A0, -A1, -A2);
+    }
+    if (e > Real(0)) {
+        const unsigned all = NRC == 32 ? FULLMASK : (1u << (NRC & 31)) - 1u;
+        o |= all;
+        a |= all;
     }
     P.occ[cur][key] = o;
     P.act[cur][key] = a;
