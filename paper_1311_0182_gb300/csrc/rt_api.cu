@@ -347,7 +347,7 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     A(P.fdx, float, n * P.kn); A(P.fdy, float, n * P.kn); A(P.fdz, float, n * P.kn);
     A(P.rev_off, int, n + 1);
     A(P.rev_ent, unsigned, n * P.kn);
-    A(P.rdx, float, n * P.kn); A(P.rdy, float, n * P.kn); A(P.rdz, float, n * P.kn);
+    A(P.rev4, float4, n * P.kn);
     A(P.grid.G, int, n_boxes);
     A(P.grid.cs, int, n_boxes);
     A(P.grid.coff, long long, n_boxes);

@@ -184,7 +184,7 @@ struct DevPtrs {              // plain pointers handed to kernels (by value)
     float *fdx, *fdy, *fdz;   // forward offsets q_j - q_i, [n * kn]
     int *rev_off;
     unsigned *rev_ent;        // (i << 5) | k
-    float *rdx, *rdy, *rdz;   // offsets in reverse order
+    float4 *rev4;             // the same order: offset q_j - q_i, and the sender i (its bits)
     Grid grid;
     // rotations
     double *R, *Rs;

@@ -186,9 +186,7 @@ __global__ void k_rev_sort(DevPtrs P) {
         unsigned v = P.rev_ent[p];
         long long f = (long long)(v >> 5) * P.kn + (v & 31);
         P.revpos[f] = p;
-        P.rdx[p] = P.fdx[f];
-        P.rdy[p] = P.fdy[f];
-        P.rdz[p] = P.fdz[f];
+        P.rev4[p] = make_float4(P.fdx[f], P.fdy[f], P.fdz[f], __int_as_float((int)(v >> 5)));
     }
 }
 

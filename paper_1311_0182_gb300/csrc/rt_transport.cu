@@ -11,10 +11,10 @@
 //      escape test, exact kNN of the point, SPH-interpolated n_HI, attenuation; absorptions
 //      go to the neighbours as fixed-point integer sums (order-independent, so reproducible);
 //      the transmitted packet becomes a free packet of the next hop.
-//   B  receiver side, group of n_rc lanes per (particle, nu), lane = reception cone: walks the
-//      particle's reverse neighbour list in sender order, expands the bitmap bits into
-//      contributions, attenuates, picks the reception cone, and merges in a fixed order
-//      (sender, slot); then the staged free-packet contributions in (packet, neighbour) order.
+//   B  receiver side, a warp per four groups (particle, nu): walks the particles' reverse
+//      neighbour lists in sender order, expands the bitmap bits into contributions, attenuates
+//      (lane = contribution), picks the reception cone, and merges in a fixed order (sender,
+//      slot); then the staged free-packet contributions in (packet, neighbour) order.
 //      No floating-point atomics: every sum has one fixed order.
 #include <algorithm>
 #include <climits>
@@ -1150,219 +1150,542 @@ __device__ __forceinline__ unsigned long long deposit_group<float>(const DevPtrs
     return old;
 }
 
-// Receiver side.  Group of G = n_rc lanes per (particle j, frequency nu); lane = reception
-// cone.  Contributions are computed in parallel and merged in their fixed order by a
-// broadcast loop (the lane owning the target cone adds).  Groups come from the work list;
-// the next buffer's occupancy words were cleared by the work-list kernel.
-// cur: the slot buffer holding the hop's packets.
+// What the receiver side keeps of one contribution: T, T d (3), T clock, T eps, then A, A eps
+// and w, and T sigma in a shared frequency bin.
+template <bool SH> struct BVals { static constexpr int N = SH ? 10 : 9; };
+
+// One gas contribution to receiver j in frequency nu: reverse edge e, bit b of its word.
+// Attenuates, stores the values in sv[.][lane] and returns its reception cone, or -1 when a
+// barrier removed it (counted escaped).
+template <typename Real, int G, bool BAR, bool SH>
+__device__ __forceinline__ int gas_contribution(const DevPtrs &P, long long e, int b, long long j,
+                                                int nu, int box, Real u, Real sig_nhi,
+                                                Real (*sv)[32], int lane) {
+    float4 ed = __ldg(P.rev4 + e);
+    bool sgs = SH && nu == 0;
+    Real w, d0, d1, d2, clk, eps, sgc = Real(0);
+    rec_load(P.rec, (long long)__float_as_int(ed.w) * P.S + (long long)nu * G + b, w, d0, d1, d2,
+             clk, eps, sgs, sgc);
+    if (BAR) {
+        int jx = P.qx[j], jy = P.qy[j], jz = P.qz[j];
+        if (barrier_crosses_call(P.bar[box], jx - (int)ed.x, jy - (int)ed.y, jz - (int)ed.z, jx,
+                                 jy, jz)) {
+            atomicAdd(&P.esc_fx[box], esc_fixed(w, P, box));
+            return -1;
+        }
+    }
+    Real t = (Real)ed.x * d0 + (Real)ed.y * d1 + (Real)ed.z * d2;
+    Real l = t * u;
+    Real A, T;
+    // in a shared bin each packet carries its own mean cross-section
+    Real sn = sgs ? (sgc * (Real)P.sunit) * ((Real *)P.nHIr)[j] : sig_nhi;
+    split_absorbed<Real>(w, sn * l, A, T);
+    sv[0][lane] = T;
+    sv[1][lane] = T * d0;
+    sv[2][lane] = T * d1;
+    sv[3][lane] = T * d2;
+    sv[4][lane] = T * (clk + l / (Real)C_LIGHT);
+    sv[5][lane] = T * eps;
+    sv[6][lane] = A;
+    sv[7][lane] = A * eps;
+    sv[8][lane] = w;
+    if (sgs) sv[SH ? 9 : 0][lane] = T * sgc;
+    return bin_fast<Real>(P.Rf + j * 9, P.R + j * 9, P.ax_rc, G, d0, d1, d2);
+}
+
+// A staged free-packet contribution: its values into sv[.][lane], its cone (-1: removed).
+template <typename Real, bool SH>
+__device__ __forceinline__ int staged_contribution(const DevPtrs &P, int s, int nu,
+                                                   Real (*sv)[32], int lane) {
+    Real *const *V = (Real *const *)P.st_v;
+    int bin = P.st_bin[s];
+    if (bin >= 0) {
+#pragma unroll
+        for (int f = 0; f < 9; ++f) sv[f][lane] = V[f][s];
+        if (SH && nu == 0) sv[SH ? 9 : 0][lane] = V[9][s];
+    }
+    return bin;
+}
+
+// the merged packet of one reception cone: N, N d, N clock, N eps (and N sigma, shared bin)
+template <typename Real, bool SH> struct ConeSum {
+    KSum<Real> N, X, Y, Z, C, E, G;
+    __device__ __forceinline__ void zero() {
+        N.init(Real(0)); X.init(Real(0)); Y.init(Real(0)); Z.init(Real(0)); C.init(Real(0));
+        E.init(Real(0)); G.init(Real(0));
+    }
+    __device__ __forceinline__ void add(Real (*sv)[32], int t, bool sgs) {
+        N.add(sv[0][t]); X.add(sv[1][t]); Y.add(sv[2][t]); Z.add(sv[3][t]); C.add(sv[4][t]);
+        E.add(sv[5][t]);
+        if (sgs) G.add(sv[SH ? 9 : 0][t]);
+    }
+    // a packet that waited in the cone
+    __device__ __forceinline__ void load(const Slots<Real> &S, const Real *SG, long long s,
+                                         long long g, bool sgs) {
+        N.init(S.N[s]); X.init(S.X[s]); Y.init(S.Y[s]); Z.init(S.Z[s]); C.init(S.C[s]);
+        E.init(S.E[s]);
+        G.init(sgs ? SG[g] : Real(0));
+    }
+    __device__ __forceinline__ void store(const Slots<Real> &S, Real *SG, long long s, long long g,
+                                          bool sgs) const {
+        S.N[s] = N.get(); S.X[s] = X.get(); S.Y[s] = Y.get(); S.Z[s] = Z.get(); S.C[s] = C.get();
+        S.E[s] = E.get();
+        if (sgs) SG[g] = G.get();
+    }
+};
+
+// number of set bits of each byte
+__device__ __forceinline__ unsigned byte_popc(unsigned x) {
+    x = x - ((x >> 1) & 0x55555555u);
+    x = (x & 0x33333333u) + ((x >> 2) & 0x33333333u);
+    return (x + (x >> 4)) & 0x0f0f0f0fu;
+}
+// inclusive prefix sum over the lanes (of packed fields that do not overflow)
+__device__ __forceinline__ unsigned lane_scan(unsigned v) {
+    int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        unsigned t = __shfl_up_sync(FULLMASK, v, o);
+        if (lane >= o) v += t;
+    }
+    return v;
+}
+
+// One receiver group of 32 cones by a whole warp, lane = reception cone, whatever its number of
+// edges, contributions and waiting packets: edges 32 at a time, contributions 32 at a time,
+// each cone's lane adding its contributions in list order.
+template <typename Real, bool BAR, bool SH>
+__device__ __forceinline__ void wide_group(const DevPtrs &P, int cur, long long key, bool touched,
+                                           int fc, int so, Real (*sv)[32], unsigned *list,
+                                           unsigned *smask, unsigned long long &pend, bool &bad) {
+    const int lane = threadIdx.x & 31;
+    const int j = (int)((unsigned)key / (unsigned)P.nf), nu = (int)((unsigned)key % (unsigned)P.nf);
+    const int box = P.pbox[j];
+    const unsigned park = P.occ[cur][key] & ~P.act[cur][key];
+    const bool sgs = SH && nu == 0;
+    const long long sidx = (long long)j * P.S + (long long)nu * 32 + lane;
+    const long long gidx = (long long)j * 32 + lane;
+    ConeSum<Real, SH> a;
+    a.zero();
+    if ((park >> lane) & 1u) a.load(Slots<Real>(P, cur), (const Real *)P.slG[cur], sidx, gidx, sgs);
+    KSum<Real> sA, sAE, sW;
+    sA.init(Real(0)); sAE.init(Real(0)); sW.init(Real(0));
+    auto merge = [&](int bin) {
+        smask[lane] = 0u;
+        __syncwarp();
+        if (bin >= 0) {
+            atomicOr(&smask[bin], 1u << lane);
+            sA.add(sv[6][lane]); sAE.add(sv[7][lane]); sW.add(sv[8][lane]);
+        }
+        __syncwarp();
+        unsigned m = smask[lane];
+        while (m) {
+            int t = __ffs(m) - 1;
+            m &= m - 1u;
+            a.add(sv, t, sgs);
+        }
+        __syncwarp();
+    };
+    if (touched) {
+        const Real u = box_unit<Real>(P, box);
+        const Real sig_nhi = sigma_of<Real>(P, nu) * ((Real *)P.nHIr)[j];
+        const int e0 = P.rev_off[j], e1 = P.rev_off[j + 1];
+        unsigned *bmr = P.bm + (long long)nu * P.n * P.kn;
+        for (int eb = e0; eb < e1; eb += 32) {
+            unsigned word = 0u;
+            if (eb + lane < e1) {
+                word = bmr[eb + lane];
+                if (word) bmr[eb + lane] = 0u;
+            }
+            const unsigned cw = (unsigned)__popc(word);
+            const unsigned incl = lane_scan(cw);
+            const int total = (int)__shfl_sync(FULLMASK, incl, 31);
+            for (int cb = 0; cb < total; cb += 32) {
+                int p = (int)(incl - cw) - cb;
+                for (unsigned x = word; x; x &= x - 1u, ++p)
+                    if (p >= 0 && p < 32) list[p] = (unsigned)(__ffs(x) - 1) | (unsigned)lane << 5;
+                __syncwarp();
+                const bool has = cb + lane < total;
+                const unsigned code = has ? list[lane] : 0u;
+                int bin = -1;
+                if (has)
+                    bin = gas_contribution<Real, 32, BAR, SH>(P, (long long)eb + (code >> 5), code & 31u, j,
+                                                              nu, box, u, sig_nhi, sv, lane);
+                merge(bin);
+            }
+        }
+    }
+    for (int cb = 0; cb < fc; cb += 32) {
+        int bin = -1;
+        if (cb + lane < fc)
+            bin = staged_contribution<Real, SH>(P, P.seg_idx[so + cb + lane], nu, sv, lane);
+        merge(bin);
+    }
+    const Real N = a.N.get();
+    const bool occ = N > Real(0);
+    const bool act = occ && (a.C.get() / N < (Real)P.dt);
+    const unsigned bo = __ballot_sync(FULLMASK, occ), ba = __ballot_sync(FULLMASK, act);
+    if (occ) a.store(Slots<Real>(P, cur ^ 1), (Real *)P.slG[cur ^ 1], sidx, gidx, sgs);
+    Real av = sA.get(), ae = sAE.get(), w = sW.get();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        av += __shfl_down_sync(FULLMASK, av, o);
+        ae += __shfl_down_sync(FULLMASK, ae, o);
+        w += __shfl_down_sync(FULLMASK, w, o);
+    }
+    if (lane == 0) {
+        P.occ[cur ^ 1][key] = bo;
+        P.act[cur ^ 1][key] = ba;
+        if (touched || fc > 0) {
+            bad |= pend > (1ull << 62);
+            pend = deposit_group<Real>(P, key, j, box, av, ae, w);
+        }
+    }
+}
+
+// Receiver side.  A warp takes four receiver groups (particle j, frequency nu) of the work list
+// at a time, expands the bitmap bits of their reverse edges into one list of contributions, and
+// computes 32 contributions of that list at a time, one per lane: gathering a sender's record,
+// attenuation, reception cone.  Then the contributions are merged in their fixed order (sender,
+// slot; staged ones after them in packet order): the lane owning a target cone adds them.
+// What bounds it: instructions and the latency of the gathers.  A group has few contributions
+// (8.6 with 8 cones behind a fast front, 3.8 with 32 cones in the HII region), so a group of
+// n_rc lanes of its own left most lanes idle in the long part, the contributions
+// (13.6 of 32 active); four groups share a pass here.  Measured per step against a
+// group of n_rc lanes each: 64^3 HII region, 32 cones, 17.5 -> 10.7 ms, the FP64 path at 32^3
+// 6.8 -> 3.5 ms; 2.1 M particles behind a fast front, 8 cones, 189 -> 132 ms.
+//   8 cones: lane = (group, cone), so the four groups' 32 cones stay in registers whatever the
+//   number of contributions.
+//   32 cones: groups of at most 32 contributions in all are merged together, the lowest lane of
+//   each (group, cone) adding; a group of more (or of waiting packets, or of more than 64
+//   edges) has enough work for a warp of its own (wide_group).
+// Each sum keeps the order and the tree that one lane per cone and contribution gives: the
+// absorption sums of a group are Kahan sums per lane (position of the contribution in its run
+// of n_rc edges, modulo n_rc), then a tree over the lanes.  Results do not depend on how
+// groups meet in a warp.
+// Groups come from the work list; the next buffer's occupancy words were cleared by the
+// work-list kernel.  cur: the slot buffer holding the hop's packets.
 template <typename Real, int G, bool BAR, bool SH>
 __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int cur, const int *wl_n) {
-    // contributions of the current chunk, one per lane: 6 values (T, T d, T clock, T eps), and
-    // T sigma in a shared frequency bin; and per reception cone of each group, the mask of the
-    // chunk's lanes that feed it
-    __shared__ Real sv[SH ? 7 : 6][256];
-    __shared__ unsigned sm[256];
-    // the current chunk of reverse edges: offset and sender; bitmap word and first
-    // contribution; and per contribution chunk, the edge lane where each range starts
-    __shared__ float4 se[256];
-    __shared__ uint2 sw2[256];
-    __shared__ int sown[256];
-    int gl = threadIdx.x & (G - 1);
-    int gbase = threadIdx.x - gl;               // first thread of this group in the block
-    unsigned base = (threadIdx.x & 31) & ~(unsigned)(G - 1);
-    unsigned gmask = (G == 32) ? FULLMASK : (((1u << G) - 1u) << base);
-    long long ng = *wl_n;
-    int nxt = cur ^ 1;
-    // each block takes one contiguous chunk of the work list; its groups pull entries from it
-    // through a shared counter, so that they finish together
+    __shared__ Real svs[8][BVals<SH>::N][32];
+    __shared__ unsigned slist[8][32];
+    __shared__ unsigned smask[8][2][32];
     __shared__ int snext;
-    long long chunk = (ng + gridDim.x - 1) / gridDim.x;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    Real (*sv)[32] = svs[wid];
+    unsigned *list = slist[wid];
+    const int kq = lane >> 3;                  // the lane's group of the four
+    const int nxt = cur ^ 1;
+    // each block takes one contiguous chunk of the work list, in fours; its warps pull from it
+    // through a shared counter, so that they finish together
+    long long ng = *wl_n;
+    long long chunk = ((ng + gridDim.x - 1) / gridDim.x + 3) & ~3ll;
     long long gb0 = (long long)blockIdx.x * chunk;
     long long gb1 = gb0 + chunk < ng ? gb0 + chunk : ng;
     if (threadIdx.x == 0) snext = 0;
     __syncthreads();
-    auto next_group = [&]() {
-        long long v = 0;
-        if (gl == 0) v = gb0 + atomicAdd(&snext, 1);
-        return __shfl_sync(gmask, v, 0, G);
-    };
     unsigned long long pend = 0ull;   // the high absorption word before the last deposit
     bool bad = false;
-    for (long long gi = next_group(); gi < gb1; gi = next_group()) {
-        unsigned wv = (unsigned)P.worklist[gi];
-        long long key = wv & 0x7fffffffu;
-        bool touched = (wv >> 31) != 0u;
-        long long j = (unsigned)key / (unsigned)P.nf;
-        int nu = (int)((unsigned)key % (unsigned)P.nf);
-        unsigned park = P.occ[cur][key] & ~P.act[cur][key];
-        int fc = P.seg_cnt[key];
+    for (;;) {
+        long long g0 = 0;
+        if (lane == 0) g0 = gb0 + atomicAdd(&snext, 4);
+        g0 = __shfl_sync(FULLMASK, g0, 0);
+        if (g0 >= gb1) break;
+        // the group of each eight lanes
+        const bool kv = g0 + kq < gb1;
+        const unsigned wv = kv ? (unsigned)P.worklist[g0 + kq] : 0u;
+        const long long key = wv & 0x7fffffffu;
+        const bool touched = (wv >> 31) != 0u;
+        const int j = (int)((unsigned)key / (unsigned)P.nf);
+        const int nu = (int)((unsigned)key % (unsigned)P.nf);
+        const unsigned park = kv ? P.occ[cur][key] & ~P.act[cur][key] : 0u;
+        const int fc = kv ? P.seg_cnt[key] : 0;
+        const int so = fc > 0 ? P.seg_off[key] : 0;
+        const int e0 = touched ? P.rev_off[j] : 0;
+        const int ne = touched ? P.rev_off[j + 1] - e0 : 0;
+        const int box = P.pbox[j];
+        const Real u = box_unit<Real>(P, box);
+        const Real sig_nhi = sigma_of<Real>(P, nu) * ((Real *)P.nHIr)[j];
         Slots<Real> So(P, cur), Sn(P, nxt);
-        long long sidx = j * P.S + (long long)nu * G + gl;
-        // a group of the shared frequency bin also merges the cross-section sums
-        bool sgs = SH && nu == 0;
-        long long gidx = j * G + gl;
-        KSum<Real> aN, aX, aY, aZ, aC, aE, aG, sA, sAE, sW;
-        if ((park >> gl) & 1u) {
-            aN.init(So.N[sidx]); aX.init(So.X[sidx]); aY.init(So.Y[sidx]);
-            aZ.init(So.Z[sidx]); aC.init(So.C[sidx]); aE.init(So.E[sidx]);
-            aG.init(sgs ? ((Real *)P.slG[cur])[gidx] : Real(0));
-        } else {
-            aN.init(Real(0)); aX.init(Real(0)); aY.init(Real(0));
-            aZ.init(Real(0)); aC.init(Real(0)); aE.init(Real(0));
-            aG.init(Real(0));
-        }
-        sA.init(Real(0)); sAE.init(Real(0)); sW.init(Real(0));
-        int box = P.pbox[j];
-        // merge this chunk's contributions: lane gl of the group holds one for reception cone
-        // mybin (-1: none).  Lanes of equal cone find each other (match), the lowest of them
-        // publishes the set, and lane b adds the contributions to cone b in lane order.
-        auto merge_chunk = [&](int mybin) {
-            unsigned peers = __match_any_sync(gmask, mybin >= 0 ? mybin : G + gl);
-            sm[threadIdx.x] = 0u;
-            __syncwarp(gmask);
-            if (mybin >= 0 && (peers & ((1u << (threadIdx.x & 31)) - 1u)) == 0u)
-                sm[gbase + mybin] = peers >> base;
-            __syncwarp(gmask);
-            unsigned m = sm[threadIdx.x];
-            while (m) {
-                int t2 = gbase + __ffs(m) - 1;
-                m &= m - 1u;
-                aN.add(sv[0][t2]); aX.add(sv[1][t2]); aY.add(sv[2][t2]);
-                aZ.add(sv[3][t2]); aC.add(sv[4][t2]); aE.add(sv[5][t2]);
-                if (sgs) aG.add(sv[SH ? 6 : 0][t2]);
-            }
-            __syncwarp(gmask);
-        };
-        if (touched) {
-            Real u = box_unit<Real>(P, box);
-            Real sig_nhi = sigma_of<Real>(P, nu) * ((Real *)P.nHIr)[j];
-            const float *Rf = P.Rf + j * 9;
-            const double *Rd = P.R + j * 9;
-            int e0 = P.rev_off[j], e1 = P.rev_off[j + 1];
-            unsigned *bmr = P.bm + (long long)nu * P.n * P.kn;
-            for (int eb = e0; eb < e1; eb += G) {
-                int e = eb + gl;
-                unsigned word = 0u;
-                int si = 0;
-                float fx = 0.f, fy = 0.f, fz = 0.f;
-                unsigned xb = 0u;   // 1u << 31: the edge's path crosses the box's barrier
-                if (e < e1) {   // the edge's data is loaded with its word (one memory round)
-                    word = bmr[e];
-                    si = (int)(P.rev_ent[e] >> 5);
-                    fx = P.rdx[e]; fy = P.rdy[e]; fz = P.rdz[e];
-                    if (word) bmr[e] = 0u;
-                    if (BAR && word) {
-                        int jx = P.qx[j], jy = P.qy[j], jz = P.qz[j];
-                        if (barrier_crosses_call(P.bar[box], jx - (int)fx, jy - (int)fy,
-                                                 jz - (int)fz, jx, jy, jz))
-                            xb = 1u << 31;
-                    }
+        // a group's values to the lanes that work on it
+        auto of = [&](auto v, int k) { return __shfl_sync(FULLMASK, v, 8 * k); };
+        if constexpr (G == 8) {
+            const int bl = lane & 7;
+            const long long sidx = (long long)j * P.S + (long long)nu * G + bl;
+            const long long gidx = (long long)j * G + bl;
+            const bool sgs = SH && nu == 0;
+            ConeSum<Real, SH> a;
+            a.zero();
+            if ((park >> bl) & 1u) a.load(So, (const Real *)P.slG[cur], sidx, gidx, sgs);
+            KSum<Real> sA, sAE, sW;
+            sA.init(Real(0)); sAE.init(Real(0)); sW.init(Real(0));
+            // merge the contributions of the lanes: group kk, cone bin (-1: none), and the lane
+            // ol of the group's absorption sums
+            auto merge = [&](int kk, int bin, int ol) {
+                smask[wid][0][lane] = 0u;
+                smask[wid][1][lane] = 0u;
+                __syncwarp();
+                if (bin >= 0) {
+                    atomicOr(&smask[wid][0][8 * kk + bin], 1u << lane);
+                    atomicOr(&smask[wid][1][8 * kk + ol], 1u << lane);
                 }
-                int cw = __popc(word);
-                int incl = cw;
+                __syncwarp();
+                unsigned m = smask[wid][0][lane], m2 = smask[wid][1][lane];
+                while (m) {
+                    int t = __ffs(m) - 1;
+                    m &= m - 1u;
+                    a.add(sv, t, sgs);
+                }
+                while (m2) {
+                    int t = __ffs(m2) - 1;
+                    m2 &= m2 - 1u;
+                    sA.add(sv[6][t]); sAE.add(sv[7][t]); sW.add(sv[8][t]);
+                }
+                __syncwarp();
+            };
+            const int nemax = __reduce_max_sync(FULLMASK, ne);
+            for (int eb = 0; eb < nemax; eb += 64) {
+                // lane: edges 2 lane and 2 lane + 1 of the block; the four groups' words, eight
+                // bits each, in one register per edge
+                unsigned w0[4], w1[4];
+                unsigned *bw[4];
 #pragma unroll
-                for (int o = 1; o < G; o <<= 1) {
-                    int v = __shfl_up_sync(gmask, incl, o, G);
-                    if (gl >= o) incl += v;
+                for (int kk = 0; kk < 4; ++kk) {
+                    int rem = of(ne, kk) - eb - 2 * lane;
+                    bw[kk] = P.bm + (long long)of(nu, kk) * P.n * P.kn + of(e0, kk) + eb + 2 * lane;
+                    w0[kk] = rem > 0 ? bw[kk][0] : 0u;
+                    w1[kk] = rem > 1 ? bw[kk][1] : 0u;
                 }
-                int total = __shfl_sync(gmask, incl, G - 1, G);
-                int excl = incl - cw;
-                // the chunk's edges in shared memory; contribution c belongs to the edge whose
-                // range [excl, excl + cw) holds it
-                se[threadIdx.x] = make_float4(fx, fy, fz, __int_as_float(si));
-                sw2[threadIdx.x] = make_uint2(word, (unsigned)excl | xb);
-                int carry = 0;   // owner of the last contribution of the previous chunk
-                for (int cb = 0; cb < total; cb += G) {
-                    bool st = cw > 0 && excl >= cb && excl < cb + G;
-                    if (st) sown[gbase + excl - cb] = gl;
-                    unsigned smk = __reduce_or_sync(gmask, st ? 1u << (excl - cb) : 0u);
-                    __syncwarp(gmask);
-                    unsigned below = smk & (0xffffffffu >> (31 - gl));
-                    int own = below ? sown[gbase + 31 - __clz(below)] : carry;
-                    carry = __shfl_sync(gmask, own, G - 1, G);
-                    int c = cb + gl;
-                    int mybin = -1;
-                    bool keep = c < total;
-                    Real w, d0, d1, d2, clk, eps, sgc = Real(0);
-                    float4 ed;
-                    if (keep) {
-                        ed = se[gbase + own];
-                        uint2 ow = sw2[gbase + own];
-                        int bsrc = __fns(ow.x, 0, c - (int)(ow.y & 0x7fffffffu) + 1);
-                        long long ridx = (long long)__float_as_int(ed.w) * P.S + (long long)nu * G + bsrc;
-                        rec_load(P.rec, ridx, w, d0, d1, d2, clk, eps, sgs, sgc);
-                        if (ow.y >> 31) {   // through the barrier: removed (counted escaped)
-                            atomicAdd(&P.esc_fx[box], esc_fixed(w, P, box));
-                            keep = false;
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                    if (w0[kk]) bw[kk][0] = 0u;
+                    if (w1[kk]) bw[kk][1] = 0u;
+                }
+                const unsigned W0 = w0[0] | w0[1] << 8 | w0[2] << 16 | w0[3] << 24;
+                const unsigned W1 = w1[0] | w1[1] << 8 | w1[2] << 16 | w1[3] << 24;
+                // positions in the list (group after group, edge order): 16-bit fields, groups
+                // 0, 1 and 2, 3
+                const unsigned cnt = byte_popc(W0) + byte_popc(W1);
+                const unsigned cl = __byte_perm(cnt, 0u, 0x4140), ch = __byte_perm(cnt, 0u, 0x4342);
+                const unsigned il = lane_scan(cl), ih = lane_scan(ch);
+                const unsigned tl = __shfl_sync(FULLMASK, il, 31), th = __shfl_sync(FULLMASK, ih, 31);
+                const unsigned o1 = tl & 0xffffu, o2 = o1 + (tl >> 16), o3 = o2 + (th & 0xffffu);
+                const int total = (int)(o3 + (th >> 16));
+                const unsigned xl = il - cl, xh = ih - ch;
+                // position in the run of eight edges
+                const unsigned ql0 = xl - __shfl_sync(FULLMASK, xl, lane & ~3);
+                const unsigned qh0 = xh - __shfl_sync(FULLMASK, xh, lane & ~3);
+                for (int cb = 0; cb < total; cb += 32) {
+                    unsigned pl = xl + (o1 << 16), ph = xh + (o2 | o3 << 16), ql = ql0, qh = qh0;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        unsigned x = h ? W1 : W0;
+                        while (x) {
+                            int q = __ffs(x) - 1;
+                            x &= x - 1u;
+                            int sh = (q & 8) << 1;
+                            unsigned one = 1u << sh, p, ol;
+                            if (q < 16) {
+                                p = (pl >> sh) & 0xffffu; ol = (ql >> sh) & 7u;
+                                pl += one; ql += one;
+                            } else {
+                                p = (ph >> sh) & 0xffffu; ol = (qh >> sh) & 7u;
+                                ph += one; qh += one;
+                            }
+                            p -= (unsigned)cb;
+                            if (p < 32u)
+                                list[p] = (unsigned)q | (unsigned)(2 * lane + h) << 5 | ol << 11;
                         }
                     }
-                    if (keep) {
-                        Real t = (Real)ed.x * d0 + (Real)ed.y * d1 + (Real)ed.z * d2;
-                        Real l = t * u;
-                        Real A, T;
-                        // in a shared bin each packet carries its own mean cross-section
-                        Real sn = sgs ? (sgc * (Real)P.sunit) * ((Real *)P.nHIr)[j] : sig_nhi;
-                        split_absorbed<Real>(w, sn * l, A, T);
-                        sA.add(A);
-                        sAE.add(A * eps);
-                        sW.add(w);
-                        mybin = bin_fast<Real>(Rf, Rd, P.ax_rc, G, d0, d1, d2);
-                        sv[0][threadIdx.x] = T;
-                        sv[1][threadIdx.x] = T * d0;
-                        sv[2][threadIdx.x] = T * d1;
-                        sv[3][threadIdx.x] = T * d2;
-                        sv[4][threadIdx.x] = T * (clk + l / (Real)C_LIGHT);
-                        sv[5][threadIdx.x] = T * eps;
-                        if (sgs) sv[SH ? 6 : 0][threadIdx.x] = T * sgc;
-                    }
-                    merge_chunk(mybin);
+                    __syncwarp();
+                    const bool has = cb + lane < total;
+                    const unsigned code = has ? list[lane] : 0u;
+                    const int kk = (int)((code >> 3) & 3u);
+                    const int jk = of(j, kk), nuk = of(nu, kk), boxk = of(box, kk), e0k = of(e0, kk);
+                    const Real uk = of(u, kk), sk = of(sig_nhi, kk);
+                    int bin = -1;
+                    if (has)
+                        bin = gas_contribution<Real, G, BAR, SH>(P, (long long)e0k + eb + ((code >> 5) & 63u),
+                                                                 code & 7u, jk, nuk, boxk, uk, sk, sv, lane);
+                    merge(kk, bin, (int)(code >> 11));
                 }
             }
-        }
-        if (fc > 0) {
-            int so = P.seg_off[key];
-            Real *const *V = (Real *const *)P.st_v;
-            for (int cb = 0; cb < fc; cb += G) {
-                int c = cb + gl;
-                int mybin = -1;
-                if (c < fc) {
-                    int s = P.seg_idx[so + c];
-                    mybin = P.st_bin[s];           // -1: removed by a barrier
-                    if (mybin >= 0) {
-                        for (int f = 0; f < 6; ++f) sv[f][threadIdx.x] = V[f][s];
-                        if (sgs) sv[SH ? 6 : 0][threadIdx.x] = V[9][s];
-                        sA.add(V[6][s]);
-                        sAE.add(V[7][s]);
-                        sW.add(V[8][s]);
-                    }
-                }
-                merge_chunk(mybin);
+            // the staged contributions, group after group
+            const int f1 = of(fc, 0), f2 = f1 + of(fc, 1), f3 = f2 + of(fc, 2), ft = f3 + of(fc, 3);
+            for (int cb = 0; cb < ft; cb += 32) {
+                const int p = cb + lane;
+                const int kk = (p >= f1) + (p >= f2) + (p >= f3);
+                const int c = p - (kk == 0 ? 0 : kk == 1 ? f1 : kk == 2 ? f2 : f3);
+                const int sok = of(so, kk), nuk = of(nu, kk);
+                int bin = -1;
+                if (p < ft) bin = staged_contribution<Real, SH>(P, P.seg_idx[sok + c], nuk, sv, lane);
+                merge(kk, bin, c & 7);
             }
-        }
-        Real N = aN.get();
-        bool occ = N > Real(0);
-        bool act = occ && (aC.get() / N < (Real)P.dt);
-        unsigned lmask = (G == 32) ? FULLMASK : ((1u << G) - 1u);
-        unsigned bo = (__ballot_sync(gmask, occ) >> base) & lmask;
-        unsigned ba = (__ballot_sync(gmask, act) >> base) & lmask;
-        if (occ) {
-            Sn.N[sidx] = N; Sn.X[sidx] = aX.get(); Sn.Y[sidx] = aY.get();
-            Sn.Z[sidx] = aZ.get(); Sn.C[sidx] = aC.get(); Sn.E[sidx] = aE.get();
-            if (sgs) ((Real *)P.slG[nxt])[gidx] = aG.get();
-        }
-        Real a = sA.get(), ae = sAE.get(), w = sW.get();
+            // the merged packets
+            const Real N = a.N.get();
+            const bool occ = kv && N > Real(0);
+            const bool act = occ && (a.C.get() / N < (Real)P.dt);
+            const unsigned bo = (__ballot_sync(FULLMASK, occ) >> (8 * kq)) & 0xffu;
+            const unsigned ba = (__ballot_sync(FULLMASK, act) >> (8 * kq)) & 0xffu;
+            if (occ) a.store(Sn, (Real *)P.slG[nxt], sidx, gidx, sgs);
+            Real av = sA.get(), ae = sAE.get(), w = sW.get();
 #pragma unroll
-        for (int o = G >> 1; o > 0; o >>= 1) {
-            a += __shfl_down_sync(gmask, a, o, G);
-            ae += __shfl_down_sync(gmask, ae, o, G);
-            w += __shfl_down_sync(gmask, w, o, G);
-        }
-        if (gl == 0) {
-            P.occ[nxt][key] = bo;
-            P.act[nxt][key] = ba;
-            if (touched || fc > 0) {
-                bad |= pend > (1ull << 62);
-                pend = deposit_group<Real>(P, key, j, box, a, ae, w);
+            for (int o = G >> 1; o > 0; o >>= 1) {
+                av += __shfl_down_sync(FULLMASK, av, o, G);
+                ae += __shfl_down_sync(FULLMASK, ae, o, G);
+                w += __shfl_down_sync(FULLMASK, w, o, G);
+            }
+            if (kv && bl == 0) {
+                P.occ[nxt][key] = bo;
+                P.act[nxt][key] = ba;
+                if (touched || fc > 0) {
+                    bad |= pend > (1ull << 62);
+                    pend = deposit_group<Real>(P, key, j, box, av, ae, w);
+                }
+            }
+        } else {
+            // 32 cones: the words of up to 64 edges of each group (lane: edges 2 lane, 2 lane + 1)
+            unsigned w0[4], w1[4];
+            int nk[4];             // contributions of the group; 33: a warp of its own
+            unsigned cnt = 0u;     // gas contributions of the lane's edges, eight bits a group
+            const bool narrow = kv && park == 0u && ne <= 64;
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                int rem = of((int)narrow, kk) ? of(ne, kk) - 2 * lane : 0;
+                const unsigned *bw = P.bm + (long long)of(nu, kk) * P.n * P.kn + of(e0, kk) + 2 * lane;
+                w0[kk] = rem > 0 ? bw[0] : 0u;
+                w1[kk] = rem > 1 ? bw[1] : 0u;
+            }
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                int pc = __popc(w0[kk]) + __popc(w1[kk]);
+                nk[kk] = __reduce_add_sync(FULLMASK, pc) + of(fc, kk);
+                if (!of((int)narrow, kk) || nk[kk] > 32) {
+                    nk[kk] = 33;
+                    w0[kk] = w1[kk] = 0u;
+                } else {
+                    cnt |= (unsigned)pc << (8 * kk);
+                    unsigned *bw = P.bm + (long long)of(nu, kk) * P.n * P.kn + of(e0, kk) + 2 * lane;
+                    if (w0[kk]) bw[0] = 0u;
+                    if (w1[kk]) bw[1] = 0u;
+                }
+            }
+            const unsigned incl = lane_scan(cnt), excl = incl - cnt;
+            const unsigned tot = __shfl_sync(FULLMASK, incl, 31);
+            const unsigned mid = __shfl_sync(FULLMASK, excl, 16);   // of the first 32 edges
+            const int nvalid = (int)(gb1 - g0 < 4 ? gb1 - g0 : 4);
+            for (int k0 = 0; k0 < nvalid;) {
+                // groups k0 .. k1 - 1 together
+                int k1 = k0, n = 0, ngas = 0;
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)
+                    if (kk == k1 && kk < nvalid && kk >= k0 && n + nk[kk] <= 32) {
+                        n += nk[kk];
+                        ngas += (int)((tot >> (8 * kk)) & 0xffu);
+                        k1 = kk + 1;
+                    }
+                if (k1 == k0) {
+                    wide_group<Real, BAR, SH>(P, cur, of(key, k0), of((int)touched, k0) != 0,
+                                              of(fc, k0), of(so, k0), sv, list, smask[wid][0], pend,
+                                              bad);
+                    ++k0;
+                    continue;
+                }
+                smask[wid][0][lane] = 0u;
+                smask[wid][1][lane] = 0u;
+                // the list: gas contributions group after group (in edge order), then staged
+                // ones; gk, sk, vk: the lane's group's first gas and staged entries, and its
+                // first lane of the absorption sums
+                int goff = 0, soff = ngas, voff = 0;
+                int myk = -1, gk = 0, m0 = 0, m1 = 0, sk = 0, m2 = 0, vk = 0;   // absorption sums
+                int ek = k0, ec = 0;                                             // staged entry
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                    if (kk < k0 || kk >= k1) continue;
+                    int gas = (int)((tot >> (8 * kk)) & 0xffu), half = (int)((mid >> (8 * kk)) & 0xffu);
+                    int st = of(fc, kk);
+                    int M = max(max(half, gas - half), st);
+                    if (lane >= voff && lane < voff + M) {
+                        myk = kk; gk = goff; m0 = half; m1 = gas - half; sk = soff; m2 = st; vk = voff;
+                    }
+                    if (lane >= soff && lane < soff + st) { ek = kk; ec = lane - soff; }
+                    int p = goff + (int)((excl >> (8 * kk)) & 0xffu);
+                    for (unsigned x = w0[kk]; x; x &= x - 1u)
+                        list[p++] = (unsigned)(__ffs(x) - 1) | (unsigned)(2 * lane) << 5 | (unsigned)kk << 11;
+                    for (unsigned x = w1[kk]; x; x &= x - 1u)
+                        list[p++] = (unsigned)(__ffs(x) - 1) | (unsigned)(2 * lane + 1) << 5 | (unsigned)kk << 11;
+                    goff += gas;
+                    soff += st;
+                    voff += M;
+                }
+                __syncwarp();
+                const bool gas = lane < ngas;
+                const unsigned code = gas ? list[lane] : 0u;
+                const int kk = gas ? (int)(code >> 11) : ek;
+                const int jk = of(j, kk), nuk = of(nu, kk), boxk = of(box, kk), e0k = of(e0, kk),
+                          sok = of(so, kk);
+                const Real uk = of(u, kk), snk = of(sig_nhi, kk);
+                int bin = -1;
+                if (gas)
+                    bin = gas_contribution<Real, G, BAR, SH>(P, (long long)e0k + ((code >> 5) & 63u),
+                                                             code & 31u, jk, nuk, boxk, uk, snk, sv, lane);
+                else if (lane < n)
+                    bin = staged_contribution<Real, SH>(P, P.seg_idx[sok + ec], nuk, sv, lane);
+                __syncwarp();
+                // the lowest lane of each (group, cone) adds its contributions in list order
+                const unsigned live = __ballot_sync(FULLMASK, bin >= 0);
+                unsigned peers = __match_any_sync(FULLMASK, bin >= 0 ? 32 * kk + bin : 128 + lane);
+                if (bin >= 0 && (peers & ((1u << lane) - 1u)) == 0u) {
+                    const bool sgs = SH && nuk == 0;
+                    ConeSum<Real, SH> a;
+                    a.zero();
+                    do {
+                        int t = __ffs(peers) - 1;
+                        peers &= peers - 1u;
+                        a.add(sv, t, sgs);
+                    } while (peers);
+                    const Real N = a.N.get();
+                    if (N > Real(0)) {
+                        a.store(Sn, (Real *)P.slG[nxt], (long long)jk * P.S + (long long)nuk * G + bin,
+                                (long long)jk * G + bin, sgs);
+                        atomicOr(&smask[wid][0][kk], 1u << bin);
+                        if (a.C.get() / N < (Real)P.dt) atomicOr(&smask[wid][1][kk], 1u << bin);
+                    }
+                }
+                // absorption sums: lane i of a group's adds the i-th contributions of its two
+                // runs of 32 edges and of its staged ones, then a tree over the lanes
+                KSum<Real> sA, sAE, sW;
+                sA.init(Real(0)); sAE.init(Real(0)); sW.init(Real(0));
+                const int i = lane - vk;
+                auto take = [&](bool on, int t) {
+                    if (on && ((live >> t) & 1u)) { sA.add(sv[6][t]); sAE.add(sv[7][t]); sW.add(sv[8][t]); }
+                };
+                if (myk >= 0) {
+                    take(i < m0, (gk + i) & 31);
+                    take(i < m1, (gk + m0 + i) & 31);
+                    take(i < m2, (sk + i) & 31);
+                }
+                const int M = myk >= 0 ? max(max(m0, m1), m2) : 0;
+                Real av = sA.get(), ae = sAE.get(), w = sW.get();
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    Real v0 = __shfl_down_sync(FULLMASK, av, o), v1 = __shfl_down_sync(FULLMASK, ae, o),
+                         v2 = __shfl_down_sync(FULLMASK, w, o);
+                    if (i + o < M) { av += v0; ae += v1; w += v2; }
+                }
+                __syncwarp();
+                if ((lane & 7) == 0 && kq >= k0 && kq < k1) {
+                    P.occ[nxt][key] = smask[wid][0][kq];
+                    P.act[nxt][key] = smask[wid][1][kq];
+                }
+                const long long keyk = of(key, myk >= 0 ? myk : 0);
+                const int jd = of(j, myk >= 0 ? myk : 0), boxd = of(box, myk >= 0 ? myk : 0);
+                if (myk >= 0 && i == 0) {
+                    bad |= pend > (1ull << 62);
+                    pend = deposit_group<Real>(P, keyk, jd, boxd, av, ae, w);
+                }
+                __syncwarp();
+                k0 = k1;
             }
         }
     }
@@ -1597,11 +1920,11 @@ static void hop_core(rt_ctx *c, cudaStream_t st, long long nfr, int cur, int fcu
     cudaStreamWaitEvent(s2, evA, 0);
     LAUNCH_ON(s2, KT_WORKLIST, 1, (k_worklist<<<rt_blocks(nkey, tb, 152 * 16), tb, 0, s2>>>(P, cur, H.lens + 4)));
     if (P.shared)
-        LAUNCH_ON(s2, KT_PHASE_B, 1, (k_phaseB<Real, NRC, true, true><<<rt_blocks(nkey * NRC, tb, GB), tb, 0, s2>>>(P, cur, H.lens + 4)));
+        LAUNCH_ON(s2, KT_PHASE_B, 1, (k_phaseB<Real, NRC, true, true><<<rt_blocks(nkey * 8, tb, GB), tb, 0, s2>>>(P, cur, H.lens + 4)));
     else if (P.any_bar)
-        LAUNCH_ON(s2, KT_PHASE_B, 1, (k_phaseB<Real, NRC, true, false><<<rt_blocks(nkey * NRC, tb, GB), tb, 0, s2>>>(P, cur, H.lens + 4)));
+        LAUNCH_ON(s2, KT_PHASE_B, 1, (k_phaseB<Real, NRC, true, false><<<rt_blocks(nkey * 8, tb, GB), tb, 0, s2>>>(P, cur, H.lens + 4)));
     else
-        LAUNCH_ON(s2, KT_PHASE_B, 1, (k_phaseB<Real, NRC, false, false><<<rt_blocks(nkey * NRC, tb, GB), tb, 0, s2>>>(P, cur, H.lens + 4)));
+        LAUNCH_ON(s2, KT_PHASE_B, 1, (k_phaseB<Real, NRC, false, false><<<rt_blocks(nkey * 8, tb, GB), tb, 0, s2>>>(P, cur, H.lens + 4)));
     cudaEventRecord(evB, s2);
     cudaStreamWaitEvent(st, evB, 0);
     LAUNCH(KT_HOP_COUNT, 1, (k_hop_counts<<<304, 256, 0, st>>>(P, cur ^ 1, fcur ^ 1, H.lens, H.esc_r, H.vstat)));
