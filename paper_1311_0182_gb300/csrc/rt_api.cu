@@ -344,7 +344,7 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     A(P.sdir, double, 3 * (long long)n_src + 3);
     A(P.sgate, int, n_src + 1);
     A(P.bar, Barrier, n_boxes);
-    A(P.fdx, float, n * P.kn); A(P.fdy, float, n * P.kn); A(P.fdz, float, n * P.kn);
+    A(P.fwd4, float4, n * P.kn);
     A(P.rev_off, int, n + 1);
     A(P.rev_ent, unsigned, n * P.kn);
     A(P.rev4, float4, n * P.kn);
@@ -369,7 +369,6 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     }
     P.rec = dalloc(c, 8 * R * nslot, &ok);
     A(P.bm, unsigned, n * P.kn * P.nf);
-    A(P.revpos, int, n * P.kn);
     A(P.worklist, int, nkey);
     A(P.emp, unsigned, nkey);
     A(P.touched, int, nkey);
@@ -1152,7 +1151,7 @@ __global__ void k_masks(DevPtrs P, int cur, unsigned *out) {
     const unsigned *bmr = P.bm + (long long)nu * P.n * P.kn;
     if ((a >> b) & 1u)
         for (int k = 0; k < P.kn; ++k)
-            m |= ((bmr[P.revpos[i * P.kn + k]] >> b) & 1u) << k;
+            m |= ((bmr[__float_as_int(P.fwd4[i * P.kn + k].w)] >> b) & 1u) << k;
     out[t] = m;
 }
 

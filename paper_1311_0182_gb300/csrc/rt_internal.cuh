@@ -181,7 +181,8 @@ struct DevPtrs {              // plain pointers handed to kernels (by value)
     int any_bar;              // some box has a barrier
     int kwide;                // some box holds more than 2^22 particles (24-bit kNN keys)
     int gated;                // some source has a gate
-    float *fdx, *fdy, *fdz;   // forward offsets q_j - q_i, [n * kn]
+    float4 *fwd4;             // [n * kn]: offset q_j - q_i, and the entry's position in the
+                              // reverse lists (its bits)
     int *rev_off;
     unsigned *rev_ent;        // (i << 5) | k
     float4 *rev4;             // the same order: offset q_j - q_i, and the sender i (its bits)
@@ -199,7 +200,6 @@ struct DevPtrs {              // plain pointers handed to kernels (by value)
     // and transposed cone bitmaps
     void *rec;
     unsigned *bm;             // receiver-ordered cone bitmaps [nu * n * kn + p], p = reverse position
-    int *revpos;              // position of forward entry (i, k) in the reverse lists
     unsigned *emp;            // empty-cone bits [n * nf]
     int *touched;             // per (j, nu): 1 when a gas sender wrote a bitmap word this hop
     // requests

@@ -141,9 +141,8 @@ __global__ void __launch_bounds__(256) k_knn(DevPtrs P, int sources) {
                 P.snbr[w * P.kn + lane] = (int)g;
             } else {
                 P.nbr[w * P.kn + lane] = (int)g;
-                P.fdx[w * P.kn + lane] = (float)(P.qx[g] - qx);
-                P.fdy[w * P.kn + lane] = (float)(P.qy[g] - qy);
-                P.fdz[w * P.kn + lane] = (float)(P.qz[g] - qz);
+                P.fwd4[w * P.kn + lane] = make_float4((float)(P.qx[g] - qx), (float)(P.qy[g] - qy),
+                                                      (float)(P.qz[g] - qz), 0.0f);
             }
         }
         if (lane == 0) {
@@ -185,8 +184,9 @@ __global__ void k_rev_sort(DevPtrs P) {
     for (int p = a; p < b; ++p) {
         unsigned v = P.rev_ent[p];
         long long f = (long long)(v >> 5) * P.kn + (v & 31);
-        P.revpos[f] = p;
-        P.rev4[p] = make_float4(P.fdx[f], P.fdy[f], P.fdz[f], __int_as_float((int)(v >> 5)));
+        float4 d = P.fwd4[f];
+        P.fwd4[f].w = __int_as_float(p);
+        P.rev4[p] = make_float4(d.x, d.y, d.z, __int_as_float((int)(v >> 5)));
     }
 }
 

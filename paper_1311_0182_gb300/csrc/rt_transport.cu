@@ -516,128 +516,191 @@ __global__ void k_emit_rec_cones(DevPtrs P, long long base) {
 // ------------------------------------------------------------------------------------------
 // hop kernels
 // ------------------------------------------------------------------------------------------
-// Sender side.  Warp per particle.  The particle's packets able to move are taken 32 at a
+// inclusive prefix sum over the lanes (of packed fields that do not overflow)
+__device__ __forceinline__ unsigned lane_scan(unsigned v) {
+    int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        unsigned t = __shfl_up_sync(FULLMASK, v, o);
+        if (lane >= o) v += t;
+    }
+    return v;
+}
+
+// The packet of a slot as the sender side reads it: photon count, direction, mean clock and
+// energy, and in a shared frequency bin the mean cross-section.
+template <typename Real> struct SentPacket {
+    Real N, d0, d1, d2, C, E, sg;
+};
+
+// Sender side.  A warp takes a few consecutive particles at a time (`per`, at most 32 / n_freq),
+// lane = (particle, frequency) word of packets able to move; their packets are taken 32 at a
 // time (lane = packet: load, direction, clock), then tested one after the other against the
-// neighbours (lane = neighbour k: cone membership, ballot).  For each (frequency, neighbour)
-// the bits of the packets whose cone holds the neighbour go to the neighbour's receiver-ordered
-// bitmap word; empty cones become virtual-particle requests.
+// neighbours of their particle (lane = neighbour k: cone membership, ballot).  For each
+// (frequency, neighbour) the bits of the packets whose cone holds the neighbour go to the
+// neighbour's receiver-ordered bitmap word; empty cones become virtual-particle requests.
+// What bounds it: the latency of the dependent gathers and instruction issue; a particle holds
+// few packets able to move (2.5 with 8 cones behind a fast front, 3.8 over 9 frequencies in the
+// HII region), so with a particle of its own most lanes of a warp idled in the packet part
+// (FP64 there: 16 cycles of an SM an instruction).  The next particle's neighbours are loaded
+// while the current one's packets are tested; what a test needs of a neighbour alone (inverse
+// distance) is computed once a particle.  Measured per step against a warp a particle: 2.1 M
+// particles behind a fast front, 8 cones, 139 -> 78 ms; 64^3 HII region, 32 cones, 13.1 -> 10.7 ms;
+// the FP64 path at 32^3 8.3 -> 5.8 ms; a 64^3 box with hardly any packets 1.77 -> 0.92 ms.
 // cur: the slot buffer holding the hop's packets.  Receivers of a bitmap word are flagged in
 // `touched` (cleared again by the work-list kernel).
 // SH: the shared frequency bin (a separate instance keeps its code out of the common case)
 template <typename Real, int NRC, bool SH>
-__global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int cur) {
-    int lane = threadIdx.x & 31;
-    Slots<Real> S(P, cur);
-    float cf = 1.0f - 2.0f / (float)P.ntc;
-    long long nrev = P.n * P.kn;
-    long long ncon = 0;
-    // each block takes one contiguous chunk of particles; its warps pull particles from it
-    // through a shared counter, so that they finish together (particles hold from none to
-    // hundreds of packets)
+__global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int cur, int per) {
+    __shared__ unsigned slist[8][32];
+    __shared__ unsigned semp[8][32];
     __shared__ int snext;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    unsigned *list = slist[wid];
+    const float cf = 1.0f - 2.0f / (float)P.ntc;
+    const long long nrev = P.n * P.kn;
+    long long ncon = 0;
+    // each block takes one contiguous chunk of particles; its warps pull from it through a
+    // shared counter, so that they finish together (particles hold from none to hundreds of
+    // packets)
     long long chunk = (P.n + gridDim.x - 1) / gridDim.x;
-    long long ib0 = (long long)blockIdx.x * chunk;
-    long long ib1 = ib0 + chunk < P.n ? ib0 + chunk : P.n;
+    const long long ib0 = (long long)blockIdx.x * chunk;
+    const long long ib1 = ib0 + chunk < P.n ? ib0 + chunk : P.n;
     if (threadIdx.x == 0) snext = 0;
     __syncthreads();
-    auto next_particle = [&]() {
+    auto next = [&]() {
         long long v = 0;
-        if (lane == 0) v = ib0 + atomicAdd(&snext, 1);
+        if (lane == 0) v = ib0 + atomicAdd(&snext, per);
         return __shfl_sync(FULLMASK, v, 0);
     };
-    for (long long i = next_particle(); i < ib1; i = next_particle()) {
-        unsigned aw = (lane < P.nf) ? P.act[cur][i * P.nf + lane] : 0u;
+    const int lp = lane / P.nf, lnu = lane - lp * P.nf;      // the lane's particle and frequency
+    auto words = [&](long long i0) {
+        return (i0 + lp < ib1 && lp < per) ? P.act[cur][(i0 + lp) * P.nf + lnu] : 0u;
+    };
+    long long i0 = next();
+    unsigned awn = words(i0);                                 // loaded one turn ahead
+    while (i0 < ib1) {
+        const unsigned aw = awn;
+        const long long ic = i0;
+        i0 = next();
+        awn = words(i0);
+        const int np = (int)(ib1 - ic < per ? ib1 - ic : per);
         if (__ballot_sync(FULLMASK, aw != 0u) == 0u) {
-            if (lane == 0) P.reqcnt[i] = 0;
+            if (lane < np) P.reqcnt[ic + lane] = 0;
             continue;
         }
-        // neighbour k = lane
-        int nb = 0, dx = 0, dy = 0, dz = 0, rp = 0;
-        float fx = 0.f, fy = 0.f, fz = 0.f;
-        bool valid = lane < P.kn;
-        if (valid) {
-            long long f = i * P.kn + lane;
-            nb = P.nbr[f];
-            rp = P.revpos[f];
-            fx = P.fdx[f]; fy = P.fdy[f]; fz = P.fdz[f];
-            dx = (int)fx; dy = (int)fy; dz = (int)fz;
-        }
-        // active packets in (nu, b) order: prefix of the per-frequency counts
-        int cnt = __popc(aw);
-        int incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int v = __shfl_up_sync(FULLMASK, incl, o);
-            if (lane >= o) incl += v;
-        }
-        int total = __shfl_sync(FULLMASK, incl, 31);
-        int excl = incl - cnt;
-        int nreq = 0;
-        unsigned emp_acc = 0u;        // lane nu: empty-cone bits of frequency nu
-        unsigned word = 0u;           // lane k: the current bitmap word and its frequency
-        int cur_nu = -1;
+        semp[wid][lane] = 0u;
+        const unsigned cnt = (unsigned)__popc(aw);
+        const unsigned incl = lane_scan(cnt);
+        const int total = (int)__shfl_sync(FULLMASK, incl, 31);
+        // the current particle's neighbour of this lane, and the next one's
+        float4 ed = make_float4(0.f, 0.f, 0.f, 0.f), edn = ed;
+        int nb = 0, nbn = 0;
+        float ir = 0.f;
+        bool valid = false;
+        int curp = -1;                    // the current particle (of the turn's)
+        unsigned word = 0u;               // the bitmap word under construction
+        int wnu = -1;                     // and its frequency
+        auto fetch = [&](int p) {
+            if (lane < P.kn) {
+                long long f = (ic + p) * P.kn + lane;
+                edn = __ldg(P.fwd4 + f);
+                nbn = __ldg(P.nbr + f);
+            }
+        };
+        auto flush = [&]() {
+            if (word) {
+                P.bm[(long long)wnu * nrev + __float_as_int(ed.w)] = word;
+                P.touched[(long long)nb * P.nf + wnu] = 1;
+            }
+            word = 0u;
+        };
         for (int cb = 0; cb < total; cb += 32) {
-            // lane t takes packet cb + t: its frequency (owner lane) and bin
-            int t = cb + lane;
-            int onu = 0;
-            for (int q = 1; q < P.nf; ++q) {
-                int eq = __shfl_sync(FULLMASK, excl, q);
-                if (eq <= t) onu = q;
-            }
-            unsigned ow = __shfl_sync(FULLMASK, aw, onu);
-            int oex = __shfl_sync(FULLMASK, excl, onu);
-            bool has = t < total;
-            int ob = has ? __fns(ow, 0, t - oex + 1) : 0;
-            long long s = i * P.S + (long long)onu * NRC + ob;
-            Real N = Real(0), d0 = Real(1), d1 = Real(0), d2 = Real(0), C = Real(0), E = Real(0);
-            Real sgr = Real(0);
-            bool sgs = SH && onu == 0;   // a slot of the shared bin: its mean cross-section
+            int p = (int)(incl - cnt) - cb;
+            for (unsigned x = aw; x; x &= x - 1u, ++p)
+                if (p >= 0 && p < 32) list[p] = (unsigned)(__ffs(x) - 1) | (unsigned)lane << 5;
+            __syncwarp();
+            const int nk = min(32, total - cb);
+            const bool has = lane < nk;
+            const unsigned code = list[has ? lane : 0];
+            const int row = (int)(code >> 5), ob = (int)(code & 31u);
+            const int op = __shfl_sync(FULLMASK, lp, row), onu = __shfl_sync(FULLMASK, lnu, row);
+            __syncwarp();
+            // the runs of packets of one particle
+            const int prevp = __shfl_up_sync(FULLMASK, op, 1);
+            unsigned first = __ballot_sync(FULLMASK, has && (lane == 0 ? op != curp : op != prevp));
+            if (first) fetch(__shfl_sync(FULLMASK, op, __ffs(first) - 1));
+            const long long s = (ic + op) * P.S + (long long)onu * NRC + ob;
+            SentPacket<Real> K = {Real(0), Real(1), Real(0), Real(0), Real(0), Real(0), Real(0)};
+            const bool sgs = SH && onu == 0;   // a slot of the shared bin: its mean cross-section
             if (has) {
-                N = S.N[s];
-                packet_dir(S.X[s], S.Y[s], S.Z[s], d0, d1, d2);
-                C = S.C[s];
-                E = S.E[s];
-                if (sgs) sgr = ((Real *)P.slG[cur])[i * NRC + ob] / N;
+                Slots<Real> S(P, cur);
+                K.N = S.N[s];
+                packet_dir(S.X[s], S.Y[s], S.Z[s], K.d0, K.d1, K.d2);
+                K.C = S.C[s];
+                K.E = S.E[s];
+                if (sgs) K.sg = ((Real *)P.slG[cur])[(ic + op) * NRC + ob] / K.N;
             }
-            int nb_chunk = min(32, total - cb);
+            const float f0 = (float)K.d0, f1 = (float)K.d1, f2 = (float)K.d2;
             int my_cm = 0;
-            // the chunk's packets one after the other (lane = neighbour k): cone membership; the
-            // bitmap word of lane k collects, frequency by frequency, the bins whose cone holds
-            // k (a word continues across chunks while the frequency does); a cone with no member
-            // adds its bin to the empty-cone word of its frequency, held on lane nu
-            for (int u = 0; u < nb_chunk; ++u) {
-                Real e0 = __shfl_sync(FULLMASK, d0, u), e1 = __shfl_sync(FULLMASK, d1, u),
-                     e2 = __shfl_sync(FULLMASK, d2, u);
-                int unu = __shfl_sync(FULLMASK, onu, u);
-                int ub = __shfl_sync(FULLMASK, ob, u);
-                bool in = valid && cone_test<Real>(dx, dy, dz, fx, fy, fz, e0, e1, e2, cf, P.ntc);
-                unsigned m = __ballot_sync(FULLMASK, in);
-                if (lane == u) my_cm = __popc(m);
-                if (unu != cur_nu) {
-                    if (valid && word) {
-                        P.bm[(long long)cur_nu * nrev + rp] = word;
-                        P.touched[(long long)nb * P.nf + cur_nu] = 1;
-                    }
-                    word = 0u;
-                    cur_nu = unu;
+            // the packets one after the other (lane = neighbour k): cone membership; the bitmap
+            // word of lane k collects, frequency by frequency, the bins whose cone holds k (a
+            // word continues across turns of 32 packets while its particle and frequency do)
+            for (int t = 0; t < nk; ++t) {
+                if ((first >> t) & 1u) {
+                    flush();
+                    ed = edn;
+                    nb = nbn;
+                    curp = __shfl_sync(FULLMASK, op, t);
+                    wnu = -1;
+                    valid = lane < P.kn && (ed.x != 0.f || ed.y != 0.f || ed.z != 0.f);
+                    ir = rsqrtf(__fmaf_rn(ed.x, ed.x, __fmaf_rn(ed.y, ed.y, ed.z * ed.z)));
+                    unsigned later = first & (0xfffffffeu << t);
+                    if (later) fetch(__shfl_sync(FULLMASK, op, __ffs(later) - 1));
+                }
+                const float e0 = __shfl_sync(FULLMASK, f0, t), e1 = __shfl_sync(FULLMASK, f1, t),
+                            e2 = __shfl_sync(FULLMASK, f2, t);
+                const int unu = __shfl_sync(FULLMASK, onu, t), ub = __shfl_sync(FULLMASK, ob, t);
+                const float cs = __fmaf_rn(ed.x, e0, __fmaf_rn(ed.y, e1, ed.z * e2)) * ir;
+                bool in = valid && cs > cf + CONE_BAND;
+                const bool amb = valid && !in && !(cs < cf - CONE_BAND);
+                if (__any_sync(FULLMASK, amb)) {   // inside the guard band: the exact test
+                    const Real x0 = __shfl_sync(FULLMASK, K.d0, t), x1 = __shfl_sync(FULLMASK, K.d1, t),
+                               x2 = __shfl_sync(FULLMASK, K.d2, t);
+                    if (amb)
+                        in = cone_exact((int)ed.x, (int)ed.y, (int)ed.z, (double)x0, (double)x1,
+                                        (double)x2, P.ntc);
+                }
+                const unsigned m = __ballot_sync(FULLMASK, in);
+                if (lane == t) my_cm = __popc(m);
+                if (unu != wnu) {
+                    flush();
+                    wnu = unu;
                 }
                 if (in) word |= 1u << ub;
-                if (m == 0u && lane == unu) emp_acc |= 1u << ub;
             }
-            ncon += (lane < nb_chunk) ? my_cm : 0;
-            if (has && my_cm > 0)
-                rec_store(P.rec, s, rdiv<Real>(N, (Real)my_cm), d0, d1, d2, rdiv<Real>(C, N),
-                          rdiv<Real>(E, N), sgs, sgr);
-            nreq += __popc(__ballot_sync(FULLMASK, has && my_cm == 0));
+            ncon += my_cm;
+            if (has) {
+                if (my_cm > 0)
+                    rec_store(P.rec, s, rdiv<Real>(K.N, (Real)my_cm), K.d0, K.d1, K.d2,
+                              rdiv<Real>(K.C, K.N), rdiv<Real>(K.E, K.N), sgs, K.sg);
+                else
+                    atomicOr(&semp[wid][row], 1u << ob);
+            }
         }
         // every word starts the hop at zero (the receiver side clears the words it reads), and
         // each (frequency, neighbour) word is written once: a plain store
-        if (valid && word) {
-            P.bm[(long long)cur_nu * nrev + rp] = word;
-            P.touched[(long long)nb * P.nf + cur_nu] = 1;
-        }
-        if (lane < P.nf) P.emp[i * P.nf + lane] = emp_acc;
-        if (lane == 0) P.reqcnt[i] = nreq;
+        flush();
+        __syncwarp();
+        const unsigned em = semp[wid][lane];
+        if (lp < np) P.emp[(ic + lp) * P.nf + lnu] = em;
+        // requests a particle: the sum over its words
+        unsigned r = (unsigned)__popc(em);
+        const unsigned ri = lane_scan(r);
+        const int la = lane * P.nf - 1, lb = min(la + P.nf, 31);   // last lanes of particles lane - 1, lane
+        const unsigned ra = __shfl_sync(FULLMASK, ri, la & 31), rb = __shfl_sync(FULLMASK, ri, lb & 31);
+        if (lane < np) P.reqcnt[ic + lane] = (int)(rb - (lane ? ra : 0u));
+        __syncwarp();
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ncon += __shfl_down_sync(FULLMASK, ncon, o);
@@ -1240,17 +1303,6 @@ __device__ __forceinline__ unsigned byte_popc(unsigned x) {
     x = (x & 0x33333333u) + ((x >> 2) & 0x33333333u);
     return (x + (x >> 4)) & 0x0f0f0f0fu;
 }
-// inclusive prefix sum over the lanes (of packed fields that do not overflow)
-__device__ __forceinline__ unsigned lane_scan(unsigned v) {
-    int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        unsigned t = __shfl_up_sync(FULLMASK, v, o);
-        if (lane >= o) v += t;
-    }
-    return v;
-}
-
 // One receiver group of 32 cones by a whole warp, lane = reception cone, whatever its number of
 // edges, contributions and waiting packets: edges 32 at a time, contributions 32 at a time,
 // each cone's lane adding its contributions in list order.
@@ -1860,6 +1912,14 @@ static void launch_virtual(rt_ctx *c, cudaStream_t st, int GV, int cur, int fcur
                                                                     H.vstat);
 }
 
+// Particles a warp of the sender side takes together: as many as its 32 (particle, frequency)
+// words hold, but no more than leave every resident warp (152 SMs x 32) a turn, since a small
+// box needs its particles spread over the chip more than it needs full lanes.
+static int send_turn(const DevPtrs &P) {
+    long long most = std::max(1, 32 / P.nf);
+    return (int)std::min(most, std::max(1ll, P.n / (152 * 32)));
+}
+
 // One hop.  Two streams: st: gas senders, the request list, virtual particles, the hop counts.
 // s2: free-packet senders and staging, receiver segments, work list, receiver side.  s2 starts
 // after everything before this hop on st; the work list waits for the gas senders (touched
@@ -1876,6 +1936,7 @@ static void hop_core(rt_ctx *c, cudaStream_t st, long long nfr, int cur, int fcu
     HopScratch &H = c->hop;
     const int tb = 256, gb = 152 * 64;
     long long n = P.n, nkey = n * P.nf;
+    const int per = send_turn(P);
     cudaStream_t s2 = c->st2;
     cudaEvent_t evFork = c->hev[0], evA = c->hev[1], evFree = c->hev[2], evB = c->hev[3];
     if (nfr < 1) nfr = 1;
@@ -1895,9 +1956,9 @@ static void hop_core(rt_ctx *c, cudaStream_t st, long long nfr, int cur, int fcu
     else
         LAUNCH_ON(s2, KT_FREE_C, 1, (k_freeC<Real, NRC, false, false><<<rt_blocks(nfr * 32, tb, gb), tb, 0, s2>>>(P, fcur, H.lens, H.fmask, H.stoff)));
     if (P.shared)
-        LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, true><<<rt_blocks(n * 32, tb, GA), tb, 0, st>>>(P, cur)));
+        LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, true><<<rt_blocks((n + per - 1) / per * 32, tb, GA), tb, 0, st>>>(P, cur, per)));
     else
-        LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, false><<<rt_blocks(n * 32, tb, GA), tb, 0, st>>>(P, cur)));
+        LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, false><<<rt_blocks((n + per - 1) / per * 32, tb, GA), tb, 0, st>>>(P, cur, per)));
     cudaEventRecord(evA, st);
     cudaStreamWaitEvent(st, evFree, 0);
     LAUNCH(KT_SCAN, 2, (rt_scan_exclusive(c, P.reqcnt, P.reqoff, n + nfr, H.lens + 1, H.lens + 2, st)));
@@ -2030,10 +2091,11 @@ static rt_status run_parts(rt_ctx *c, int part, long long step, cudaStream_t st)
     if (part == 3) {  // cone masks of the held packets only (inspection)
         clear_cone_bits(c, st);
         c->bm_dirty = true;
+        const int per = send_turn(P);
         if (P.shared)
-            LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, true><<<rt_blocks(n * 32, tb, 152 * 64), tb, 0, st>>>(P, c->cur)));
+            LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, true><<<rt_blocks((n + per - 1) / per * 32, tb, 152 * 64), tb, 0, st>>>(P, c->cur, per)));
         else
-            LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, false><<<rt_blocks(n * 32, tb, 152 * 64), tb, 0, st>>>(P, c->cur)));
+            LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, false><<<rt_blocks((n + per - 1) / per * 32, tb, 152 * 64), tb, 0, st>>>(P, c->cur, per)));
         return rt_cuda_check(c, cudaGetLastError(), "cone masks");
     }
     // part 4: the hop loop, driven from the host (one synchronisation per hop)
