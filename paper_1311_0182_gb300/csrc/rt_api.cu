@@ -321,6 +321,7 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     A(x->src_emit, double, n_boxes);
     A(P.pbox, int, n);
     A(P.qx, int, n); A(P.qy, int, n); A(P.qz, int, n);
+    A(P.q4, int4, n);
     A(P.nH, double, n); A(P.NH, double, n); A(P.xHI, double, n); A(P.T, double, n);
     A(P.Nrec, double, n); A(P.epsrec, double, n); A(P.nHI, double, n); A(P.phot, double, n);
     P.nHIr = dalloc(c, R * n, &ok);
@@ -364,16 +365,16 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     for (int b = 0; b < 2; ++b) {
         for (int f = 0; f < 6; ++f) P.sl[b][f] = dalloc(c, R * nslot, &ok);
         if (P.shared) P.slG[b] = dalloc(c, R * n * P.nrc, &ok);
-        A(P.occ[b], unsigned, nkey);
-        A(P.act[b], unsigned, nkey);
+        A(P.occ[b], unsigned, nkey + 4);   // the work list reads whole fours of the key arrays
+        A(P.act[b], unsigned, nkey + 4);
     }
     P.rec = dalloc(c, 8 * R * nslot, &ok);
     A(P.bm, unsigned, n * P.kn * P.nf);
     A(P.worklist, int, nkey);
     A(P.emp, unsigned, nkey);
-    A(P.touched, int, nkey);
+    A(P.touched, unsigned char, nkey + 4);
     A(P.reqcnt, int, n + fc);
-    A(P.reqoff, int, n + fc);
+    A(P.reqsum, int, n / RT_REQ_CHUNK + fc / RT_REQ_CHUNK + 2);
     A(P.req, unsigned long long, fc);
     for (int b = 0; b < 2; ++b) {
         FreeBuf &F = P.fr[b];
@@ -389,12 +390,15 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     }
     A(P.st_key, int, P.ST_cap);
     A(P.st_bin, int, P.ST_cap);
+    A(P.st_ord, int, P.ST_cap);
+    A(P.st_rank, int, P.ST_cap);
     for (int f = 0; f < 9; ++f) P.st_v[f] = dalloc(c, R * P.ST_cap, &ok);
     if (P.shared) P.st_v[9] = dalloc(c, R * P.ST_cap, &ok);
-    long long segn = std::max<long long>(nkey, ncell) + 1;
+    long long segn = std::max<long long>(nkey, ncell) + 4;
     A(P.seg_cnt, int, segn);
     A(P.seg_off, int, segn);
     A(P.seg_fill, int, segn);
+    A(P.seg_ent, int2, P.ST_cap);
     A(P.seg_idx, int, P.ST_cap);
     A(P.abs, double, nkey); A(P.absE, double, nkey); A(P.pass, double, nkey);
     A(P.passf, float, nkey);
@@ -403,16 +407,10 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     A(P.fx_lo, unsigned long long, nkey);
     A(P.cnt, long long, CNT_N);
     A(x->hop.lens, int, 8);
-    A(x->hop.fmask, unsigned, fc);
-    A(x->hop.stcnt, int, fc);
-    A(x->hop.stoff, int, fc);
-    A(x->hop.esc_r, unsigned long long, fc);
-    A(x->hop.vstat, unsigned char, fc);
 #undef A
     // the scan scratch: one partial sum per block of a scan (no allocation later)
     c->scan_tmp_n = RT_SCAN_NB;
     if (cudaMalloc(&c->scan_tmp, sizeof(int) * c->scan_tmp_n) != cudaSuccess) ok = false;
-    if (cudaMalloc(&c->scan_tmp2, sizeof(int) * c->scan_tmp_n) != cudaSuccess) ok = false;
     if (cudaMallocHost(&c->cnt_h, sizeof(long long) * CNT_N) != cudaSuccess) ok = false;
     // the hop loop's second stream, at the highest priority: its receiver-side kernels take
     // SM slots ahead of the virtual-particle kernel that runs beside them
@@ -480,7 +478,6 @@ extern "C" rt_status rt_destroy(rt_ctx *c) {
     for (size_t k = 0; k < c->allocs.size(); ++k) cudaFree(c->allocs[k]);
     if (c->d.grid.cand) cudaFree(c->d.grid.cand);
     if (c->scan_tmp) cudaFree(c->scan_tmp);
-    if (c->scan_tmp2) cudaFree(c->scan_tmp2);
     if (c->cnt_h) cudaFreeHost(c->cnt_h);
     if (c->st2) {
         cudaStreamSynchronize(c->st2);

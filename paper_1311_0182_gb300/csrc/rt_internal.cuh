@@ -22,6 +22,7 @@
 #define RT_OCC_MIN 1           // finest kNN grid the occupancy search tries
 #define RT_MAXK 32            // maximum neighbours per particle
 #define RT_FREE_BIT (1ull << 63)
+#define RT_REQ_CHUNK 1024      // particles (or free packets) of one partial sum of the requests
 #define RT_SCAN_NB 608         // blocks of every prefix-sum launch (4 per SM)
 
 // error bits of the sticky device error word
@@ -47,9 +48,9 @@ enum {
     CNT_WLS = 15,       // receiver work-list entries, summed over hops
     CNT_OUT = 16,       // occupied slots written by the receiver side, summed over hops
     // hop state: kept on the device so that a captured graph replays the hop loop unchanged
-    // (19: unused)
     CNT_CUR = 17,       // slot buffer holding the current packets (0 or 1)
     CNT_FCUR = 18,      // free-packet buffer of the current hop (0 or 1)
+    CNT_MORE = 19,      // 1: another hop follows
     CNT_HOP = 20,       // hops done in this step
     CNT_STEP = 21,      // step number (random streams of the rotations and virtual particles)
     CNT_DROP = 22,      // 1: the hop cap stopped the loop with packets still moving
@@ -93,12 +94,8 @@ struct Grid {                 // per-box uniform cell lists (device arrays)
     long long cand_cap;       // entries allocated
 };
 
-struct HopScratch {           // per-hop scratch: [0] free packets, [1] n + free, [2] requests, [3] staged
-    int *lens;
-    unsigned *fmask;
-    int *stcnt, *stoff;
-    unsigned long long *esc_r;
-    unsigned char *vstat;
+struct HopScratch {           // counts of the hop: [0] free packets, [2] requests, [3] staged
+    int *lens;                // contributions, [4] receiver groups, [5] segment entries given out
 };
 
 // Artificial photon barrier of a box (Sec. 4): a disk perpendicular to coordinate `axis`, in
@@ -161,6 +158,7 @@ struct DevPtrs {              // plain pointers handed to kernels (by value)
     double *bpart;            // [nbch * 2]
     // particles
     int *pbox, *qx, *qy, *qz;
+    int4 *q4;                 // (qx, qy, qz, box)
     double *nH, *NH, *xHI, *T, *Nrec, *epsrec, *nHI, *phot;
     void *nHIr, *Vr, *depE_s;  // Real [n]
     void *dep_s;               // Real [n]: fixed-point scale of photon deposits
@@ -201,18 +199,23 @@ struct DevPtrs {              // plain pointers handed to kernels (by value)
     void *rec;
     unsigned *bm;             // receiver-ordered cone bitmaps [nu * n * kn + p], p = reverse position
     unsigned *emp;            // empty-cone bits [n * nf]
-    int *touched;             // per (j, nu): 1 when a gas sender wrote a bitmap word this hop
+    unsigned char *touched;   // per (j, nu): 1 when a gas sender wrote a bitmap word this hop
     // requests
-    int *reqcnt, *reqoff;     // [n + F_cap]
+    int *reqcnt;              // [n + F_cap] requests of each particle and free packet
+    int *reqsum;              // and of each RT_REQ_CHUNK of them (particles, then free packets)
     unsigned long long *req;  // [F_cap]
     FreeBuf fr[2];
     // staged free-packet contributions
     int *st_key;              // receiver key j*nf+nu
-    long long *st_ord;        // ordering key f*kn + k
+    int *st_ord;              // ordering key: the packet f (one contribution a receiver)
+    int *st_rank;             // place among the receiver's contributions, in arrival order
     int *st_bin;
     void *st_v[10];           // T, T dx, T dy, T dz, T clock, T eps, A, A eps, w, T sigma (Real;
                               // the last with a shared bin only)
-    int *seg_cnt, *seg_off, *seg_fill, *seg_idx;
+    int *seg_cnt, *seg_off;   // per key: contributions (zero between hops) and first entry
+    int2 *seg_ent;            // (packet, contribution), in arrival order
+    int *seg_idx;             // contributions in packet order
+    int *seg_fill;            // scratch of the neighbour build
     // accumulators
     double *abs, *absE, *pass;                // [n * nf]
     unsigned long long *fx_abs, *fx_lo, *fx_E;  // [n * nf]: photons (2 words), energy
@@ -280,7 +283,6 @@ struct rt_ctx {
     // scan scratch
     int *scan_tmp = nullptr;
     long long scan_tmp_n = 0;
-    int *scan_tmp2 = nullptr;     // scratch of the scans on the second stream
     // second stream of the hop loop (work independent of the caller's stream's kernels) and
     // the events that order the two
     cudaStream_t st2 = nullptr;
@@ -298,6 +300,7 @@ struct rt_ctx {
     bool use_graph = true;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t graph_exec = nullptr;
+    cudaGraphConditionalHandle loop_h = 0, pair_h = 0;   // the hop loop, and its buffer switch
     cudaStream_t st_cap = nullptr;     // capture stream
     DevPtrs graph_P;                   // parameters the graph was captured with
     int graph_hop_cap = -1;

@@ -31,6 +31,7 @@ __global__ void k_quantise(DevPtrs P, const double *x, const double *y, const do
     }
     P.pbox[i] = lo;
     P.qx[i] = q[0]; P.qy[i] = q[1]; P.qz[i] = q[2];
+    P.q4[i] = make_int4(q[0], q[1], q[2], lo);
     double V = P.NH[i] / P.nH[i] / P.vunit[lo];   // volume in the box's volume unit
     if (P.fp32) ((float *)P.Vr)[i] = (float)V;
     else ((double *)P.Vr)[i] = V;
@@ -523,6 +524,8 @@ rt_status rt_knn_build(rt_ctx *c, cudaStream_t st) {
     // the virtual particles' candidate lists, on the grid the occupancy search picks (it needs
     // the smoothing lengths just computed)
     s = c->grid_tuned ? cand_lists(c, st) : tune_grid(c, st);
+    // the hop loop finds the counts of staged contributions at zero
+    cudaMemsetAsync(P.seg_cnt, 0, sizeof(int) * (n * P.nf + 4), st);
     // the step graph holds the grid description by value
     rt_graph_destroy(c);
     return s;
