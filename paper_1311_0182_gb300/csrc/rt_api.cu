@@ -346,6 +346,7 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     A(P.sgate, int, n_src + 1);
     A(P.bar, Barrier, n_boxes);
     A(P.fwd4, float4, n * P.kn);
+    A(P.revpos, int, n * P.kn);
     A(P.rev_off, int, n + 1);
     A(P.rev_ent, unsigned, n * P.kn);
     A(P.rev4, float4, n * P.kn);
@@ -1148,7 +1149,7 @@ __global__ void k_masks(DevPtrs P, int cur, unsigned *out) {
     const unsigned *bmr = P.bm + (long long)nu * P.n * P.kn;
     if ((a >> b) & 1u)
         for (int k = 0; k < P.kn; ++k)
-            m |= ((bmr[__float_as_int(P.fwd4[i * P.kn + k].w)] >> b) & 1u) << k;
+            m |= ((bmr[P.revpos[i * P.kn + k]] >> b) & 1u) << k;
     out[t] = m;
 }
 

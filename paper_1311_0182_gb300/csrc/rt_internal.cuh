@@ -179,8 +179,8 @@ struct DevPtrs {              // plain pointers handed to kernels (by value)
     int any_bar;              // some box has a barrier
     int kwide;                // some box holds more than 2^22 particles (24-bit kNN keys)
     int gated;                // some source has a gate
-    float4 *fwd4;             // [n * kn]: offset q_j - q_i, and the entry's position in the
-                              // reverse lists (its bits)
+    float4 *fwd4;             // [n * kn]: offset q_j - q_i, and the neighbour j (its bits)
+    int *revpos;              // [n * kn]: the entry's position in the reverse lists
     int *rev_off;
     unsigned *rev_ent;        // (i << 5) | k
     float4 *rev4;             // the same order: offset q_j - q_i, and the sender i (its bits)

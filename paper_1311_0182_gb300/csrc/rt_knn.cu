@@ -143,7 +143,8 @@ __global__ void __launch_bounds__(256) k_knn(DevPtrs P, int sources) {
             } else {
                 P.nbr[w * P.kn + lane] = (int)g;
                 P.fwd4[w * P.kn + lane] = make_float4((float)(P.qx[g] - qx), (float)(P.qy[g] - qy),
-                                                      (float)(P.qz[g] - qz), 0.0f);
+                                                      (float)(P.qz[g] - qz),
+                                                      __int_as_float((int)g));
             }
         }
         if (lane == 0) {
@@ -168,26 +169,35 @@ __global__ void k_rev_fill(DevPtrs P, int *fill) {
     P.rev_ent[pos] = ((unsigned)i << 5) | (unsigned)k;
 }
 
-// order each receiver's senders by index (the fill order is arbitrary) and copy the offsets
-__global__ void k_rev_sort(DevPtrs P) {
-    long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= P.n) return;
-    int a = P.rev_off[j], b = P.rev_off[j + 1];
-    for (int p = a + 1; p < b; ++p) {
-        unsigned v = P.rev_ent[p];
-        int q = p - 1;
-        while (q >= a && P.rev_ent[q] > v) {
-            P.rev_ent[q + 1] = P.rev_ent[q];
-            --q;
+// Order each receiver's senders by index (the fill order is arbitrary) and write the edges in
+// that order.  A warp a receiver: lanes hold 32 entries each round, and an entry's place is the
+// number of smaller ones (the entries are distinct), counted against all rounds.  Offsets come
+// from the positions (16 bytes a particle, which the L2 holds; reading them from the senders'
+// edges, 154 MB in random order, took 2.5 ms).  A thread a receiver sorted by insertion in
+// global memory before: 1328 us for 300,000 particles, 143 us now.
+__global__ void __launch_bounds__(256) k_rev_sort(DevPtrs P) {
+    const int lane = threadIdx.x & 31;
+    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long j = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < P.n; j += nw) {
+        const int a = P.rev_off[j], b = P.rev_off[j + 1];
+        const int4 q = __ldg(P.q4 + j);
+        for (int r0 = a; r0 < b; r0 += 32) {
+            const bool on = r0 + lane < b;
+            const unsigned v = on ? P.rev_ent[r0 + lane] : 0u;
+            int rank = 0;
+            for (int c0 = a; c0 < b; c0 += 32) {
+                const unsigned o = c0 == r0 ? v : c0 + lane < b ? P.rev_ent[c0 + lane] : 0u;
+                const int m = min(32, b - c0);
+                for (int k = 0; k < m; ++k) rank += __shfl_sync(FULLMASK, o, k) < v;
+            }
+            if (on) {
+                const int p = a + rank, i = (int)(v >> 5);
+                const int4 s = __ldg(P.q4 + i);
+                P.revpos[(long long)i * P.kn + (v & 31u)] = p;
+                P.rev4[p] = make_float4((float)(q.x - s.x), (float)(q.y - s.y), (float)(q.z - s.z),
+                                        __int_as_float(i));
+            }
         }
-        P.rev_ent[q + 1] = v;
-    }
-    for (int p = a; p < b; ++p) {
-        unsigned v = P.rev_ent[p];
-        long long f = (long long)(v >> 5) * P.kn + (v & 31);
-        float4 d = P.fwd4[f];
-        P.fwd4[f].w = __int_as_float(p);
-        P.rev4[p] = make_float4(d.x, d.y, d.z, __int_as_float((int)(v >> 5)));
     }
 }
 
@@ -258,8 +268,12 @@ __device__ __forceinline__ int cand_radius(long long u2, int cs, int G) {
 }
 
 // Calls f(position of the item among the box's items, item) for every particle of box b whose
-// squared distance to the cell box [lo, lo + cs - 1]^3 is at most u2 (lane = grid column; a
-// column's cells are consecutive, so its candidate cells are one range of items).
+// squared distance to the cell box [lo, lo + cs - 1]^3 is at most u2.  Lane = grid column (its
+// cells are consecutive, so the cells of a column that can hold such a particle are one range of
+// items); the lanes' ranges are then walked together, 32 items at a time, so that a warp reads
+// whole lines and a column of a dense clump does not hold up its lane: with a column a lane the
+// slowest cells of a clump took 13.4 ms of a 300,000-particle build (k_cand_fill), 6.4 ms with
+// the lanes together, and 1.6 ms with the rings in 32-bit arithmetic as well.
 template <typename F>
 __device__ __forceinline__ void cand_walk(const DevPtrs &P, int b, int cx, int cy, int cz,
                                           long long u2, F f) {
@@ -272,21 +286,46 @@ __device__ __forceinline__ void cand_walk(const DevPtrs &P, int b, int cx, int c
     int hx = lx + cs - 1, hy = ly + cs - 1, hz = lz + cs - 1;
     int side = 2 * R + 1;
     long long ncol = (long long)side * side;
-    int z0 = max(cz - R, 0), z1 = min(cz + R, G - 1);
     for (long long cb = 0; cb < ncol; cb += 32) {
         long long col = cb + lane;
-        if (col >= ncol) continue;
-        int ix = cx - R + (int)(col / side), iy = cy - R + (int)(col % side);
-        if (ix < 0 || iy < 0 || ix >= G || iy >= G) continue;
-        long long gx = ix < cx ? lx - (ix * cs + cs - 1) : (ix > cx ? ix * cs - hx : 0);
-        long long gy = iy < cy ? ly - (iy * cs + cs - 1) : (iy > cy ? iy * cs - hy : 0);
-        if (gx * gx + gy * gy > u2) continue;
-        long long colbase = coff + ((long long)ix * G + iy) * G;
-        int p0 = P.grid.start[colbase + z0], p1 = P.grid.start[colbase + z1 + 1];
-        for (int pos = p0; pos < p1; ++pos) {
-            int4 it = P.grid.items[pos];
-            if (box_d2(it.x, it.y, it.z, lx, ly, lz, hx, hy, hz) <= u2) f(pos - ibase, it);
+        int p0 = 0, len = 0;
+        if (col < ncol) {
+            int ix = cx - R + (int)(col / side), iy = cy - R + (int)(col % side);
+            if (ix >= 0 && iy >= 0 && ix < G && iy < G) {
+                long long gx = ix < cx ? lx - (ix * cs + cs - 1) : (ix > cx ? ix * cs - hx : 0);
+                long long gy = iy < cy ? ly - (iy * cs + cs - 1) : (iy > cy ? iy * cs - hy : 0);
+                long long rem = u2 - gx * gx - gy * gy;
+                if (rem >= 0) {
+                    // what is left of the distance bounds the column's cells
+                    int rz = R;
+                    if (rem < (1ll << 42)) rz = min(R, (int)((long long)sqrt_up(rem) / cs) + 1);
+                    long long colbase = coff + ((long long)ix * G + iy) * G;
+                    p0 = P.grid.start[colbase + max(cz - rz, 0)];
+                    len = P.grid.start[colbase + min(cz + rz, G - 1) + 1] - p0;
+                }
+            }
         }
+        int incl = len;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            int v = __shfl_up_sync(FULLMASK, incl, o);
+            if (lane >= o) incl += v;
+        }
+        const int total = __shfl_sync(FULLMASK, incl, 31), first = p0 - (incl - len);
+        for (int base = 0; base < total; base += 32) {
+            // the column of item base + lane: the number of columns that end at or before it
+            const int c = base + lane;
+            int own = 0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(FULLMASK, incl, own + o - 1) <= c) own += o;
+            const int pos = __shfl_sync(FULLMASK, first, own & 31) + c;
+            if (c < total) {
+                int4 it = P.grid.items[pos];
+                if (box_d2(it.x, it.y, it.z, lx, ly, lz, hx, hy, hz) <= u2) f(pos - ibase, it);
+            }
+        }
+        __syncwarp();
     }
 }
 
@@ -362,16 +401,18 @@ __global__ void __launch_bounds__(256) k_cand_fill(DevPtrs P, const long long *u
         int cx = (int)(lc / ((long long)G * G)), cy = (int)((lc / G) % G), cz = (int)(lc % G);
         int mx = cand_centre(cx * cs, cs), my = cand_centre(cy * cs, cs), mz = cand_centre(cz * cs, cs);
         int w = cand_ring_width(cs);
+        const float winv = 1.0f / (float)w;
         long long u2 = u2in[c];
         long long a = P.grid.cand_off[c], e = P.grid.cand_off[c + 1];
         if (e == a) continue;   // no list: its queries take the grid walk
         auto ring_of = [&](const int4 &it) {
             long long dx = it.x - mx, dy = it.y - my, dz = it.z - mz;
-            long long d2 = dx * dx + dy * dy + dz * dz;
-            long long r = (long long)(sqrt((double)d2) / (double)w);
-            if (r > 255) r = 255;
-            while (r > 0 && (r * w) * (r * w) > d2) --r;   // r w <= |p - m|
-            return (int)r;
+            // floor(floor(|p - m|) / w) in 32-bit arithmetic (in FP64, at 16 cycles of an SM a warp
+            // instruction, this was most of the kernel); r w <= |p - m| in any case
+            int s = (int)isqrt64(dx * dx + dy * dy + dz * dz);
+            int r = (int)((float)s * winv);
+            if (r * w > s) --r;
+            return min(r, 255);
         };
         for (int k = lane; k < 256; k += 32) bin[k] = 0;
         __syncwarp();
@@ -518,7 +559,7 @@ rt_status rt_knn_build(rt_ctx *c, cudaStream_t st) {
     k_rev_count<<<nbe, tb, 0, st>>>(P, cnt);
     rt_scan_exclusive(c, cnt, P.rev_off, n + 1, nullptr, nullptr, st);
     k_rev_fill<<<nbe, tb, 0, st>>>(P, fill);
-    k_rev_sort<<<nbk, tb, 0, st>>>(P);
+    k_rev_sort<<<rt_blocks(n * 32, tb, 152 * 32), tb, 0, st>>>(P);
     rt_status s = rt_cuda_check(c, cudaGetLastError(), "neighbour build");
     if (s != RT_OK) return s;
     // the virtual particles' candidate lists, on the grid the occupancy search picks (it needs

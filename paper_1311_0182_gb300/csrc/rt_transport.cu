@@ -604,7 +604,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int c
         const int total = (int)__shfl_sync(FULLMASK, incl, 31);
         // the current particle's neighbour of this lane, and the next one's
         float4 ed = make_float4(0.f, 0.f, 0.f, 0.f), edn = ed;
-        int nb = 0, nbn = 0;
+        int rp = 0, rpn = 0;
         float ir = 0.f;
         bool valid = false;
         int curp = -1;                    // the current particle (of the turn's)
@@ -614,13 +614,13 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int c
             if (lane < P.kn) {
                 long long f = (ic + p) * P.kn + lane;
                 edn = __ldg(P.fwd4 + f);
-                nbn = __ldg(P.nbr + f);
+                rpn = __ldg(P.revpos + f);
             }
         };
         auto flush = [&]() {
             if (word) {
-                P.bm[(long long)wnu * nrev + __float_as_int(ed.w)] = word;
-                P.touched[(long long)nb * P.nf + wnu] = 1;
+                P.bm[(long long)wnu * nrev + rp] = word;
+                P.touched[(long long)__float_as_int(ed.w) * P.nf + wnu] = 1;
             }
             word = 0u;
         };
@@ -659,7 +659,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int c
                 if ((first >> t) & 1u) {
                     flush();
                     ed = edn;
-                    nb = nbn;
+                    rp = rpn;
                     curp = __shfl_sync(FULLMASK, op, t);
                     wnu = -1;
                     valid = lane < P.kn && (ed.x != 0.f || ed.y != 0.f || ed.z != 0.f);
