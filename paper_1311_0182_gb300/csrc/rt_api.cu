@@ -328,6 +328,7 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     P.Vr = dalloc(c, R * n, &ok);
     P.dep_s = dalloc(c, R * n, &ok);
     P.depE_s = dalloc(c, R * n, &ok);
+    P.vpv = dalloc(c, 4 * R * n, &ok);
     A(P.sbox, int, n_src + 1);
     A(P.gid0, long long, n_boxes);
     A(P.sid, long long, n_src + 1);
@@ -359,6 +360,7 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     P.grid.cand_cap = 0;
     c->grid_cap = ncell;
     A(P.grid.items, int4, n);
+    A(P.grid.fitems, float4, n);
     A(P.grid.tab, int, KNN_TAB_N);
     A(P.R, double, 9 * n);
     A(P.Rf, float, 9 * n);

@@ -85,6 +85,7 @@ struct Grid {                 // per-box uniform cell lists (device arrays)
     long long *coff;          // first cell of the box
     int *start;               // [ncells + 1] offsets into items
     int4 *items;              // (qx, qy, qz, local index) sorted by cell
+    float4 *fitems;           // the same, coordinates as FP32 (exact), the index as its bits
     long long ncells;
     int *tab;                 // cell offsets of the kNN search, nearest first (rt_knn.cuh)
     // per-cell candidate lists of the virtual particles' kNN (rt_knn.cuh): cand_off[ncells + 1]
@@ -162,6 +163,7 @@ struct DevPtrs {              // plain pointers handed to kernels (by value)
     double *nH, *NH, *xHI, *T, *Nrec, *epsrec, *nHI, *phot;
     void *nHIr, *Vr, *depE_s;  // Real [n]
     void *dep_s;               // Real [n]: fixed-point scale of photon deposits
+    void *vpv;                 // Real [n * 4]: volume, n_HI and the two deposit scales, together
     // sources
     int *sbox, *sqx, *sqy, *sqz;
     // identities in the random streams: particle i of box b draws as gid0[b] + (i - box_off[b]),

@@ -75,7 +75,9 @@ __global__ void k_cell_fill(DevPtrs P, int *fill) {
     long long c = cell_of_particle(P, i);
     int pos = P.grid.start[c] + atomicAdd(&fill[c], 1);
     int b = P.pbox[i];
-    P.grid.items[pos] = make_int4(P.qx[i], P.qy[i], P.qz[i], (int)(i - P.box_off[b]));
+    const int q[3] = {P.qx[i], P.qy[i], P.qz[i]}, idx = (int)(i - P.box_off[b]);
+    P.grid.items[pos] = make_int4(q[0], q[1], q[2], idx);
+    P.grid.fitems[pos] = make_float4((float)q[0], (float)q[1], (float)q[2], __int_as_float(idx));
 }
 
 void knn_offset_table(int *out) {
@@ -202,13 +204,10 @@ __global__ void __launch_bounds__(256) k_rev_sort(DevPtrs P) {
 }
 
 // Timing probe of the occupancy search: the kNN search of virtual-particle-like points, one
-// per fourth particle, up to 0.44 smoothing lengths from it in a hashed direction, from the
-// candidate list of its cell (or the grid walk where it has none) like the virtual particles'
-// search.  Writes one word no one reads,
-// so that the search is not dropped.
-template <bool FB>
+// per fourth particle, up to 0.44 smoothing lengths from it in a hashed direction, like the
+// virtual particles' search.  Writes one word no one reads, so that the search is not dropped.
 __global__ void __launch_bounds__(256) k_knn_probe(DevPtrs P, unsigned long long *sink) {
-    __shared__ int sdelta[FB ? 8 : 1][32];
+    __shared__ unsigned scratch[8][32];
     int lane = threadIdx.x & 31;
     long long w0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -228,20 +227,11 @@ __global__ void __launch_bounds__(256) k_knn_probe(DevPtrs P, unsigned long long
         int qz = min(max(P.qz[i] + o[2], 0), RT_Q - 1);
         long long d2;
         int idx;
-        int *sd = sdelta[FB ? threadIdx.x >> 5 : 0];
-        bool wide = knn_wide_box(P.box_off[b + 1] - P.box_off[b]);
-        if (FB) {
-            if (wide) vp_knn<KNN_IB_LARGE>(P.grid, b, qx, qy, qz, P.kn, d2, idx, sd);
-            else vp_knn<KNN_IB_SMALL>(P.grid, b, qx, qy, qz, P.kn, d2, idx, sd);
-        } else {
-            CandQuery Q = cand_query(P.grid, b, qx, qy, qz);
-            if (wide)
-                cand_knn<KNN_IB_LARGE>(Q.items, P.grid.cand, Q.a, Q.e, qx, qy, qz, Q.rq_up, Q.w,
-                                       P.kn, d2, idx);
-            else
-                cand_knn<KNN_IB_SMALL>(Q.items, P.grid.cand, Q.a, Q.e, qx, qy, qz, Q.rq_up, Q.w,
-                                       P.kn, d2, idx);
-        }
+        CandQuery Q = cand_query(P.grid, b, qx, qy, qz);
+        if (knn_wide_box(P.box_off[b + 1] - P.box_off[b]))
+            vp_knn<KNN_IB_LARGE>(P.grid, b, Q, qx, qy, qz, P.kn, d2, idx, scratch[threadIdx.x >> 5]);
+        else
+            vp_knn<KNN_IB_SMALL>(P.grid, b, Q, qx, qy, qz, P.kn, d2, idx, scratch[threadIdx.x >> 5]);
         acc += (unsigned long long)idx;
     }
     if (lane == 0 && acc == 0xffffffffffffffffull) *sink = acc;
@@ -518,12 +508,9 @@ static rt_status tune_grid(rt_ctx *c, cudaStream_t st) {
         cell_lists(c, st);
         if ((s = cand_lists(c, st)) != RT_OK) break;
         cudaEventRecord(e0, st);
-        // the probe takes the instance the virtual particles will (with the grid-walk
-        // fallback only when some cell has no list)
         unsigned long long *sink = (unsigned long long *)&P.cnt[CNT_N - 1];   // an unused counter
         int pb = rt_blocks((P.n / 4 + 1) * 32, tb, 152 * 64);
-        if (c->cand_fallback > 0) k_knn_probe<true><<<pb, tb, 0, st>>>(P, sink);
-        else k_knn_probe<false><<<pb, tb, 0, st>>>(P, sink);
+        k_knn_probe<<<pb, tb, 0, st>>>(P, sink);
         cudaEventRecord(e1, st);
         cudaEventSynchronize(e1);
         float ms = 0.f;
@@ -576,7 +563,7 @@ rt_status rt_knn_build(rt_ctx *c, cudaStream_t st) {
 // failed search
 __global__ void __launch_bounds__(256) k_query(DevPtrs P, int b, long long m, const int *q,
                                                int *nbr, long long *d2out, int *fail) {
-    __shared__ int sdelta[8][32];
+    __shared__ unsigned scratch[8][32];
     int lane = threadIdx.x & 31;
     long long w0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -588,9 +575,10 @@ __global__ void __launch_bounds__(256) k_query(DevPtrs P, int b, long long m, co
         long long d2 = -1;
         int idx = 0;
         if (ok) {
-            int *sd = sdelta[threadIdx.x >> 5];
-            ok = wide ? vp_knn<KNN_IB_LARGE>(P.grid, b, qx, qy, qz, P.kn, d2, idx, sd)
-                      : vp_knn<KNN_IB_SMALL>(P.grid, b, qx, qy, qz, P.kn, d2, idx, sd);
+            unsigned *sd = scratch[threadIdx.x >> 5];
+            CandQuery Q = cand_query(P.grid, b, qx, qy, qz);
+            ok = wide ? vp_knn<KNN_IB_LARGE>(P.grid, b, Q, qx, qy, qz, P.kn, d2, idx, sd)
+                      : vp_knn<KNN_IB_SMALL>(P.grid, b, Q, qx, qy, qz, P.kn, d2, idx, sd);
             if (!ok && lane == 0) atomicOr(fail, 2);
         }
         if (lane < P.kn) {

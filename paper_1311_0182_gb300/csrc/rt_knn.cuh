@@ -407,6 +407,154 @@ __device__ inline bool cand_knn(const int4 *items, const unsigned *cand, long lo
     return kth != KNN_KEY_NONE && (IB == KNN_IB_SMALL || (long long)(kth >> IB) < knn_d2max<IB>());
 }
 
+// ---- the search itself: 32-bit keys --------------------------------------------------------
+// compare-exchange of an ascending network: the lower lane of the pair keeps the smaller key
+__device__ __forceinline__ void key_step(unsigned &k, int partner, bool lower) {
+    unsigned o = __shfl_xor_sync(FULLMASK, k, partner);
+    k = lower ? min(k, o) : max(k, o);
+}
+__device__ __forceinline__ void key_merge(unsigned &k) {   // a bitonic sequence -> ascending
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) key_step(k, j, (lane & j) == 0);
+}
+__device__ __forceinline__ void key_sort(unsigned &k) {    // ascending across the warp
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int s = 2; s <= 32; s <<= 1) {
+        key_step(k, s - 1, (lane & (s >> 1)) == 0);
+#pragma unroll
+        for (int j = s >> 2; j > 0; j >>= 1) key_step(k, j, (lane & j) == 0);
+    }
+}
+
+#define KEY32_NONE 0xffffffffu
+#define KEY32_SLACK 4u         // keys of two candidates closer than this leave their order open
+
+// The kn nearest of q among a cell's candidates, in (d2, index) order: lane l < kn returns the
+// l-th nearest.  Works on 32-bit keys: the distance squared in FP32, scaled so that the farthest
+// of the first 96 candidates is just below 2^23 (a fused multiply-add onto 2^23 leaves the
+// scaled value in the low bits), above seven bits that say where in the list the candidate
+// stands.  A compare-exchange is then a shuffle and a min or max, where exact 64-bit keys take
+// about ten instructions; distances and exact order are recomputed for the kn found.  Three
+// batches of 32 are loaded at once (a query scans about 95 candidates); the first is sorted, and
+// what of the others is nearer than its last is packed together, sorted and merged.
+// The scaled value is within 2 of the exact one (three FP32 roundings of the distance at 2^23,
+// half a unit of the last one), so two keys more than 4 apart are in exact order.  When two
+// neighbours among the kn + 1 smallest are closer (ties above all), or the list cannot be stopped
+// within 128 entries, or it is empty, the answer is false and the caller takes the exact search:
+// results are those of warp_knn either way.
+// items: the box's items as (x, y, z, index); cd: the list, len its length; rq_up: an upper bound
+// on the distance of q from the cell's centre; w: ring width; list: 32 words of the warp.
+
+// squared distance of the candidate of list entry `ent` from (fx, fy, fz) (three roundings)
+__device__ __forceinline__ float cand_dist(const float4 *items, unsigned ent, float fx, float fy,
+                                           float fz) {
+    const float4 it = __ldg(items + (ent & 0xffffffu));
+    const float dx = it.x - fx, dy = it.y - fy, dz = it.z - fz;   // exact: coordinates below 2^20
+    return __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, dz * dz));
+}
+
+// The order: f0, f1, f2 are the distances of the lane's candidates of the first three batches
+// (any value beyond the list); on success lane l < kn holds in `at` the place in the list of
+// the l-th nearest.
+__device__ __forceinline__ bool cand_order(float f0, float f1, float f2, const float4 *items,
+                                           const unsigned *cd, int len, float fx, float fy, float fz,
+                                           float rq_up, int w, int kn, unsigned *list, int &at) {
+    const int lane = threadIdx.x & 31;
+    if (len < kn) return false;
+    const bool v0 = lane < len, v1 = lane + 32 < len, v2 = lane + 64 < len;
+    // (distances are >= 0: their bits order like the values)
+    const float mx = __uint_as_float(__reduce_max_sync(
+        FULLMASK, max(max(v0 ? __float_as_uint(f0) : 0u, v1 ? __float_as_uint(f1) : 0u),
+                      v2 ? __float_as_uint(f2) : 0u)));
+    if (!(mx > 0.0f)) return false;
+    const float sc = __fdividef(8388600.0f, mx);
+    auto key = [&](float f, int at) {
+        return (__float_as_uint(fminf(__fmaf_rn(f, sc, 8388608.0f), 16777215.0f)) << 7) |
+               (unsigned)at;
+    };
+    unsigned k = v0 ? key(f0, lane) : KEY32_NONE;
+    key_sort(k);
+    unsigned rest = KEY32_NONE;       // the lane's smallest key left out
+    auto take = [&](unsigned a, unsigned b) {
+        const unsigned kth = __shfl_sync(FULLMASK, k, 31);
+        const bool pa = a < kth, pb = b < kth;
+        const unsigned ma = __ballot_sync(FULLMASK, pa), mb = __ballot_sync(FULLMASK, pb);
+        const int ca = __popc(ma), c = ca + __popc(mb);
+        rest = min(rest, min(pa ? KEY32_NONE : a, pb ? KEY32_NONE : b));
+        if (c == 0) return;
+        const unsigned below = (1u << lane) - 1u;
+        for (int turn = c > 32 ? 0 : 2; turn < 3; ++turn) {   // one turn, or a and b one by one
+            unsigned o = turn == 0 ? a : b;
+            if (turn == 2) {
+                if (c > 32) break;
+                if (pa) list[__popc(ma & below)] = a;
+                if (pb) list[ca + __popc(mb & below)] = b;
+                __syncwarp();
+                o = lane < c ? list[lane] : KEY32_NONE;
+                __syncwarp();
+            }
+            key_sort(o);
+            o = __shfl_xor_sync(FULLMASK, o, 31);
+            rest = min(rest, max(k, o));
+            k = min(k, o);
+            key_merge(k);
+        }
+    };
+    // no entry from `ent` on can be among the kn nearest: its ring is out of their reach
+    auto beyond = [&](unsigned ent) {
+        const float kv = (float)((__shfl_sync(FULLMASK, k, kn - 1) >> 7 & 0x7fffffu) + KEY32_SLACK);
+        const float reach = sqrtf(kv * mx * (1.00002f / 8388600.0f)) * 1.00001f + rq_up;
+        return (float)((int)(ent >> 24) * w) > reach;
+    };
+    unsigned ka = v1 ? key(f1, lane + 32) : KEY32_NONE, kb = v2 ? key(f2, lane + 64) : KEY32_NONE;
+#pragma unroll 1
+    for (int seen = 96;; seen += 32) {
+        take(ka, kb);
+        if (len <= seen) break;
+        const unsigned n = lane + seen < len ? __ldg(cd + lane + seen) : 0u;
+        if (beyond(__shfl_sync(FULLMASK, n, 0))) break;
+        if (seen >= 128) return false;
+        ka = lane + seen < len ? key(cand_dist(items, n, fx, fy, fz), lane + seen) : KEY32_NONE;
+        kb = KEY32_NONE;
+    }
+    const unsigned v = k >> 7, p = __shfl_up_sync(FULLMASK, v, 1);
+    bool open = lane > 0 && lane <= kn && v - p <= KEY32_SLACK;
+    const unsigned r = __reduce_min_sync(FULLMASK, rest) >> 7;
+    open = open || (kn == 32 && lane == 31 && r - v <= KEY32_SLACK);
+    if (__any_sync(FULLMASK, open)) return false;
+    at = (int)(k & 127u);
+    return true;
+}
+
+// exact squared distance of a candidate
+__device__ __forceinline__ long long exact_d2(float4 it, float fx, float fy, float fz) {
+    const long long dx = (int)(it.x - fx), dy = (int)(it.y - fy), dz = (int)(it.z - fz);
+    return dx * dx + dy * dy + dz * dz;
+}
+
+__device__ __forceinline__ bool cand_knn_fast(const float4 *items, const unsigned *cd, int len,
+                                              int qx, int qy, int qz, float rq_up, int w, int kn,
+                                              unsigned *list, long long &d2, int &idx) {
+    const int lane = threadIdx.x & 31;
+    const float fx = (float)qx, fy = (float)qy, fz = (float)qz;
+    float f[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+        f[b] = lane + 32 * b < len ? cand_dist(items, __ldg(cd + lane + 32 * b), fx, fy, fz) : 0.0f;
+    int at = 0;
+    if (!cand_order(f[0], f[1], f[2], items, cd, len, fx, fy, fz, rq_up, w, kn, list, at)) return false;
+    d2 = 0;
+    idx = 0;
+    if (lane < kn) {
+        const float4 it = __ldg(items + (__ldg(cd + at) & 0xffffffu));
+        d2 = exact_d2(it, fx, fy, fz);
+        idx = __float_as_int(it.w);
+    }
+    return true;
+}
+
 // A cell keeps a candidate list when its walk radius (in cells, from U) is at most CAND_R_MAX
 // and the list holds at most CAND_MAX entries.  Other cells (deep in a void, where the n_ngb
 // nearest lie far away and U takes in a large part of a distant cluster) get an empty list; a
@@ -418,8 +566,9 @@ __device__ inline bool cand_knn(const int4 *items, const unsigned *cand, long lo
 // The query of a virtual particle at (qx, qy, qz) in box b: its cell's list, ring width and
 // the bound on its distance to the cell's centre point.
 struct CandQuery {
-    const int4 *items;
-    long long a, e;
+    const float4 *items;      // the box's items
+    long long a;              // the cell's list
+    int len;
     int w;
     float rq_up;
 };
@@ -430,8 +579,8 @@ __device__ __forceinline__ CandQuery cand_query(const Grid &gr, int b, int qx, i
     int cx = cell_coord(qx, cs, G), cy = cell_coord(qy, cs, G), cz = cell_coord(qz, cs, G);
     long long cell = coff + ((long long)cx * G + cy) * G + cz;
     Q.a = gr.cand_off[cell];
-    Q.e = gr.cand_off[cell + 1];
-    Q.items = gr.items + gr.start[coff];
+    Q.len = (int)(gr.cand_off[cell + 1] - Q.a);   // at most CAND_MAX
+    Q.items = gr.fitems + gr.start[coff];
     Q.w = cand_ring_width(cs);
     long long mx = cand_centre(cx * cs, cs) - qx, my = cand_centre(cy * cs, cs) - qy,
               mz = cand_centre(cz * cs, cs) - qz;
@@ -457,26 +606,32 @@ struct KnnOut {
     bool ok;
 };
 
-// The grid walk for a query in a cell without a candidate list, kept out of line: it is rare,
-// and inlined it would take registers from the common path.  Called by the whole warp.
+// The exact search of the box, for a query whose cell has no candidate list (the grid walk) or
+// whose nearest candidates the 32-bit keys cannot order (the list with 64-bit keys).  Out of
+// line: it is rare, and inlined it would take registers from the common path.  Called by the
+// whole warp.
 template <int IB>
-__device__ __noinline__ KnnOut knn_walk_query(BoxGrid g, int qx, int qy, int qz, int kn,
-                                              int *sdelta) {
+__device__ __noinline__ KnnOut knn_exact_query(BoxGrid g, const unsigned *cand, long long a,
+                                               long long e, float rq_up, int w, int qx, int qy,
+                                               int qz, int kn, int *sdelta) {
     KnnOut o;
-    o.ok = warp_knn<IB>(g, qx, qy, qz, -1, kn, o.d2, o.idx, sdelta);
+    if (e > a)
+        o.ok = cand_knn<IB>(g.items + g.start[g.coff], cand, a, e, qx, qy, qz, rq_up, w, kn, o.d2, o.idx);
+    else
+        o.ok = warp_knn<IB>(g, qx, qy, qz, -1, kn, o.d2, o.idx, sdelta);
     return o;
 }
 
-// The virtual particles' exact kNN of (qx, qy, qz) in box b: from the cell's candidate list,
-// or by the grid walk where the cell has none.  Both give warp_knn's result.  sdelta: 32 ints
-// of shared memory owned by the calling warp (the grid walk's).
+// The virtual particles' exact kNN of (qx, qy, qz) in box b.  scratch: 32 words of shared
+// memory owned by the calling warp.  False as warp_knn's.
 template <int IB>
-__device__ __forceinline__ bool vp_knn(const Grid &gr, int b, int qx, int qy, int qz, int kn,
-                                       long long &d2, int &idx, int *sdelta) {
-    CandQuery Q = cand_query(gr, b, qx, qy, qz);
-    if (Q.e > Q.a)
-        return cand_knn<IB>(Q.items, gr.cand, Q.a, Q.e, qx, qy, qz, Q.rq_up, Q.w, kn, d2, idx);
-    KnnOut o = knn_walk_query<IB>(grid_of_box(gr, b), qx, qy, qz, kn, sdelta);
+__device__ __forceinline__ bool vp_knn(const Grid &gr, int b, const CandQuery &Q, int qx, int qy,
+                                       int qz, int kn, long long &d2, int &idx, unsigned *scratch) {
+    if (cand_knn_fast(Q.items, gr.cand + Q.a, Q.len, qx, qy, qz, Q.rq_up, Q.w, kn, scratch, d2, idx))
+        return IB == KNN_IB_SMALL ||
+               __shfl_sync(FULLMASK, d2, kn - 1) < knn_d2max<IB>();
+    KnnOut o = knn_exact_query<IB>(grid_of_box(gr, b), gr.cand, Q.a, Q.a + Q.len, Q.rq_up, Q.w, qx,
+                                   qy, qz, kn, (int *)scratch);
     d2 = o.d2;
     idx = o.idx;
     return o.ok;

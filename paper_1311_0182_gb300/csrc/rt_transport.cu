@@ -389,6 +389,12 @@ __global__ void k_emit_rec(DevPtrs P, int *lens, int np) {
     double NHI = x * NH;
     ((Real *)P.dep_s)[i] = NHI > 0.0 ? (Real)(FX_ABS_SCALE * nm / NHI) : Real(0);
     ((Real *)P.depE_s)[i] = NHI > 0.0 ? (Real)(FX_E_SCALE * nm * P.eunit / (NHI * EV_ERG)) : Real(0);
+    // the four a virtual particle reads of a neighbour, in one piece
+    Real *pv = (Real *)P.vpv + 4 * i;
+    pv[0] = ((Real *)P.Vr)[i];
+    pv[1] = (Real)nHI;
+    pv[2] = ((Real *)P.dep_s)[i];
+    pv[3] = ((Real *)P.depE_s)[i];
     double Nr = P.Nrec[i];
     if (!(Nr > 0.0) || P.rec_mode == RT_REC_EMISSION_CONES) return;
     double e_phys = Nr / (double)NRC;
@@ -981,71 +987,127 @@ template <typename Real> struct VDec {
     long long h2, boff;
     unsigned long long fid;
     Real N, d0, d1, d2, clk, eps, sg, sig, bu;
+    float f0, f1, f2, h2f;        // the direction and the smoothing length squared in FP32
     int box, qx, qy, qz, nu, H;
 };
-// requests a warp takes together: one lane decodes each, into shared memory
+// requests a warp takes together
 #ifndef VREQ_GROUP
 #define VREQ_GROUP 4
 #endif
 
-// Virtual particles (Sec. 2.1): one warp per request.
+// volume, n_HI and deposit scales of a particle
+__device__ __forceinline__ void vpv_load(const DevPtrs &P, long long j, float &V, float &n, float &a,
+                                         float &e) {
+    float4 v = ((const float4 *)P.vpv)[j];
+    V = v.x; n = v.y; a = v.z; e = v.w;
+}
+__device__ __forceinline__ void vpv_load(const DevPtrs &P, long long j, double &V, double &n,
+                                         double &a, double &e) {
+    double2 v = ((const double2 *)P.vpv)[2 * j], w = ((const double2 *)P.vpv)[2 * j + 1];
+    V = v.x; n = v.y; a = w.x; e = w.y;
+}
+
+// a / b, correctly rounded, for 0 < a <= b from y = the correctly rounded 1 / b (div_by_rcp);
+// the plain division where the exact remainder could underflow
+__device__ __forceinline__ double share_of(double a, double b, double y) {
+    return a > 1e-200 && b < 1e200 ? div_by_rcp(a, b, y) : a / b;
+}
+__device__ __forceinline__ float share_of(float a, float b, float y) {
+    if (!(a > 1e-20f && b < 1e20f)) return a / b;
+    float q = __fmul_rn(a, y);
+    return __fmaf_rn(__fmaf_rn(-q, b, a), y, q);
+}
+__device__ __forceinline__ double rcp_rn(double b) { return __drcp_rn(b); }
+__device__ __forceinline__ float rcp_rn(float b) { return __frcp_rn(b); }
+
+// Virtual particles (Sec. 2.1): a warp takes up to VREQ_GROUP consecutive requests at a time and
+// passes over them in six turns, alternating between lane v serving request v (what a request
+// needs once) and all lanes serving one request after the other:
+//   1 lane v    decode: slot or free packet, direction, clock, identity
+//   2 all       position: first accepted of 64 counter-based draws, lane = draw
+//   3 lane v    escape test, cell and candidate list
+//   4 all       exact kNN (rt_knn.cuh); n_HI interpolated over the neighbours, lane = neighbour
+//   5 lane v    attenuation; the packet of the next hop
+//   6 all       deposits, lane = neighbour
+// What bounds it: instruction issue and the latency of dependent loads with FP32 packets; FP64
+// (16 cycles of an SM a warp instruction) with FP64 packets.  With one request after the other
+// through everything, each of the once-a-request parts took a whole warp's instructions, the
+// exponential and four divisions among them; here four requests share them, and the loads of
+// turn 3 and the stores of turn 5 overlap.  Measured steps against one request at a
+// time with 64-bit keys: 64^3 HII region 34.6 -> 32.0 ms, the FP64 path at 32^3 19.1 -> 15.7 ms, the
+// shadow test (FP64) 8.7 -> 7.8 ms.
+// Work queue: every warp of the launch takes its next group from one device counter (CNT_VQ,
+// zero before the hop), so all resident warps stay busy until the requests run out, whatever
+// each request costs; the grid is one wave of resident blocks.  Results do not depend on which
+// warp takes a request.
 // BAR: some box has a barrier (a separate instance keeps the test out of the common case);
-// SH: the shared frequency bin (likewise); IB: index bits of the kNN keys (24 when a box holds
-// more than 2^22 particles); FB: some cell has no candidate list, and queries there take the
-// grid walk (a separate instance keeps that call, and the registers it costs, out of the
-// common case)
+// SH: the shared frequency bin (likewise); IB: index bits of the exact kNN's keys (24 when a box
+// holds more than 2^22 particles)
 // cur, fcur: the hop's slot and free-packet buffers (launch parameters, so that buffer
 // pointers are re-read from the parameter space instead of being held in registers); the
 // step and hop of the random draws are read from the device counters where they are used.
-template <typename Real, int NRC, bool BAR, bool SH, int IB, bool FB>
+template <typename Real, int NRC, bool BAR, bool SH, int IB>
 __global__ void __launch_bounds__(256, VIRT_MINB(Real)) k_virtual(DevPtrs P, int cur, int fcur,
-                                                 const int *lens) {
-    int lane = threadIdx.x & 31;
+                                                                  const int *lens) {
+    __shared__ VDec<Real> sdec[8][VREQ_GROUP];
+    __shared__ CandQuery scell[8][VREQ_GROUP];
+    __shared__ int3 spos[8][VREQ_GROUP];
+    // the distances of the first 96 candidates; then the neighbours' distances, replaced by their
+    // weights in the interpolated n_HI, their deposit scales and indices
+    union Work {
+        float f[VREQ_GROUP][96];
+        struct { Real wn[VREQ_GROUP][32], ds[VREQ_GROUP][32], de[VREQ_GROUP][32]; int j[VREQ_GROUP][32]; } n;
+    };
+    __shared__ Work swork[8];
+    __shared__ int sat[8][VREQ_GROUP][32];    // the neighbours' places in the candidate list
+    __shared__ unsigned scratch[8][32];
+    __shared__ unsigned sstep[2];             // step, hop << 8
+    // per warp (its lane 0 keeps them): packets that go on, virtual particles outside their box,
+    // and the escaped photons of one box (other boxes' are booked at once)
+    __shared__ int scount[8][2], sebox[8];
+    __shared__ unsigned long long sesc[8];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (threadIdx.x < 2) {
+        sstep[threadIdx.x] = threadIdx.x ? cnt_word(P, CNT_HOP) << 8 : cnt_word(P, CNT_STEP);
+    }
+    if (threadIdx.x < 8) {
+        sesc[threadIdx.x] = 0ull;
+        sebox[threadIdx.x] = -1;
+        scount[threadIdx.x][0] = scount[threadIdx.x][1] = 0;
+    }
+    __syncthreads();
     long long nreq = lens[2];
     if (nreq > P.F_cap) nreq = P.F_cap;
-    FreeBuf Fi = P.fr[fcur], Fo = P.fr[fcur ^ 1];
-    Slots<Real> S(P, cur);
-    uint2 key = philox_key(P.seed, 3u);
-    // A warp takes VREQ_GROUP consecutive requests at a time; lane v decodes request v of the
-    // group (slot or free packet, direction, clock, identity, per-box and per-frequency values)
-    // into shared memory, so that the group's loads and divisions run side by side instead of
-    // once per request on every lane.  Then the warp serves the requests one after the other.
-    // Latency: the kNN search loads each batch of its cell's candidates before merging the
-    // previous one; the four per-neighbour inputs of the interpolation and deposit are gathered
-    // together; the values returned by the deposit atomics are checked one request later.
-    // Work queue: every warp of the launch takes its next group from one device counter
-    // (CNT_VQ, set to zero before the hop), so all resident warps stay busy until the requests
-    // run out, whatever each request costs; the grid is one wave of resident blocks.  (Blocks
-    // that own a fixed chunk each leave most of their warps idle while the slowest finishes:
-    // 25 of 40 warps per SM were active.)  Results do not depend on which warp takes a request.
-    __shared__ VDec<Real> sdec[8][VREQ_GROUP];
-    __shared__ int sdelta[FB ? 8 : 1][32];   // the grid walk of cells without a candidate list
-    VDec<Real> *mine = sdec[threadIdx.x >> 5];
+    const FreeBuf Fi = P.fr[fcur], Fo = P.fr[fcur ^ 1];
+    VDec<Real> *mine = sdec[wid];
     unsigned long long *queue = (unsigned long long *)&P.cnt[CNT_VQ];
     const float cf = 1.0f - 2.0f / (float)P.ntc;
-    // requests a warp takes at a time: fewer when the hop has fewer than the warps could take
-    const int grp = (int)min((long long)VREQ_GROUP, 1 + nreq / (long long)(gridDim.x * 8u));
-    unsigned long long pend_a = 0ull, pend_e = 0ull;   // words before this lane's last adds
+    // requests a warp takes at a time: fewer when few are left, so that the warps end together
+    const long long nwarps = 8ll * gridDim.x;
+    int grp = (int)min((long long)VREQ_GROUP, 1 + nreq / nwarps);
+    // words before this lane's last adds, checked a group later (no wait for the atomics).  With
+    // FP64 packets, bound by FP64 and short of instruction cache, the deposits are not unrolled and
+    // a request's words are checked at the next one's.
+    constexpr int DU = sizeof(Real) == 4 ? VREQ_GROUP : 1;
+    unsigned long long pend_a[DU], pend_e[DU];
+#pragma unroll
+    for (int v = 0; v < DU; ++v) pend_a[v] = pend_e[v] = 0ull;
     bool bad = false, bad_knn = false;
-    // the block's packets that go on and virtual particles outside their box; per warp, the
-    // escaped photons not yet booked with their box (in shared memory: only lane 0 of a warp
-    // keeps them, and registers are what this kernel is short of)
-    __shared__ int stot[2], sebox[8];
-    __shared__ unsigned long long sesc[8];
-    if (threadIdx.x < 2) stot[threadIdx.x] = 0;
-    if (threadIdx.x < 8) sesc[threadIdx.x] = 0ull;
-    __syncthreads();
     for (;;) {
         long long g0 = 0;
         if (lane == 0) g0 = (long long)atomicAdd(queue, (unsigned long long)grp);
         g0 = __shfl_sync(FULLMASK, g0, 0);
         if (g0 >= nreq) break;
         const int gn = (int)(nreq - g0 < grp ? nreq - g0 : grp);
+        const long long r = g0 + lane;          // the lane's request (lane < gn)
+        grp = (int)min((long long)VREQ_GROUP, 1 + (nreq - g0) / nwarps);
+        // ---- 1: decode
         if (lane < gn) {
-            unsigned long long code = P.req[g0 + lane];
+            unsigned long long code = P.req[r];
             VDec<Real> D;
             D.sg = Real(0);          // shared bin: the packet's mean cross-section (sunit)
             if (!(code & RT_FREE_BIT)) {
+                Slots<Real> S(P, cur);
                 long long i = (unsigned)code / (unsigned)P.S;   // slot codes < 2^31
                 int s = (int)((unsigned)code % (unsigned)P.S);
                 D.nu = s / NRC;
@@ -1074,166 +1136,269 @@ __global__ void __launch_bounds__(256, VIRT_MINB(Real)) k_virtual(DevPtrs P, int
             D.sig = (SH && D.nu == 0) ? D.sg * (Real)P.sunit : sigma_of<Real>(P, D.nu);
             D.bu = box_unit<Real>(P, D.box);
             D.H = (int)isqrt64(D.h2);   // = floor(sqrt(h2)) exactly (h2 < 3 * 2^40), < 2^21
+            D.f0 = (float)D.d0; D.f1 = (float)D.d1; D.f2 = (float)D.d2;
+            D.h2f = i64_to_f(D.h2);
             mine[lane] = D;
         }
         __syncwarp();
+        // ---- 2: positions
+        int Dx = 0, Dy = 0, Dz = 0;             // the lane's request's offset, |D| <= H < 2^21
+        bool found = false;
+#pragma unroll 1
         for (int v = 0; v < gn; ++v) {
-            const long long r = g0 + v;
-            const int box = mine[v].box, qx = mine[v].qx, qy = mine[v].qy, qz = mine[v].qz,
-                      nu = mine[v].nu;
-            const long long h2 = mine[v].h2, boff = mine[v].boff;
-            const Real N = mine[v].N, d0 = mine[v].d0, d1 = mine[v].d1, d2 = mine[v].d2,
-                       clk = mine[v].clk, eps = mine[v].eps, sg = mine[v].sg, sig = mine[v].sig,
-                       bu = mine[v].bu;
+            const int H = mine[v].H;
+            const unsigned span = (unsigned)(2 * H + 1);   // < 2^22
             const unsigned long long fid = mine[v].fid;
-            const bool sgs = SH && nu == 0;
-            // position: first accepted of 64 counter-based draws in [-H, H]^3, else on the axis
-            const long long H = mine[v].H;
-            unsigned span = (unsigned)(2 * H + 1);   // < 2^22
-            int Dx = 0, Dy = 0, Dz = 0;   // |D| <= H < 2^21
-            bool found = false;
-            for (int a0 = 0; a0 < 64 && !found; a0 += 32) {
+            const float f0 = mine[v].f0, f1 = mine[v].f1, f2 = mine[v].f2, h2f = mine[v].h2f;
+            const uint2 key = philox_key(P.seed, 3u);
+#pragma unroll 1
+            for (int a0 = 0; a0 < 64; a0 += 32) {
                 unsigned a = (unsigned)(a0 + lane);
-                // counter: (step, hop << 8 | draw, packet id); step and hop from the device counters
-                uint4 u = philox4x32_10(make_uint4(cnt_word(P, CNT_STEP), (cnt_word(P, CNT_HOP) << 8) | a,
-                                                   (unsigned)fid, (unsigned)(fid >> 32)), key);
+                // counter: (step, hop << 8 | draw, packet id)
+                uint4 u = philox4x32_10(make_uint4(sstep[0], sstep[1] | a, (unsigned)fid, (unsigned)(fid >> 32)), key);
                 // floor(u * span / 2^32) - H, |e| <= H < 2^21: 32-bit integers (a 64-bit integer to
                 // float conversion would run on the FP64 pipe)
-                int ix = (int)__umulhi(u.x, span) - (int)H;
-                int iy = (int)__umulhi(u.y, span) - (int)H;
-                int iz = (int)__umulhi(u.z, span) - (int)H;
-                long long ex = ix, ey = iy, ez = iz;
-                long long r2 = ex * ex + ey * ey + ez * ez;
-                bool ok = r2 > 0 && r2 <= h2 &&
-                          cone_test<Real>(ix, iy, iz, (float)ix, (float)iy, (float)iz, d0, d1, d2, cf,
-                                          P.ntc);
+                int ix = (int)__umulhi(u.x, span) - H;
+                int iy = (int)__umulhi(u.y, span) - H;
+                int iz = (int)__umulhi(u.z, span) - H;
+                const float fx = (float)ix, fy = (float)iy, fz = (float)iz;
+                const float r2 = __fmaf_rn(fx, fx, __fmaf_rn(fy, fy, fz * fz));
+                const float cs = __fmaf_rn(fx, f0, __fmaf_rn(fy, f1, fz * f2)) * rsqrtf(r2);
+                // inside the sphere and the cone; FP32 with guard bands (relative error of r2 below
+                // 2e-7), the exact tests inside them
+                bool ok = r2 > 0.0f && r2 < h2f * 0.999999f && cs > cf + CONE_BAND;
+                const bool open = r2 > 0.0f && !ok && r2 < h2f * 1.000001f && !(cs < cf - CONE_BAND);
+                if (__any_sync(FULLMASK, open)) {
+                    if (open) {
+                        long long ex = ix, ey = iy, ez = iz;
+                        ok = ex * ex + ey * ey + ez * ez <= mine[v].h2 &&
+                             (cs > cf + CONE_BAND ||
+                              cone_exact(ix, iy, iz, (double)mine[v].d0, (double)mine[v].d1,
+                                         (double)mine[v].d2, P.ntc));
+                    }
+                }
                 unsigned m = __ballot_sync(FULLMASK, ok);
                 if (m) {
                     int src = __ffs(m) - 1;
-                    Dx = __shfl_sync(FULLMASK, ix, src);
-                    Dy = __shfl_sync(FULLMASK, iy, src);
-                    Dz = __shfl_sync(FULLMASK, iz, src);
-                    found = true;
+                    ix = __shfl_sync(FULLMASK, ix, src);
+                    iy = __shfl_sync(FULLMASK, iy, src);
+                    iz = __shfl_sync(FULLMASK, iz, src);
+                    if (lane == v) { Dx = ix; Dy = iy; Dz = iz; found = true; }
+                    break;
                 }
             }
-            if (!found) axis_offset(d0, d1, d2, H, Dx, Dy, Dz);
-            int vx = qx + Dx, vy = qy + Dy, vz = qz + Dz;
+        }
+#pragma unroll
+        for (int v = 0; v < DU; ++v) bad |= pend_a[v] > (1ull << 62) || pend_e[v] > (1ull << 62);
+        // ---- 3: escapes; cells
+        bool alive = false;
+        int gone = 0, box = 0;
+        if (lane < gn) {
+            const VDec<Real> &D = mine[lane];
+            box = D.box;
+            if (!found) axis_offset(D.d0, D.d1, D.d2, (long long)D.H, Dx, Dy, Dz);
+            const int vx = D.qx + Dx, vy = D.qy + Dy, vz = D.qz + Dz;
             // outside the box: the photons escape (1); on a path through the barrier they are
             // removed, counted with the escapes (3)
-            int gone = (vx < 0 || vy < 0 || vz < 0 || vx >= RT_Q || vy >= RT_Q || vz >= RT_Q) ? 1
-                     : (BAR && barrier_crosses_call(P.bar[box], qx, qy, qz, vx, vy, vz)) ? 3 : 0;
+            gone = (vx < 0 || vy < 0 || vz < 0 || vx >= RT_Q || vy >= RT_Q || vz >= RT_Q) ? 1
+                     : (BAR && barrier_crosses_call(P.bar[box], D.qx, D.qy, D.qz, vx, vy, vz)) ? 3 : 0;
             if (gone) {
-                if (lane == 0) {
-                    const int w = threadIdx.x >> 5;
-                    unsigned long long es = sesc[w];
-                    if (es && box != sebox[w]) {
-                        atomicAdd(&P.esc_fx[sebox[w]], es);
-                        es = 0ull;
-                    }
-                    sebox[w] = box;
-                    sesc[w] = es + esc_fixed(N, P, box);
-                    if (gone == 1) atomicAdd(&stot[1], 1);
-                    ((Real *)Fo.N)[r] = Real(0);
-                }
-                continue;
-            }
-            bad |= pend_a > (1ull << 62) || pend_e > (1ull << 62);
-            // exact kNN from the candidate list of the virtual particle's cell (the grid walk
-            // in a cell without one)
-            long long kd2;
-            int kidx;
-            bool kok;
-            if (FB) {
-                kok = vp_knn<IB>(P.grid, box, vx, vy, vz, P.kn, kd2, kidx,
-                                 sdelta[FB ? threadIdx.x >> 5 : 0]);
+                ((Real *)Fo.N)[r] = Real(0);
             } else {
-                CandQuery Q = cand_query(P.grid, box, vx, vy, vz);
-                kok = cand_knn<IB>(Q.items, P.grid.cand, Q.a, Q.e, vx, vy, vz, Q.rq_up, Q.w, P.kn,
-                                   kd2, kidx);
+                alive = true;
+                spos[wid][lane] = make_int3(vx, vy, vz);
+                scell[wid][lane] = cand_query(P.grid, box, vx, vy, vz);
             }
-            if (!kok) {
+        }
+        const unsigned am = __ballot_sync(FULLMASK, alive), gm = __ballot_sync(FULLMASK, gone != 0);
+        if (gm) {
+            int eb = sebox[wid];
+            if (eb < 0) eb = __shfl_sync(FULLMASK, box, __ffs(gm) - 1);
+            unsigned long long es = gone ? esc_fixed(mine[lane & (VREQ_GROUP - 1)].N, P, box) : 0ull;
+            if (gone && box != eb) {
+                atomicAdd(&P.esc_fx[box], es);
+                es = 0ull;
+            }
+#pragma unroll
+            for (int o = 1; o < VREQ_GROUP; o <<= 1) es += __shfl_xor_sync(FULLMASK, es, o);
+            const int out = __popc(__ballot_sync(FULLMASK, gone == 1));
+            __syncwarp();
+            if (lane == 0) {
+                sebox[wid] = eb;
+                sesc[wid] += es;
+                scount[wid][1] += out;
+            }
+        }
+        __syncwarp();
+        // ---- 4: neighbours and n_HI.  Loads of all four requests side by side: the candidates'
+        // distances; after the order of each, the neighbours and their properties
+        Work &W = swork[wid];
+        const bool valid = lane < P.kn;
+#pragma unroll
+        for (int v = 0; v < VREQ_GROUP; ++v) {
+            if (!((am >> v) & 1u)) continue;
+            const int3 q = spos[wid][v];
+            const float4 *items = scell[wid][v].items;
+            const unsigned *cd = P.grid.cand + scell[wid][v].a;
+            const int len = scell[wid][v].len;
+#pragma unroll
+            for (int b = 0; b < 3; ++b)
+                if (lane + 32 * b < len)
+                    W.f[v][lane + 32 * b] = cand_dist(items, __ldg(cd + lane + 32 * b), (float)q.x,
+                                                      (float)q.y, (float)q.z);
+        }
+#pragma unroll 1
+        for (unsigned m = am; m; m &= m - 1u) {
+            const int v = __ffs(m) - 1;
+            const int3 q = spos[wid][v];
+            const CandQuery Q = scell[wid][v];
+            int at;
+            if (!cand_order(W.f[v][lane], W.f[v][lane + 32], W.f[v][lane + 64], Q.items, P.grid.cand + Q.a,
+                            Q.len, (float)q.x, (float)q.y, (float)q.z, Q.rq_up, Q.w, P.kn, scratch[wid],
+                            at)) {
+                KnnOut o = knn_exact_query<IB>(grid_of_box(P.grid, mine[v].box), P.grid.cand, Q.a,
+                                               Q.a + Q.len, Q.rq_up, Q.w, q.x, q.y, q.z, P.kn,
+                                               (int *)scratch[wid]);
                 // a k-th neighbour beyond the key range: reported; indices kept inside the box
-                bad_knn = true;
-                long long nbx = P.box_off[box + 1] - boff;
-                if (kidx < 0 || kidx >= nbx) { kidx = 0; kd2 = 0; }
+                if (!o.ok) bad_knn = true;
+                const int box = mine[v].box;
+                if (o.idx < 0 || o.idx >= P.box_off[box + 1] - mine[v].boff) o.idx = 0;
+                at = o.idx | INT_MIN;
             }
-            long long h2v = __shfl_sync(FULLMASK, kd2, P.kn - 1);
-            bool valid = lane < P.kn;
-            long long j = valid ? boff + kidx : 0;
-            Real om = Real(0), nhj = Real(0), Vj = Real(0), dsj = Real(0), dej = Real(0);
+            sat[wid][v][lane] = at;
+        }
+        __syncwarp();
+        Real msw = Real(1), mswn = Real(0);
+        long long mh2v = 0;
+        float4 it[VREQ_GROUP];
+#pragma unroll
+        for (int v = 0; v < VREQ_GROUP; ++v) {
+            it[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (!((am >> v) & 1u) || !valid) continue;
+            const int at = sat[wid][v][lane];
+            if (at >= 0) {
+                it[v] = __ldg(scell[wid][v].items + (__ldg(P.grid.cand + scell[wid][v].a + at) & 0xffffffu));
+            } else {   // (the exact search gives the particle)
+                const int i = at & INT_MAX;
+                const int4 p = __ldg(P.q4 + mine[v].boff + i);
+                it[v] = make_float4((float)p.x, (float)p.y, (float)p.z, __int_as_float(i));
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < VREQ_GROUP; ++v) {
+            if (!((am >> v) & 1u)) continue;
+            const int3 q = spos[wid][v];
+            const long long kd2 = exact_d2(it[v], (float)q.x, (float)q.y, (float)q.z);
+            const long long h2v = __shfl_sync(FULLMASK, kd2, P.kn - 1);
+            if (IB != KNN_IB_SMALL && h2v >= knn_d2max<IB>()) bad_knn = true;
+            if (lane == v) mh2v = h2v;
+            W.n.wn[v][lane] = to_real<Real>(kd2);
+            W.n.j[v][lane] = (int)(mine[v].boff + __float_as_int(it[v].w));
+        }
+        // (a lane reads back its own words)
+        Real Vn = Real(0), nn = Real(0), dsn = Real(0), den = Real(0);
+        if (am && valid) vpv_load(P, W.n.j[__ffs(am) - 1][lane], Vn, nn, dsn, den);
+#pragma unroll 1
+        for (unsigned m = am; m; m &= m - 1u) {
+            const int v = __ffs(m) - 1;
+            const Real Vj = Vn, nhj = nn;
+            W.n.ds[v][lane] = dsn;
+            W.n.de[v][lane] = den;
+            const unsigned m2 = m & (m - 1u);   // the next request's neighbours, loaded ahead
+            if (m2 && valid) vpv_load(P, W.n.j[__ffs(m2) - 1][lane], Vn, nn, dsn, den);
+            const Real kr = W.n.wn[v][lane], hr = __shfl_sync(FULLMASK, kr, P.kn - 1);
+            Real om = Real(0);
             if (valid) {
-                Vj = ((Real *)P.Vr)[j];
-                nhj = ((Real *)P.nHIr)[j];
-                dsj = ((Real *)P.dep_s)[j];
-                dej = ((Real *)P.depE_s)[j];
-                Real q = h2v > 0 ? rt_sqrt<Real>(to_real<Real>(kd2) / to_real<Real>(h2v)) : Real(0);
-                om = Vj * kernel_w<Real>(q);
+                Real qq = hr > Real(0) ? rt_sqrt<Real>(kr / hr) : Real(0);
+                om = Vj * kernel_w<Real>(qq);
+                Fo.nbr[(g0 + v) * P.kn + lane] = W.n.j[v][lane];
             }
             Real sw = om;
-    #pragma unroll
+#pragma unroll
             for (int o = 16; o > 0; o >>= 1) sw += __shfl_xor_sync(FULLMASK, sw, o);
             if (!(sw > Real(0))) {
-                om = Vj;
+                om = valid ? Vj : Real(0);
                 sw = om;
-    #pragma unroll
+#pragma unroll
                 for (int o = 16; o > 0; o >>= 1) sw += __shfl_xor_sync(FULLMASK, sw, o);
             }
-            Real wn = om * nhj;
-            Real swn = wn;
-    #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) swn += __shfl_xor_sync(FULLMASK, swn, o);
-            Real nHIv = swn / sw;
-            Real t = (Real)Dx * d0 + (Real)Dy * d1 + (Real)Dz * d2;
-            Real l = t * bu;
-            Real tau = (sig * nHIv) * l;
-            Real A, T;
-            split_absorbed<Real>(N, tau, A, T);
-            if (valid && swn > Real(0) && wn > Real(0)) {
-                Real Ak = A * (wn / swn);
-                long long key2 = j * P.nf + nu;
+            const Real wn = valid ? om * nhj : Real(0);
+            Real sn = wn;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sn += __shfl_xor_sync(FULLMASK, sn, o);
+            W.n.wn[v][lane] = wn;
+            if (lane == v) { msw = sw; mswn = sn; }
+        }
+        // ---- 5: attenuation; the packet of the next hop
+        Real A = Real(0), ry = Real(0);
+        bool on = false;
+        if (alive) {
+            const VDec<Real> &D = mine[lane];
+            const Real nHIv = mswn / msw;
+            const Real t = (Real)Dx * D.d0 + (Real)Dy * D.d1 + (Real)Dz * D.d2;
+            const Real l = t * D.bu;
+            const Real tau = (D.sig * nHIv) * l;
+            Real T;
+            split_absorbed<Real>(D.N, tau, A, T);
+            ry = rcp_rn(mswn);
+            on = T > Real(0);
+            Fo.box[r] = D.box;
+            Fo.qx[r] = D.qx + Dx; Fo.qy[r] = D.qy + Dy; Fo.qz[r] = D.qz + Dz;
+            Fo.h2[r] = mh2v;
+            ((Real *)Fo.N)[r] = T;
+            ((Real *)Fo.dx)[r] = D.d0; ((Real *)Fo.dy)[r] = D.d1; ((Real *)Fo.dz)[r] = D.d2;
+            ((Real *)Fo.clock)[r] = D.clk + l / (Real)C_LIGHT;
+            ((Real *)Fo.eps)[r] = D.eps;
+            if (SH && D.nu == 0) ((Real *)Fo.sig)[r] = D.sg;
+            Fo.nu[r] = D.nu;
+            Fo.fid[r] = mix64(D.fid);
+        }
+        const int non = __popc(__ballot_sync(FULLMASK, on));
+        if (lane == 0) scount[wid][0] += non;
+        // ---- 6: deposits
+#pragma unroll DU
+        for (int v = 0; v < VREQ_GROUP; ++v) {
+            const int ps = DU == 1 ? 0 : v;
+            if (DU == 1) bad |= pend_a[0] > (1ull << 62) || pend_e[0] > (1ull << 62);
+            pend_a[ps] = 0ull;
+            pend_e[ps] = 0ull;
+            if (!((am >> v) & 1u)) continue;
+            const Real Av = __shfl_sync(FULLMASK, A, v), sn = __shfl_sync(FULLMASK, mswn, v),
+                       y = __shfl_sync(FULLMASK, ry, v);
+            const Real wn = W.n.wn[v][lane];
+            if (valid && sn > Real(0) && wn > Real(0)) {
+                const long long j = W.n.j[v][lane];
+                const Real dsj = W.n.ds[v][lane], dej = W.n.de[v][lane];
+                const Real Ak = Av * share_of(wn, sn, y);
+                const long long key2 = j * P.nf + mine[v].nu;
                 // two fixed-point words: units of 2^-40 N_HI and 2^-72 N_HI (integer sums do not
                 // depend on their order)
-                Real fa = Ak * dsj;
-                Real fe = Ak * eps * dej;
-                pend_a = 0ull;
-                pend_e = 0ull;
+                const Real fa = Ak * dsj;
+                const Real fe = Ak * mine[v].eps * dej;
                 if (fa > Real(0)) {
                     unsigned long long qh = 0, ql = 0;
                     bad |= !fx_split(fa, qh, ql);
-                    if (qh) pend_a = atomicAdd(&P.fx_abs[key2], qh);
+                    if (qh) pend_a[ps] = atomicAdd(&P.fx_abs[key2], qh);
                     if (ql) atomicAdd(&P.fx_lo[key2], ql);
                 }
                 if (fe > Real(0)) {
                     bad |= fe > Real(4.0e18);
-                    pend_e = atomicAdd(&P.fx_E[key2], to_fixed(fe));
+                    pend_e[ps] = atomicAdd(&P.fx_E[key2], to_fixed(fe));
                 }
             }
-            if (valid) Fo.nbr[r * P.kn + lane] = (int)j;
-            if (lane == 0) {
-                if (T > Real(0)) atomicAdd(&stot[0], 1);
-                Fo.box[r] = box;
-                Fo.qx[r] = vx; Fo.qy[r] = vy; Fo.qz[r] = vz;
-                Fo.h2[r] = h2v;
-                ((Real *)Fo.N)[r] = T;
-                ((Real *)Fo.dx)[r] = d0; ((Real *)Fo.dy)[r] = d1; ((Real *)Fo.dz)[r] = d2;
-                ((Real *)Fo.clock)[r] = clk + l / (Real)C_LIGHT;
-                ((Real *)Fo.eps)[r] = eps;
-                if (sgs) ((Real *)Fo.sig)[r] = sg;
-                Fo.nu[r] = nu;
-                Fo.fid[r] = mix64(fid);
-            }
         }
-        __syncwarp();   // the group's decoded requests are read before the next group's decode
+        __syncwarp();   // the group's shared values are read before the next group's are written
     }
-    bad |= pend_a > (1ull << 62) || pend_e > (1ull << 62);
+#pragma unroll
+    for (int v = 0; v < DU; ++v) bad |= pend_a[v] > (1ull << 62) || pend_e[v] > (1ull << 62);
     if (bad) atomicOr((unsigned long long *)&P.cnt[CNT_ERR], (unsigned long long)ERRB_RANGE);
     if (bad_knn) atomicOr((unsigned long long *)&P.cnt[CNT_ERR], (unsigned long long)ERRB_KNN);
-    if (lane == 0 && sesc[threadIdx.x >> 5])
-        atomicAdd(&P.esc_fx[sebox[threadIdx.x >> 5]], sesc[threadIdx.x >> 5]);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        if (stot[0]) atomicAdd((unsigned long long *)&P.cnt[CNT_LIVE], (unsigned long long)stot[0]);
-        if (stot[1]) atomicAdd((unsigned long long *)&P.cnt[CNT_VESC], (unsigned long long)stot[1]);
+    if (lane == 0 && sesc[wid]) atomicAdd(&P.esc_fx[sebox[wid]], sesc[wid]);
+    if (threadIdx.x < 2) {
+        int t = 0;
+        for (int k = 0; k < 8; ++k) t += scount[k][threadIdx.x];
+        if (t) atomicAdd((unsigned long long *)&P.cnt[threadIdx.x ? CNT_VESC : CNT_LIVE], (unsigned long long)t);
     }
 }
 
@@ -2013,20 +2178,6 @@ static void set_step(rt_ctx *c, long long step, cudaStream_t st) {
     c->step_dev = step;
 }
 
-// The virtual-particle kernel of the hop: the instance with the grid-walk fallback only when
-// some cell of the context has no candidate list.
-template <typename Real, int NRC, bool BAR, bool SH, int IB>
-static void launch_virtual(rt_ctx *c, cudaStream_t st, int GV, int cur, int fcur) {
-    DevPtrs &P = c->d;
-    HopScratch &H = c->hop;
-    const int tb = 256;
-    int nb = rt_blocks(P.F_cap * 32, tb, GV);
-    if (c->cand_fallback > 0)
-        k_virtual<Real, NRC, BAR, SH, IB, true><<<nb, tb, 0, st>>>(P, cur, fcur, H.lens);
-    else
-        k_virtual<Real, NRC, BAR, SH, IB, false><<<nb, tb, 0, st>>>(P, cur, fcur, H.lens);
-}
-
 // Particles a warp of the sender side takes together: as many as its 32 (particle, frequency)
 // words hold, but no more than leave every resident warp (152 SMs x 32) a turn, since a small
 // box needs its particles spread over the chip more than it needs full lanes.
@@ -2091,16 +2242,17 @@ static void hop_core(rt_ctx *c, cudaStream_t st, long long nfr, int cur, int fcu
         LAUNCH_ON(s2, KT_PHASE_B, 1, (k_phaseB<Real, NRC, false, false><<<nbb, tb, 0, s2>>>(P, cur, H.lens)));
     cudaEventRecord(evB, s2);
     const int IS = KNN_IB_SMALL, IL = KNN_IB_LARGE;
+    const int nbv = rt_blocks(P.F_cap * 32, tb, GV);
     if (P.kwide && P.shared)   // boxes above 2^22 particles: the general instance, 24-bit keys
-        LAUNCH(KT_VIRTUAL, 1, (launch_virtual<Real, NRC, true, true, IL>(c, st, GV, cur, fcur)));
+        LAUNCH(KT_VIRTUAL, 1, (k_virtual<Real, NRC, true, true, IL><<<nbv, tb, 0, st>>>(P, cur, fcur, H.lens)));
     else if (P.kwide)
-        LAUNCH(KT_VIRTUAL, 1, (launch_virtual<Real, NRC, true, false, IL>(c, st, GV, cur, fcur)));
+        LAUNCH(KT_VIRTUAL, 1, (k_virtual<Real, NRC, true, false, IL><<<nbv, tb, 0, st>>>(P, cur, fcur, H.lens)));
     else if (P.shared)
-        LAUNCH(KT_VIRTUAL, 1, (launch_virtual<Real, NRC, true, true, IS>(c, st, GV, cur, fcur)));
+        LAUNCH(KT_VIRTUAL, 1, (k_virtual<Real, NRC, true, true, IS><<<nbv, tb, 0, st>>>(P, cur, fcur, H.lens)));
     else if (P.any_bar)
-        LAUNCH(KT_VIRTUAL, 1, (launch_virtual<Real, NRC, true, false, IS>(c, st, GV, cur, fcur)));
+        LAUNCH(KT_VIRTUAL, 1, (k_virtual<Real, NRC, true, false, IS><<<nbv, tb, 0, st>>>(P, cur, fcur, H.lens)));
     else
-        LAUNCH(KT_VIRTUAL, 1, (launch_virtual<Real, NRC, false, false, IS>(c, st, GV, cur, fcur)));
+        LAUNCH(KT_VIRTUAL, 1, (k_virtual<Real, NRC, false, false, IS><<<nbv, tb, 0, st>>>(P, cur, fcur, H.lens)));
     cudaStreamWaitEvent(st, evB, 0);
 }
 
