@@ -584,6 +584,46 @@ template <> struct KSum<double> {
     __device__ __forceinline__ double get() const { return s; }
 };
 
+// Two values side by side, and two compensated sums added together.  Blackwell adds a pair of
+// FP32 values in one instruction (each rounded as on its own), so a pair of Kahan additions
+// takes four instructions instead of eight (the step of 2.1 M particles behind a fast front: 1.7%).
+template <typename Real> struct PairOf;
+template <> struct PairOf<float> { typedef float2 T; };
+template <> struct PairOf<double> { typedef double2 T; };
+template <typename Real> using Pair = typename PairOf<Real>::T;
+__device__ __forceinline__ float2 make_pair2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ double2 make_pair2(double a, double b) { return make_double2(a, b); }
+
+template <typename Real> struct KSum2;
+template <> struct KSum2<float> {
+    unsigned long long s, c;      // low word: the first of the pair
+    static __device__ __forceinline__ unsigned long long pack(float a, float b) {
+        unsigned long long r;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+        return r;
+    }
+    __device__ __forceinline__ void init(float a, float b) { s = pack(a, b); c = 0ull; }
+    __device__ __forceinline__ void add(float2 v) {
+        unsigned long long y, t;
+        asm("sub.rn.ftz.f32x2 %0, %1, %2;" : "=l"(y) : "l"(pack(v.x, v.y)), "l"(c));
+        asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(t) : "l"(s), "l"(y));
+        asm("sub.rn.ftz.f32x2 %0, %1, %2;" : "=l"(c) : "l"(t), "l"(s));
+        asm("sub.rn.ftz.f32x2 %0, %1, %2;" : "=l"(c) : "l"(c), "l"(y));
+        s = t;
+    }
+    __device__ __forceinline__ float2 get() const {
+        float2 r;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(s));
+        return r;
+    }
+};
+template <> struct KSum2<double> {
+    double2 s;
+    __device__ __forceinline__ void init(double a, double b) { s = make_double2(a, b); }
+    __device__ __forceinline__ void add(double2 v) { s.x = s.x + v.x; s.y = s.y + v.y; }
+    __device__ __forceinline__ double2 get() const { return s; }
+};
+
 static inline int rt_blocks(long long items, int per_block, int cap = 152 * 32) {
     long long b = (items + per_block - 1) / per_block;
     if (b < 1) b = 1;

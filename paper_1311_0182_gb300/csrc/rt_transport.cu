@@ -1512,9 +1512,9 @@ __device__ __forceinline__ unsigned long long deposit_group<float>(const DevPtrs
     return old;
 }
 
-// What the receiver side keeps of one contribution: T, T d (3), T clock, T eps, then A, A eps
-// and w, and T sigma in a shared frequency bin.
-template <bool SH> struct BVals { static constexpr int N = SH ? 10 : 9; };
+// What the receiver side keeps of one contribution, in pairs: (T, T d0), (T d1, T d2),
+// (T clock, T eps), (A, A eps), and w with, in a shared frequency bin, T sigma.
+#define BV_N 5
 
 // One gas contribution to receiver j in frequency nu: reverse edge e, bit b of its word.
 // Attenuates, stores the values in sv[.][lane] and returns its reception cone, or -1 when a
@@ -1522,7 +1522,7 @@ template <bool SH> struct BVals { static constexpr int N = SH ? 10 : 9; };
 template <typename Real, int G, bool BAR, bool SH>
 __device__ __forceinline__ int gas_contribution(const DevPtrs &P, long long e, int b, long long j,
                                                 int nu, int box, Real u, Real sig_nhi,
-                                                Real (*sv)[32], int lane) {
+                                                Pair<Real> (*sv)[32], int lane) {
     float4 ed = __ldg(P.rev4 + e);
     bool sgs = SH && nu == 0;
     Real w, d0, d1, d2, clk, eps, sgc = Real(0);
@@ -1542,29 +1542,24 @@ __device__ __forceinline__ int gas_contribution(const DevPtrs &P, long long e, i
     // in a shared bin each packet carries its own mean cross-section
     Real sn = sgs ? (sgc * (Real)P.sunit) * ((Real *)P.nHIr)[j] : sig_nhi;
     split_absorbed<Real>(w, sn * l, A, T);
-    sv[0][lane] = T;
-    sv[1][lane] = T * d0;
-    sv[2][lane] = T * d1;
-    sv[3][lane] = T * d2;
-    sv[4][lane] = T * (clk + l / (Real)C_LIGHT);
-    sv[5][lane] = T * eps;
-    sv[6][lane] = A;
-    sv[7][lane] = A * eps;
-    sv[8][lane] = w;
-    if (sgs) sv[SH ? 9 : 0][lane] = T * sgc;
+    sv[0][lane] = make_pair2(T, T * d0);
+    sv[1][lane] = make_pair2(T * d1, T * d2);
+    sv[2][lane] = make_pair2(T * (clk + l / (Real)C_LIGHT), T * eps);
+    sv[3][lane] = make_pair2(A, A * eps);
+    sv[4][lane] = make_pair2(w, sgs ? T * sgc : Real(0));
     return bin_fast<Real>(P.Rf + j * 9, P.R + j * 9, P.ax_rc, G, d0, d1, d2);
 }
 
 // A staged free-packet contribution: its values into sv[.][lane], its cone (-1: removed).
 template <typename Real, bool SH>
 __device__ __forceinline__ int staged_contribution(const DevPtrs &P, int s, int nu,
-                                                   Real (*sv)[32], int lane) {
+                                                   Pair<Real> (*sv)[32], int lane) {
     Real *const *V = (Real *const *)P.st_v;
     int bin = P.st_bin[s];
     if (bin >= 0) {
 #pragma unroll
-        for (int f = 0; f < 9; ++f) sv[f][lane] = V[f][s];
-        if (SH && nu == 0) sv[SH ? 9 : 0][lane] = V[9][s];
+        for (int f = 0; f < 4; ++f) sv[f][lane] = make_pair2(V[2 * f][s], V[2 * f + 1][s]);
+        sv[4][lane] = make_pair2(V[8][s], SH && nu == 0 ? V[9][s] : Real(0));
     }
     return bin;
 }
@@ -1584,28 +1579,43 @@ static __device__ __noinline__ void order_segment(const int2 *ent, int *idx, int
 
 // the merged packet of one reception cone: N, N d, N clock, N eps (and N sigma, shared bin)
 template <typename Real, bool SH> struct ConeSum {
-    KSum<Real> N, X, Y, Z, C, E, G;
+    KSum2<Real> NX, YZ, CE;
+    KSum<Real> G;
     __device__ __forceinline__ void zero() {
-        N.init(Real(0)); X.init(Real(0)); Y.init(Real(0)); Z.init(Real(0)); C.init(Real(0));
-        E.init(Real(0)); G.init(Real(0));
+        NX.init(Real(0), Real(0)); YZ.init(Real(0), Real(0)); CE.init(Real(0), Real(0));
+        G.init(Real(0));
     }
-    __device__ __forceinline__ void add(Real (*sv)[32], int t, bool sgs) {
-        N.add(sv[0][t]); X.add(sv[1][t]); Y.add(sv[2][t]); Z.add(sv[3][t]); C.add(sv[4][t]);
-        E.add(sv[5][t]);
-        if (sgs) G.add(sv[SH ? 9 : 0][t]);
+    __device__ __forceinline__ void add(Pair<Real> (*sv)[32], int t, bool sgs) {
+        NX.add(sv[0][t]); YZ.add(sv[1][t]); CE.add(sv[2][t]);
+        if (sgs) G.add(sv[4][t].y);
     }
     // a packet that waited in the cone
     __device__ __forceinline__ void load(const Slots<Real> &S, const Real *SG, long long s,
                                          long long g, bool sgs) {
-        N.init(S.N[s]); X.init(S.X[s]); Y.init(S.Y[s]); Z.init(S.Z[s]); C.init(S.C[s]);
-        E.init(S.E[s]);
+        NX.init(S.N[s], S.X[s]); YZ.init(S.Y[s], S.Z[s]); CE.init(S.C[s], S.E[s]);
         G.init(sgs ? SG[g] : Real(0));
     }
+    __device__ __forceinline__ Real photons() const { return NX.get().x; }
+    __device__ __forceinline__ Real clock() const { return CE.get().x; }
     __device__ __forceinline__ void store(const Slots<Real> &S, Real *SG, long long s, long long g,
                                           bool sgs) const {
-        S.N[s] = N.get(); S.X[s] = X.get(); S.Y[s] = Y.get(); S.Z[s] = Z.get(); S.C[s] = C.get();
-        S.E[s] = E.get();
+        const Pair<Real> a = NX.get(), b = YZ.get(), c = CE.get();
+        S.N[s] = a.x; S.X[s] = a.y; S.Y[s] = b.x; S.Z[s] = b.y; S.C[s] = c.x; S.E[s] = c.y;
         if (sgs) SG[g] = G.get();
+    }
+};
+
+// the absorption sums of a group: A, A eps, w
+template <typename Real> struct AbsSum {
+    KSum2<Real> A;
+    KSum<Real> W;
+    __device__ __forceinline__ void zero() {
+        A.init(Real(0), Real(0));
+        W.init(Real(0));
+    }
+    __device__ __forceinline__ void add(Pair<Real> (*sv)[32], int t) {
+        A.add(sv[3][t]);
+        W.add(sv[4][t].x);
     }
 };
 
@@ -1620,7 +1630,7 @@ __device__ __forceinline__ unsigned byte_popc(unsigned x) {
 // each cone's lane adding its contributions in list order.
 template <typename Real, bool BAR, bool SH>
 __device__ __forceinline__ void wide_group(const DevPtrs &P, int cur, long long key, bool touched,
-                                           int fc, int so, Real (*sv)[32], unsigned *list,
+                                           int fc, int so, Pair<Real> (*sv)[32], unsigned *list,
                                            unsigned *smask, unsigned long long &pend, bool &bad,
                                            int *stot) {
     const int lane = threadIdx.x & 31;
@@ -1633,14 +1643,14 @@ __device__ __forceinline__ void wide_group(const DevPtrs &P, int cur, long long 
     ConeSum<Real, SH> a;
     a.zero();
     if ((park >> lane) & 1u) a.load(Slots<Real>(P, cur), (const Real *)P.slG[cur], sidx, gidx, sgs);
-    KSum<Real> sA, sAE, sW;
-    sA.init(Real(0)); sAE.init(Real(0)); sW.init(Real(0));
+    AbsSum<Real> ab;
+    ab.zero();
     auto merge = [&](int bin) {
         smask[lane] = 0u;
         __syncwarp();
         if (bin >= 0) {
             atomicOr(&smask[bin], 1u << lane);
-            sA.add(sv[6][lane]); sAE.add(sv[7][lane]); sW.add(sv[8][lane]);
+            ab.add(sv, lane);
         }
         __syncwarp();
         unsigned m = smask[lane];
@@ -1686,12 +1696,12 @@ __device__ __forceinline__ void wide_group(const DevPtrs &P, int cur, long long 
             bin = staged_contribution<Real, SH>(P, P.seg_idx[so + cb + lane], nu, sv, lane);
         merge(bin);
     }
-    const Real N = a.N.get();
+    const Real N = a.photons();
     const bool occ = N > Real(0);
-    const bool act = occ && (a.C.get() / N < (Real)P.dt);
+    const bool act = occ && (a.clock() / N < (Real)P.dt);
     const unsigned bo = __ballot_sync(FULLMASK, occ), ba = __ballot_sync(FULLMASK, act);
     if (occ) a.store(Slots<Real>(P, cur ^ 1), (Real *)P.slG[cur ^ 1], sidx, gidx, sgs);
-    Real av = sA.get(), ae = sAE.get(), w = sW.get();
+    Real av = ab.A.get().x, ae = ab.A.get().y, w = ab.W.get();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         av += __shfl_down_sync(FULLMASK, av, o);
@@ -1734,13 +1744,13 @@ __device__ __forceinline__ void wide_group(const DevPtrs &P, int cur, long long 
 // work-list kernel.  cur: the slot buffer holding the hop's packets.
 template <typename Real, int G, bool BAR, bool SH>
 __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int cur, const int *lens) {
-    __shared__ Real svs[8][BVals<SH>::N][32];
+    __shared__ Pair<Real> svs[8][BV_N][32];
     __shared__ unsigned slist[8][32];
     __shared__ unsigned smask[8][2][32];
     __shared__ int snext;
     __shared__ int stot[2];            // the block's packets written, and those able to move
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    Real (*sv)[32] = svs[wid];
+    Pair<Real> (*sv)[32] = svs[wid];
     unsigned *list = slist[wid];
     const int kq = lane >> 3;                  // the lane's group of the four
     const int nxt = cur ^ 1;
@@ -1789,8 +1799,8 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int c
             ConeSum<Real, SH> a;
             a.zero();
             if ((park >> bl) & 1u) a.load(So, (const Real *)P.slG[cur], sidx, gidx, sgs);
-            KSum<Real> sA, sAE, sW;
-            sA.init(Real(0)); sAE.init(Real(0)); sW.init(Real(0));
+            AbsSum<Real> ab;
+            ab.zero();
             // merge the contributions of the lanes: group kk, cone bin (-1: none), and the lane
             // ol of the group's absorption sums
             auto merge = [&](int kk, int bin, int ol) {
@@ -1811,7 +1821,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int c
                 while (m2) {
                     int t = __ffs(m2) - 1;
                     m2 &= m2 - 1u;
-                    sA.add(sv[6][t]); sAE.add(sv[7][t]); sW.add(sv[8][t]);
+                    ab.add(sv, t);
                 }
                 __syncwarp();
             };
@@ -1894,13 +1904,13 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int c
                 merge(kk, bin, c & 7);
             }
             // the merged packets
-            const Real N = a.N.get();
+            const Real N = a.photons();
             const bool occ = kv && N > Real(0);
-            const bool act = occ && (a.C.get() / N < (Real)P.dt);
+            const bool act = occ && (a.clock() / N < (Real)P.dt);
             const unsigned bo = (__ballot_sync(FULLMASK, occ) >> (8 * kq)) & 0xffu;
             const unsigned ba = (__ballot_sync(FULLMASK, act) >> (8 * kq)) & 0xffu;
             if (occ) a.store(Sn, (Real *)P.slG[nxt], sidx, gidx, sgs);
-            Real av = sA.get(), ae = sAE.get(), w = sW.get();
+            Real av = ab.A.get().x, ae = ab.A.get().y, w = ab.W.get();
 #pragma unroll
             for (int o = G >> 1; o > 0; o >>= 1) {
                 av += __shfl_down_sync(FULLMASK, av, o, G);
@@ -2018,21 +2028,21 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int c
                         peers &= peers - 1u;
                         a.add(sv, t, sgs);
                     } while (peers);
-                    const Real N = a.N.get();
+                    const Real N = a.photons();
                     if (N > Real(0)) {
                         a.store(Sn, (Real *)P.slG[nxt], (long long)jk * P.S + (long long)nuk * G + bin,
                                 (long long)jk * G + bin, sgs);
                         atomicOr(&smask[wid][0][kk], 1u << bin);
-                        if (a.C.get() / N < (Real)P.dt) atomicOr(&smask[wid][1][kk], 1u << bin);
+                        if (a.clock() / N < (Real)P.dt) atomicOr(&smask[wid][1][kk], 1u << bin);
                     }
                 }
                 // absorption sums: lane i of a group's adds the i-th contributions of its two
                 // runs of 32 edges and of its staged ones, then a tree over the lanes
-                KSum<Real> sA, sAE, sW;
-                sA.init(Real(0)); sAE.init(Real(0)); sW.init(Real(0));
+                AbsSum<Real> ab;
+                ab.zero();
                 const int i = lane - vk;
                 auto take = [&](bool on, int t) {
-                    if (on && ((live >> t) & 1u)) { sA.add(sv[6][t]); sAE.add(sv[7][t]); sW.add(sv[8][t]); }
+                    if (on && ((live >> t) & 1u)) ab.add(sv, t);
                 };
                 if (myk >= 0) {
                     take(i < m0, (gk + i) & 31);
@@ -2040,7 +2050,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int c
                     take(i < m2, (sk + i) & 31);
                 }
                 const int M = myk >= 0 ? max(max(m0, m1), m2) : 0;
-                Real av = sA.get(), ae = sAE.get(), w = sW.get();
+                Real av = ab.A.get().x, ae = ab.A.get().y, w = ab.W.get();
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) {
                     Real v0 = __shfl_down_sync(FULLMASK, av, o), v1 = __shfl_down_sync(FULLMASK, ae, o),
