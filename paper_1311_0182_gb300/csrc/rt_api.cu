@@ -374,10 +374,7 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     P.rec = dalloc(c, 8 * R * nslot, &ok);
     A(P.bm, unsigned, n * P.kn * P.nf);
     A(P.worklist, int, nkey);
-    A(P.emp, unsigned, nkey);
     A(P.touched, unsigned char, nkey + 4);
-    A(P.reqcnt, int, n + fc);
-    A(P.reqsum, int, n / RT_REQ_CHUNK + fc / RT_REQ_CHUNK + 2);
     A(P.req, unsigned long long, fc);
     for (int b = 0; b < 2; ++b) {
         FreeBuf &F = P.fr[b];
@@ -386,6 +383,7 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
         A(F.nbr, int, fc * P.kn);
         A(F.h2, long long, fc);
         A(F.fid, unsigned long long, fc);
+        A(F.okey, unsigned long long, fc);
         F.N = dalloc(c, R * fc, &ok); F.dx = dalloc(c, R * fc, &ok);
         F.dy = dalloc(c, R * fc, &ok); F.dz = dalloc(c, R * fc, &ok);
         F.clock = dalloc(c, R * fc, &ok); F.eps = dalloc(c, R * fc, &ok);
@@ -393,7 +391,7 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     }
     A(P.st_key, int, P.ST_cap);
     A(P.st_bin, int, P.ST_cap);
-    A(P.st_ord, int, P.ST_cap);
+    A(P.st_ord, unsigned long long, P.ST_cap);
     A(P.st_rank, int, P.ST_cap);
     for (int f = 0; f < 9; ++f) P.st_v[f] = dalloc(c, R * P.ST_cap, &ok);
     if (P.shared) P.st_v[9] = dalloc(c, R * P.ST_cap, &ok);
@@ -401,7 +399,7 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     A(P.seg_cnt, int, segn);
     A(P.seg_off, int, segn);
     A(P.seg_fill, int, segn);
-    A(P.seg_ent, int2, P.ST_cap);
+    A(P.seg_ent, ulonglong2, P.ST_cap);
     A(P.seg_idx, int, P.ST_cap);
     A(P.abs, double, nkey); A(P.absE, double, nkey); A(P.pass, double, nkey);
     A(P.passf, float, nkey);

@@ -22,7 +22,11 @@
 #define RT_OCC_MIN 1           // finest kNN grid the occupancy search tries
 #define RT_MAXK 32            // maximum neighbours per particle
 #define RT_FREE_BIT (1ull << 63)
-#define RT_REQ_CHUNK 1024      // particles (or free packets) of one partial sum of the requests
+// Order of the free packets: generations since the packet was held by a gas particle (or
+// emitted), above the slot it left (or its place among the emitted ones).  Packets made by gas
+// particles come before those made by free packets, each in the order of what they came from;
+// their places in the buffers are arbitrary.
+#define RT_OKEY_GEN (1ull << 40)
 #define RT_SCAN_NB 608         // blocks of every prefix-sum launch (4 per SM)
 
 // error bits of the sticky device error word
@@ -74,6 +78,7 @@ struct FreeBuf {  // packets not held by gas particles: source packets and virtu
     int *nbr;                 // [cap * kn]
     long long *h2;
     unsigned long long *fid;
+    unsigned long long *okey; // order among the hop's free packets
     void *N, *dx, *dy, *dz, *clock, *eps;  // Real [cap]
     void *sig;                // Real [cap]: cross-section of the photons in units of sunit
                               // (shared frequency bin only, else null)
@@ -200,22 +205,19 @@ struct DevPtrs {              // plain pointers handed to kernels (by value)
     // and transposed cone bitmaps
     void *rec;
     unsigned *bm;             // receiver-ordered cone bitmaps [nu * n * kn + p], p = reverse position
-    unsigned *emp;            // empty-cone bits [n * nf]
     unsigned char *touched;   // per (j, nu): 1 when a gas sender wrote a bitmap word this hop
     // requests
-    int *reqcnt;              // [n + F_cap] requests of each particle and free packet
-    int *reqsum;              // and of each RT_REQ_CHUNK of them (particles, then free packets)
-    unsigned long long *req;  // [F_cap]
+    unsigned long long *req;  // [F_cap], in arbitrary order
     FreeBuf fr[2];
     // staged free-packet contributions
     int *st_key;              // receiver key j*nf+nu
-    int *st_ord;              // ordering key: the packet f (one contribution a receiver)
+    unsigned long long *st_ord;  // the packet's order (one contribution a receiver)
     int *st_rank;             // place among the receiver's contributions, in arrival order
     int *st_bin;
     void *st_v[10];           // T, T dx, T dy, T dz, T clock, T eps, A, A eps, w, T sigma (Real;
                               // the last with a shared bin only)
     int *seg_cnt, *seg_off;   // per key: contributions (zero between hops) and first entry
-    int2 *seg_ent;            // (packet, contribution), in arrival order
+    ulonglong2 *seg_ent;      // (order of the packet, contribution), in arrival order
     int *seg_idx;             // contributions in packet order
     int *seg_fill;            // scratch of the neighbour build
     // accumulators

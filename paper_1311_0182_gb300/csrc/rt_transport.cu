@@ -482,6 +482,7 @@ __global__ void k_emit_src(DevPtrs P) {
     if (P.shared) ((Real *)F.sig)[p] = sigma_units<Real>(P, nu);
     F.nu[p] = nu;
     // identity (source, emission, frequency, cone), with the source's identity
+    F.okey[p] = RT_OKEY_GEN | (unsigned long long)p;
     F.fid[p] = (1ull << 62) |
                ((((unsigned long long)P.sid[j] * P.K + k) * P.nfs + nu) * P.nec + e);
 }
@@ -521,6 +522,7 @@ __global__ void k_emit_rec_cones(DevPtrs P, long long base) {
     ((Real *)F.eps)[f] = (Real)(P.epsrec[i] / P.eunit);
     if (P.shared) ((Real *)F.sig)[f] = (Real)(P.sigma_rec / P.sunit);
     F.nu[f] = P.rbin;
+    F.okey[f] = RT_OKEY_GEN | (unsigned long long)f;
     F.fid[f] = (2ull << 62) | ((gi * P.K + k) * P.nec + e);   // (particle, emission, cone)
 }
 
@@ -549,7 +551,9 @@ template <typename Real> struct SentPacket {
 // time (lane = packet: load, direction, clock), then tested one after the other against the
 // neighbours of their particle (lane = neighbour k: cone membership, ballot).  For each
 // (frequency, neighbour) the bits of the packets whose cone holds the neighbour go to the
-// neighbour's receiver-ordered bitmap word; empty cones become virtual-particle requests.
+// neighbour's receiver-ordered bitmap word; empty cones become virtual-particle requests, in no
+// particular order: what depends on an order of the packets they become orders itself (FreeBuf
+// okey).
 // What bounds it: the latency of the dependent gathers and instruction issue; a particle holds
 // few packets able to move (2.5 with 8 cones behind a fast front, 3.8 over 9 frequencies in the
 // HII region), so with a particle of its own most lanes of a warp idled in the packet part
@@ -561,13 +565,15 @@ template <typename Real> struct SentPacket {
 // cur: the slot buffer holding the hop's packets.  Receivers of a bitmap word are flagged in
 // `touched` (cleared again by the work-list kernel).
 // SH: the shared frequency bin (a separate instance keeps its code out of the common case)
+// lens: the hop's counts (the request list is lens[2] long); null: no requests (inspection)
 template <typename Real, int NRC, bool SH>
-__global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int cur, int per) {
+__global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int cur, int per, int *lens) {
     __shared__ unsigned slist[8][32];
-    __shared__ unsigned semp[8][32];
-    __shared__ int snext;
+    __shared__ unsigned sreq[8][64];   // requests not yet in the list
+    __shared__ int snext, scnt[8];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    unsigned *list = slist[wid];
+    unsigned *list = slist[wid], *rq = sreq[wid];
+    int nrq = 0;
     const float cf = 1.0f - 2.0f / (float)P.ntc;
     const long long nrev = P.n * P.kn;
     const unsigned pmask = P.nf < 32 ? (1u << P.nf) - 1u : FULLMASK;   // a particle's words
@@ -581,30 +587,32 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int c
     const long long ib1 = ib0 + chunk < P.n ? ib0 + chunk : P.n;
     if (threadIdx.x == 0) snext = 0;
     __syncthreads();
-    auto next = [&]() {
-        long long v = 0;
-        if (lane == 0) v = ib0 + atomicAdd(&snext, per);
-        return __shfl_sync(FULLMASK, v, 0);
-    };
     const int lp = lane / P.nf, lnu = lane - lp * P.nf;      // the lane's particle and frequency
-    auto words = [&](long long i0) {
-        return (i0 + lp < ib1 && lp < per) ? P.act[cur][(i0 + lp) * P.nf + lnu] : 0u;
+    auto words = [&](long long i) {
+        return (i + lp < ib1 && lp < per) ? P.act[cur][(i + lp) * P.nf + lnu] : 0u;
     };
-    long long i0 = next();
-    unsigned awn = words(i0);                                 // loaded one turn ahead
-    while (i0 < ib1) {
-        const unsigned aw = awn;
-        const long long ic = i0;
-        i0 = next();
-        awn = words(i0);
-        const int np = (int)(ib1 - ic < per ? ib1 - ic : per);
+    // turns a warp takes at once: up to four, whose words it loads together (where nothing moves it
+    // goes on after one load), fewer towards the end of the chunk, so that the warps end together
+    auto at_once = [&](long long left) { return (int)max(1ll, min(4ll, left / (16 * per))); };
+    int turns = at_once(chunk);
+    for (;;) {
+        long long i0 = 0;
+        if (lane == 0) i0 = ib0 + atomicAdd(&snext, per * turns);
+        i0 = __shfl_sync(FULLMASK, i0, 0);
+        if (i0 >= ib1) break;
+        const int now = turns;
+        turns = at_once(ib1 - i0);
+        unsigned w4[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) w4[u] = u < now ? words(i0 + u * per) : 0u;
+        if (__ballot_sync(FULLMASK, (w4[0] | w4[1] | w4[2] | w4[3]) != 0u) == 0u) continue;
+#pragma unroll 1
+        for (int u = 0; u < now; ++u) {
+        const unsigned aw = u < 2 ? (u == 0 ? w4[0] : w4[1]) : (u == 2 ? w4[2] : w4[3]);
+        const long long ic = i0 + u * per;
         const unsigned moving = __ballot_sync(FULLMASK, aw != 0u);
-        if (moving == 0u) {
-            if (lane < np) P.reqcnt[ic + lane] = 0;
-            continue;
-        }
-        nsend += lane < np && ((moving >> (lane * P.nf)) & pmask) != 0u;
-        semp[wid][lane] = 0u;
+        if (moving == 0u) continue;
+        nsend += lane < per && ((moving >> (lane * P.nf)) & pmask) != 0u;
         const unsigned cnt = (unsigned)__popc(aw);
         const unsigned incl = lane_scan(cnt);
         const int total = (int)__shfl_sync(FULLMASK, incl, 31);
@@ -696,28 +704,47 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int c
             }
             ncon += my_cm;
             if (has) {
-                if (my_cm > 0)
+                if (my_cm > 0) {
                     rec_store(P.rec, s, rdiv<Real>(K.N, (Real)my_cm), K.d0, K.d1, K.d2,
                               rdiv<Real>(K.C, K.N), rdiv<Real>(K.E, K.N), sgs, K.sg);
-                else
-                    atomicOr(&semp[wid][row], 1u << ob);
+                }
+            }
+            // packets without a member request a virtual particle
+            const unsigned rm = lens ? __ballot_sync(FULLMASK, has && my_cm == 0) : 0u;
+            if (rm) {
+                if ((rm >> lane) & 1u) rq[nrq + __popc(rm & ((1u << lane) - 1u))] = (unsigned)s;
+                nrq += __popc(rm);
+                __syncwarp();
+                if (nrq >= 32) {
+                    int base = 0;
+                    if (lane == 0) base = atomicAdd(&lens[2], 32);
+                    base = __shfl_sync(FULLMASK, base, 0);
+                    const unsigned v0 = rq[lane], v1 = rq[32 + lane];
+                    if (base + lane < P.F_cap) P.req[base + lane] = v0;
+                    __syncwarp();
+                    nrq -= 32;
+                    if (lane < nrq) rq[lane] = v1;
+                    __syncwarp();
+                }
             }
         }
         // every word starts the hop at zero (the receiver side clears the words it reads), and
         // each (frequency, neighbour) word is written once: a plain store
         flush();
-        __syncwarp();
-        const unsigned em = semp[wid][lane];
-        if (lp < np) P.emp[(ic + lp) * P.nf + lnu] = em;
-        // requests a particle: the sum over its words
-        unsigned r = (unsigned)__popc(em);
-        const unsigned ri = lane_scan(r);
-        const int la = lane * P.nf - 1, lb = min(la + P.nf, 31);   // last lanes of particles lane - 1, lane
-        const unsigned ra = __shfl_sync(FULLMASK, ri, la & 31), rb = __shfl_sync(FULLMASK, ri, lb & 31);
-        const int nr = lane < np ? (int)(rb - (lane ? ra : 0u)) : 0;
-        if (lane < np) P.reqcnt[ic + lane] = nr;
-        if (nr) atomicAdd(&P.reqsum[(ic + lane) / RT_REQ_CHUNK], nr);
-        __syncwarp();
+        }
+    }
+    if (lens) {   // what is left of the block's requests, in one piece
+        if (lane == 0) scnt[wid] = nrq;
+        __syncthreads();
+        int before = 0, all = 0;
+        for (int k = 0; k < 8; ++k) {
+            if (k < wid) before += scnt[k];
+            all += scnt[k];
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && all) snext = atomicAdd(&lens[2], all);
+        __syncthreads();
+        if (lane < nrq && snext + before + lane < P.F_cap) P.req[snext + before + lane] = rq[lane];
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ncon += __shfl_down_sync(FULLMASK, ncon, o);
@@ -734,7 +761,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int c
 // collects the members of their cones in a list.  32 members at a time (lane = member) become
 // staged contributions, at a position from one counter: a packet has about one member, so a
 // warp of its own computed one contribution with one lane.  The position is arbitrary; a
-// contribution carries its packet (st_ord), by which the receiver orders its segment, and its
+// contribution carries its packet's order (st_ord), by which the receiver orders its segment, and its
 // place among the receiver's (st_rank, the count before it).  A packet without a member
 // requests a virtual particle.  Measured per step against two kernels and a prefix sum with a
 // warp a packet: 64^3 HII region 7.4 -> 3.6 ms, the FP64 path at 32^3 4.7 -> 1.8 ms.
@@ -753,7 +780,6 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_free(DevPtrs P, int fcu
     while (per < 32 && 2 * per * nw <= nfree) per *= 2;
     const FreeBuf F = P.fr[fcur];
     const float cf = 1.0f - 2.0f / (float)P.ntc;
-    const long long C0 = (P.n + RT_REQ_CHUNK - 1) / RT_REQ_CHUNK;
     int nlist = 0;
     // stage the first `cnt` members of the list
     auto stage = [&](int cnt) {
@@ -779,7 +805,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_free(DevPtrs P, int fcu
             const long long key = j * P.nf + nu;
             Real **V = (Real **)P.st_v;
             P.st_key[s] = (int)key;
-            P.st_ord[s] = (int)f;
+            P.st_ord[s] = F.okey[f];
             int bt = -1;
             if (BAR && barrier_crosses_call(P.bar[q.w], fx, fy, fz, q.x, q.y, q.z)) {
                 // the share crosses the barrier: removed (counted escaped); the staged
@@ -876,90 +902,15 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_free(DevPtrs P, int fcu
                 __syncwarp();
             }
         }
-        if (on) P.reqcnt[P.n + f] = req ? 1 : 0;
-        const int nr = __popc(__ballot_sync(FULLMASK, req));
-        if (lane == 0 && nr) atomicAdd(&P.reqsum[C0 + f0 / RT_REQ_CHUNK], nr);
+        const unsigned rm = __ballot_sync(FULLMASK, req);
+        if (rm) {
+            int base = 0;
+            if (lane == 0) base = atomicAdd(&lens[2], __popc(rm));
+            base = __shfl_sync(FULLMASK, base, 0) + __popc(rm & ((1u << lane) - 1u));
+            if (req && base < P.F_cap) P.req[base] = RT_FREE_BIT | (unsigned long long)f;
+        }
     }
     if (nlist) stage(nlist);
-}
-
-// The request list in its fixed order: gas slots with empty cones (particle order, slot order),
-// then free packets.  The senders have added the requests of every RT_REQ_CHUNK particles (or
-// free packets) to reqsum; a block takes a chunk with any, sums the chunks before it, scans its
-// own counts and writes its requests: one pass and one launch, nothing but reqsum read where
-// there are no requests.  The first block also books the hop's request count and checks the
-// capacities.
-__global__ void __launch_bounds__(256) k_requests(DevPtrs P, int *lens) {
-    __shared__ int sh[33];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const long long nfree = lens[0];
-    const int C0 = (int)((P.n + RT_REQ_CHUNK - 1) / RT_REQ_CHUNK);
-    const int C = C0 + (int)((nfree + RT_REQ_CHUNK - 1) / RT_REQ_CHUNK);
-    // sum over the block's threads
-    auto block_total = [&](int v) {
-        v = __reduce_add_sync(FULLMASK, v);
-        if (lane == 0) sh[wid] = v;
-        __syncthreads();
-        int t = 0;
-        for (int k = 0; k < 8; ++k) t += sh[k];
-        __syncthreads();
-        return t;
-    };
-    if (blockIdx.x == 0) {
-        int v = 0;
-        for (int k = tid; k < C; k += 256) v += P.reqsum[k];
-        const long long nr = block_total(v);
-        if (tid == 0) {
-            long long *cnt = P.cnt;
-            if (nr > P.F_cap)
-                atomicOr((unsigned long long *)&cnt[CNT_ERR], (unsigned long long)ERRB_FREE_CAP);
-            lens[2] = (int)nr;
-            cnt[CNT_NREQ] = nr;
-            cnt[CNT_VIRT] += nr < P.F_cap ? nr : P.F_cap;
-        }
-    }
-    for (int c = blockIdx.x; c < C; c += gridDim.x) {
-        if (P.reqsum[c] == 0) continue;
-        int v = 0;
-        for (int k = tid; k < c; k += 256) v += P.reqsum[k];
-        const int before = block_total(v);
-        // four consecutive items a thread
-        const bool gas = c < C0;
-        const long long i0 = (gas ? (long long)c : (long long)(c - C0)) * RT_REQ_CHUNK + 4 * tid;
-        const long long lim = gas ? P.n : nfree;
-        const int *rc = P.reqcnt + (gas ? 0 : P.n);
-        int rq[4], own = 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            rq[k] = i0 + k < lim ? rc[i0 + k] : 0;
-            own += rq[k];
-        }
-        const int incl = (int)lane_scan((unsigned)own);
-        if (lane == 31) sh[wid] = incl;
-        __syncthreads();
-        long long o = before + incl - own;
-        for (int k = 0; k < wid; ++k) o += sh[k];
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if (!rq[k]) continue;
-            const long long t = i0 + k;
-            if (gas) {
-                for (int nu = 0; nu < P.nf; ++nu) {
-                    unsigned e = P.emp[t * P.nf + nu];
-                    while (e) {
-                        int b = __ffs(e) - 1;
-                        e &= e - 1u;
-                        if (o < P.F_cap) P.req[o] = (unsigned long long)(t * P.S + (long long)nu * P.nrc + b);
-                        ++o;
-                    }
-                }
-            } else {
-                if (o < P.F_cap) P.req[o] = RT_FREE_BIT | (unsigned long long)t;
-                ++o;
-            }
-        }
-    }
 }
 
 // No accepted draw: the point on the packet's axis at h/2 (at least one quantum), rounded to
@@ -985,7 +936,7 @@ __device__ __forceinline__ void axis_offset(float d0, float d1, float d2, long l
 // and the per-box and per-frequency values the request needs.
 template <typename Real> struct VDec {
     long long h2, boff;
-    unsigned long long fid;
+    unsigned long long fid, okey;
     Real N, d0, d1, d2, clk, eps, sg, sig, bu;
     float f0, f1, f2, h2f;        // the direction and the smoothing length squared in FP32
     int box, qx, qy, qz, nu, H;
@@ -1119,6 +1070,7 @@ __global__ void __launch_bounds__(256, VIRT_MINB(Real)) k_virtual(DevPtrs P, int
                 D.clk = S.C[code] / D.N;
                 D.eps = S.E[code] / D.N;
                 if (SH && D.nu == 0) D.sg = ((Real *)P.slG[cur])[i * NRC + s] / D.N;
+                D.okey = RT_OKEY_GEN | code;
                 D.fid = gid_of(P, i, D.box) * P.S + (code - (unsigned long long)i * P.S) + 1ull;
             } else {
                 long long f = (long long)(code & ~RT_FREE_BIT);
@@ -1130,6 +1082,7 @@ __global__ void __launch_bounds__(256, VIRT_MINB(Real)) k_virtual(DevPtrs P, int
                 D.eps = ((Real *)Fi.eps)[f];
                 D.nu = Fi.nu[f];
                 if (SH && D.nu == 0) D.sg = ((Real *)Fi.sig)[f];
+                D.okey = Fi.okey[f] + RT_OKEY_GEN;
                 D.fid = Fi.fid[f];
             }
             D.boff = P.box_off[D.box];
@@ -1351,6 +1304,7 @@ __global__ void __launch_bounds__(256, VIRT_MINB(Real)) k_virtual(DevPtrs P, int
             ((Real *)Fo.eps)[r] = D.eps;
             if (SH && D.nu == 0) ((Real *)Fo.sig)[r] = D.sg;
             Fo.nu[r] = D.nu;
+            Fo.okey[r] = D.okey;
             Fo.fid[r] = mix64(D.fid);
         }
         const int non = __popc(__ballot_sync(FULLMASK, on));
@@ -1466,7 +1420,7 @@ __global__ void __launch_bounds__(256) k_seg_fill(DevPtrs P, const int *lens) {
     if (nst > P.ST_cap) nst = P.ST_cap;
     for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < nst;
          s += (long long)gridDim.x * blockDim.x)
-        P.seg_ent[P.seg_off[P.st_key[s]] + P.st_rank[s]] = make_int2(P.st_ord[s], (int)s);
+        P.seg_ent[P.seg_off[P.st_key[s]] + P.st_rank[s]] = make_ulonglong2(P.st_ord[s], (unsigned long long)s);
 }
 
 // absorptions of one receiver group in one hop.  FP64 path: FP64 sums.  FP32 path: the
@@ -1565,14 +1519,14 @@ __device__ __forceinline__ int staged_contribution(const DevPtrs &P, int s, int 
 }
 
 // A segment of n staged contributions in packet order, by eight lanes: each takes the place
-// given by the number of smaller packets (distinct).  Out of line: few groups have any, and
+// given by the number of earlier packets (distinct).  Out of line: few groups have any, and
 // inlined it costs the receiver side registers.
-static __device__ __noinline__ void order_segment(const int2 *ent, int *idx, int n) {
+static __device__ __noinline__ void order_segment(const ulonglong2 *ent, int *idx, int n) {
     for (int c = threadIdx.x & 7; c < n; c += 8) {
-        const int2 e = ent[c];
+        const ulonglong2 e = ent[c];
         int r = 0;
         for (int k = 0; k < n; ++k) r += ent[k].x < e.x;
-        idx[r] = e.y;
+        idx[r] = (int)e.y;
     }
     __syncwarp();
 }
@@ -2086,27 +2040,24 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int c
     }
 }
 
-// bookkeeping of the hop loop (one block)
+// bookkeeping of the hop loop (single thread)
 enum { HL_END = 2, HL_TRANSPORT = 4, HL_STEP = 5 };
 // in_graph: the launch is a node of the step graph; `loop` is the hop loop's conditional and
 // `pair` the switch that picks the copy of the next hop (its slot and free-packet buffers)
-__global__ void __launch_bounds__(256) k_hop_lens(DevPtrs P, int *lens, int phase, long long arg,
-                                                  int in_graph, cudaGraphConditionalHandle loop,
-                                                  cudaGraphConditionalHandle pair) {
+__global__ void k_hop_lens(DevPtrs P, int *lens, int phase, long long arg, int in_graph,
+                           cudaGraphConditionalHandle loop, cudaGraphConditionalHandle pair) {
     long long *cnt = P.cnt;
     if (phase == HL_STEP) {             // the step number (arg)
-        if (threadIdx.x == 0) cnt[CNT_STEP] = arg;
+        cnt[CNT_STEP] = arg;
         return;
     }
-    // the chunk sums of the requests back to zero: those of this hop, or all before the first
-    const long long nfree = phase == HL_TRANSPORT ? P.F_cap : (long long)lens[0];
-    const long long C = (P.n + RT_REQ_CHUNK - 1) / RT_REQ_CHUNK + (nfree + RT_REQ_CHUNK - 1) / RT_REQ_CHUNK;
-    for (long long k = threadIdx.x; k < C; k += blockDim.x) P.reqsum[k] = 0;
-    __syncthreads();
-    if (threadIdx.x != 0) return;
     if (phase == HL_END) {              // after the hop (arg = hop cap)
         long long nr = lens[2];
+        if (nr > P.F_cap) cnt[CNT_ERR] |= ERRB_FREE_CAP;
+        if (lens[3] > P.ST_cap) cnt[CNT_ERR] |= ERRB_STAGE_CAP;
+        cnt[CNT_NREQ] = nr;
         lens[0] = (int)(nr < P.F_cap ? nr : P.F_cap);
+        cnt[CNT_VIRT] += lens[0];
         cnt[CNT_STG] += lens[3];
         cnt[CNT_WLS] += lens[4];
         if (nr > cnt[CNT_PKFREE]) cnt[CNT_PKFREE] = nr;
@@ -2184,7 +2135,7 @@ __global__ void k_drop_free(DevPtrs P, const int *lens) {
 // the step number the rotations and virtual particles draw with (kept on the device)
 static void set_step(rt_ctx *c, long long step, cudaStream_t st) {
     if (c->step_dev == step && step != LLONG_MIN) return;
-    LAUNCH(KT_HOP_LENS, 1, (k_hop_lens<<<1, 256, 0, st>>>(c->d, c->hop.lens, HL_STEP, step, 0, 0, 0)));
+    LAUNCH(KT_HOP_LENS, 1, (k_hop_lens<<<1, 1, 0, st>>>(c->d, c->hop.lens, HL_STEP, step, 0, 0, 0)));
     c->step_dev = step;
 }
 
@@ -2196,15 +2147,15 @@ static int send_turn(const DevPtrs &P) {
     return (int)std::min(most, std::max(1ll, P.n / (152 * 32)));
 }
 
-// One hop, in seven launches and a bookkeeping kernel (k_hop_lens HL_END, launched by the
+// One hop, in six launches and a bookkeeping kernel (k_hop_lens HL_END, launched by the
 // caller), with no pass over a capacity.  Two streams:
-//   st: gas senders; request list (after both senders); virtual particles
+//   st: gas senders; virtual particles (after both senders)
 //   s2: free-packet senders; work list (after both senders); segments; receiver side
 // The caller's stream continues after the receiver side.  What a small box costs is its
 // chain of dependent launches: 5 here (senders, work list, segments, receiver side,
 // bookkeeping), where the hop was 20 launches with a chain of 15 before: the 12^3 sphere's step
-// of 10 hops went from 0.90 to 0.51 ms, that of a 64^3 box with hardly any packets and 39 hops
-// from 6.1 to 3.5 ms.
+// of 10 hops went from 0.90 to 0.50 ms, that of a 64^3 box with hardly any packets and 39 hops
+// from 6.1 to 3.4 ms.
 // nfr bounds the free packets of the hop (their count is on the device); cur and fcur are the
 // hop's slot and free-packet buffers.
 template <typename Real, int NRC>
@@ -2234,15 +2185,14 @@ static void hop_core(rt_ctx *c, cudaStream_t st, long long nfr, int cur, int fcu
     cudaEventRecord(evFree, s2);
     const int nba = rt_blocks((n + per - 1) / per * 32, tb, GA);
     if (P.shared)
-        LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, true><<<nba, tb, 0, st>>>(P, cur, per)));
+        LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, true><<<nba, tb, 0, st>>>(P, cur, per, H.lens)));
     else
-        LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, false><<<nba, tb, 0, st>>>(P, cur, per)));
+        LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, false><<<nba, tb, 0, st>>>(P, cur, per, H.lens)));
     cudaEventRecord(evA, st);
     cudaStreamWaitEvent(s2, evA, 0);
     LAUNCH_ON(s2, KT_WORKLIST, 1, (k_worklist<<<rt_blocks(nkey, 1024, 152 * 8), tb, 0, s2>>>(P, cur, H.lens)));
     LAUNCH_ON(s2, KT_SEG_FILL, 1, (k_seg_fill<<<rt_blocks(nfr * 2, tb, 152 * 8), tb, 0, s2>>>(P, H.lens)));
     cudaStreamWaitEvent(st, evFree, 0);
-    LAUNCH(KT_EXPAND, 1, (k_requests<<<rt_blocks(n + nfr, RT_REQ_CHUNK, 152 * 8), tb, 0, st>>>(P, H.lens)));
     const int nbb = rt_blocks(nkey * 8, tb, GB);
     if (P.shared)
         LAUNCH_ON(s2, KT_PHASE_B, 1, (k_phaseB<Real, NRC, true, true><<<nbb, tb, 0, s2>>>(P, cur, H.lens)));
@@ -2286,7 +2236,7 @@ static void transport_begin(rt_ctx *c, cudaStream_t st) {
         clear_cone_bits(c, st);
         c->bm_dirty = false;
     }
-    LAUNCH(KT_HOP_LENS, 1, (k_hop_lens<<<1, 256, 0, st>>>(P, c->hop.lens, HL_TRANSPORT, c->cfg.hop_cap, 0, 0, 0)));
+    LAUNCH(KT_HOP_LENS, 1, (k_hop_lens<<<1, 1, 0, st>>>(P, c->hop.lens, HL_TRANSPORT, c->cfg.hop_cap, 0, 0, 0)));
 }
 
 // after the hop loop (the counters are in cnt_h): statistics, modelled bytes, status
@@ -2367,9 +2317,9 @@ static rt_status run_parts(rt_ctx *c, int part, long long step, cudaStream_t st)
         c->bm_dirty = true;
         const int per = send_turn(P);
         if (P.shared)
-            LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, true><<<rt_blocks((n + per - 1) / per * 32, tb, 152 * 64), tb, 0, st>>>(P, c->cur, per)));
+            LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, true><<<rt_blocks((n + per - 1) / per * 32, tb, 152 * 64), tb, 0, st>>>(P, c->cur, per, nullptr)));
         else
-            LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, false><<<rt_blocks((n + per - 1) / per * 32, tb, 152 * 64), tb, 0, st>>>(P, c->cur, per)));
+            LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, false><<<rt_blocks((n + per - 1) / per * 32, tb, 152 * 64), tb, 0, st>>>(P, c->cur, per, nullptr)));
         return rt_cuda_check(c, cudaGetLastError(), "cone masks");
     }
     // part 4: the hop loop, driven from the host (one synchronisation per hop)
@@ -2377,7 +2327,7 @@ static rt_status run_parts(rt_ctx *c, int part, long long step, cudaStream_t st)
     transport_begin(c, st);
     for (;;) {
         hop_core<Real, NRC>(c, st, c->nfree_h, c->cur, c->fcur);
-        LAUNCH(KT_HOP_LENS, 1, (k_hop_lens<<<1, 256, 0, st>>>(P, H.lens, HL_END, c->cfg.hop_cap, 0, 0, 0)));
+        LAUNCH(KT_HOP_LENS, 1, (k_hop_lens<<<1, 1, 0, st>>>(P, H.lens, HL_END, c->cfg.hop_cap, 0, 0, 0)));
         c->cur ^= 1;
         c->fcur ^= 1;
         cudaMemcpyAsync(c->cnt_h, P.cnt, sizeof(long long) * CNT_N, cudaMemcpyDeviceToHost, st);
@@ -2439,7 +2389,7 @@ static rt_status seg_prologue(rt_ctx *c, cudaStream_t st) {
     if ((s = run_parts<Real, NRC>(c, 0, 0, st))) return s;
     if ((s = run_parts<Real, NRC>(c, 1, 0, st))) return s;
     if ((s = run_parts<Real, NRC>(c, 2, 0, st))) return s;
-    LAUNCH(KT_HOP_LENS, 1, (k_hop_lens<<<1, 256, 0, st>>>(c->d, c->hop.lens, HL_TRANSPORT, c->cfg.hop_cap, 1, c->loop_h, c->pair_h)));
+    LAUNCH(KT_HOP_LENS, 1, (k_hop_lens<<<1, 1, 0, st>>>(c->d, c->hop.lens, HL_TRANSPORT, c->cfg.hop_cap, 1, c->loop_h, c->pair_h)));
     cudaStreamWaitEvent(st, c->hev[1], 0);
     return rt_cuda_check(c, cudaGetLastError(), "graph prologue");
 }
@@ -2488,7 +2438,7 @@ static cudaError_t build_hop_body(rt_ctx *c, cudaGraph_t body) {
         cudaKernelNodeParams kp = {};
         kp.func = (void *)k_hop_lens;
         kp.gridDim = dim3(1);
-        kp.blockDim = dim3(256);
+        kp.blockDim = dim3(1);
         kp.kernelParams = args;
         c->graph_launch_hop[KT_HOP_LENS] += 1;
         e = cudaGraphAddKernelNode(&nend, body, &nsw, 1, &kp);
