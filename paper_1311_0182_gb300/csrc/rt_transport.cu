@@ -216,13 +216,29 @@ __device__ __forceinline__ void rec_load(const void *rec, long long s, double &w
     if (sg) sig = p[3].x;
 }
 
+// Quotients with a shared divisor, correctly rounded like a division each (div_by_rcp): an FP64
+// division takes about ten FP64 instructions, a further quotient by the same divisor three.  The
+// plain division where an operand is so large or small that the exact remainder could leave
+// the range.
+__device__ __forceinline__ bool in_range(double a) {   // 2^-400 <= |a| < 2^401
+    return (((unsigned)__double2hiint(a) >> 20) & 0x7ffu) - 623u < 801u;
+}
+__device__ __forceinline__ double quot(double a, double b, double y) {   // y = 1 / b, rounded
+    bool zero = (__double_as_longlong(a) << 1) == 0ll;
+    return (in_range(a) || zero) && in_range(b) ? div_by_rcp(a, b, y) : a / b;
+}
+
 // unit direction of a packet from its summed momentum M (the luminosity-weighted mean
 // direction of merged packets, Sec. 2.1, Fig. 1b)
 __device__ __forceinline__ void packet_dir(double Mx, double My, double Mz, double &d0, double &d1,
                                            double &d2) {
     double nn = sqrt(Mx * Mx + My * My + Mz * Mz);
-    if (nn > 0.0) { d0 = Mx / nn; d1 = My / nn; d2 = Mz / nn; }
-    else { d0 = 1.0; d1 = 0.0; d2 = 0.0; }
+    if (nn > 0.0) {
+        double y = __drcp_rn(nn);
+        d0 = quot(Mx, nn, y); d1 = quot(My, nn, y); d2 = quot(Mz, nn, y);
+    } else {
+        d0 = 1.0; d1 = 0.0; d2 = 0.0;
+    }
 }
 
 // FP32: normalised photon counts can be small enough for |M|^2 to underflow, so scale first.
@@ -249,6 +265,34 @@ __device__ __forceinline__ void packet_dir(float Mx, float My, float Mz, float &
 template <typename Real> __device__ __forceinline__ Real rdiv(Real a, Real b);
 template <> __device__ __forceinline__ double rdiv<double>(double a, double b) { return a / b; }
 template <> __device__ __forceinline__ float rdiv<float>(float a, float b) { return a * __frcp_rn(b); }
+
+// mean clock and energy of a packet: C / N and E / N (rdiv's arithmetic)
+__device__ __forceinline__ void means(double C, double E, double N, double &c, double &e) {
+    double y = __drcp_rn(N);
+    c = quot(C, N, y);
+    e = quot(E, N, y);
+}
+__device__ __forceinline__ void means(float C, float E, float N, float &c, float &e) {
+    float y = __frcp_rn(N);
+    c = C * y;
+    e = E * y;
+}
+// the same as IEEE quotients in both precisions
+__device__ __forceinline__ void ratios(double C, double E, double N, double &c, double &e) {
+    means(C, E, N, c, e);
+}
+__device__ __forceinline__ void ratios(float C, float E, float N, float &c, float &e) {
+    c = C / N;
+    e = E / N;
+}
+// l / c: the time a packet takes for the length l
+__device__ __forceinline__ double light_time(double l) { return quot(l, C_LIGHT, 1.0 / C_LIGHT); }
+__device__ __forceinline__ float light_time(float l) {
+    const float c = (float)C_LIGHT, y = 1.0f / c;
+    if (!(fabsf(l) > 1e-15f)) return l / c;
+    float q = __fmul_rn(l, y);
+    return __fmaf_rn(__fmaf_rn(-q, c, l), y, q);
+}
 
 // precision-matched constants: FP64 values on the FP64 path, FP32 copies on the FP32 path
 template <typename Real> __device__ __forceinline__ Real box_unit(const DevPtrs &P, int b);
@@ -705,8 +749,9 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int c
             ncon += my_cm;
             if (has) {
                 if (my_cm > 0) {
-                    rec_store(P.rec, s, rdiv<Real>(K.N, (Real)my_cm), K.d0, K.d1, K.d2,
-                              rdiv<Real>(K.C, K.N), rdiv<Real>(K.E, K.N), sgs, K.sg);
+                    Real c, e;
+                    means(K.C, K.E, K.N, c, e);
+                    rec_store(P.rec, s, rdiv<Real>(K.N, (Real)my_cm), K.d0, K.d1, K.d2, c, e, sgs, K.sg);
                 }
             }
             // packets without a member request a virtual particle
@@ -823,7 +868,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_free(DevPtrs P, int fcu
                 V[1][s] = T * d0;
                 V[2][s] = T * d1;
                 V[3][s] = T * d2;
-                V[4][s] = T * (clk + l / (Real)C_LIGHT);
+                V[4][s] = T * (clk + light_time(l));
                 V[5][s] = T * eps;
                 V[6][s] = A;
                 V[7][s] = A * eps;
@@ -1067,8 +1112,7 @@ __global__ void __launch_bounds__(256, VIRT_MINB(Real)) k_virtual(DevPtrs P, int
                 D.h2 = P.h2[i];
                 D.N = S.N[code];
                 packet_dir(S.X[code], S.Y[code], S.Z[code], D.d0, D.d1, D.d2);
-                D.clk = S.C[code] / D.N;
-                D.eps = S.E[code] / D.N;
+                ratios(S.C[code], S.E[code], D.N, D.clk, D.eps);
                 if (SH && D.nu == 0) D.sg = ((Real *)P.slG[cur])[i * NRC + s] / D.N;
                 D.okey = RT_OKEY_GEN | code;
                 D.fid = gid_of(P, i, D.box) * P.S + (code - (unsigned long long)i * P.S) + 1ull;
@@ -1300,7 +1344,7 @@ __global__ void __launch_bounds__(256, VIRT_MINB(Real)) k_virtual(DevPtrs P, int
             Fo.h2[r] = mh2v;
             ((Real *)Fo.N)[r] = T;
             ((Real *)Fo.dx)[r] = D.d0; ((Real *)Fo.dy)[r] = D.d1; ((Real *)Fo.dz)[r] = D.d2;
-            ((Real *)Fo.clock)[r] = D.clk + l / (Real)C_LIGHT;
+            ((Real *)Fo.clock)[r] = D.clk + light_time(l);
             ((Real *)Fo.eps)[r] = D.eps;
             if (SH && D.nu == 0) ((Real *)Fo.sig)[r] = D.sg;
             Fo.nu[r] = D.nu;
@@ -1498,7 +1542,7 @@ __device__ __forceinline__ int gas_contribution(const DevPtrs &P, long long e, i
     split_absorbed<Real>(w, sn * l, A, T);
     sv[0][lane] = make_pair2(T, T * d0);
     sv[1][lane] = make_pair2(T * d1, T * d2);
-    sv[2][lane] = make_pair2(T * (clk + l / (Real)C_LIGHT), T * eps);
+    sv[2][lane] = make_pair2(T * (clk + light_time(l)), T * eps);
     sv[3][lane] = make_pair2(A, A * eps);
     sv[4][lane] = make_pair2(w, sgs ? T * sgc : Real(0));
     return bin_fast<Real>(P.Rf + j * 9, P.R + j * 9, P.ax_rc, G, d0, d1, d2);
@@ -2140,11 +2184,13 @@ static void set_step(rt_ctx *c, long long step, cudaStream_t st) {
 }
 
 // Particles a warp of the sender side takes together: as many as its 32 (particle, frequency)
-// words hold, but no more than leave every resident warp (152 SMs x 32) a turn, since a small
-// box needs its particles spread over the chip more than it needs full lanes.
+// words hold, but no more than leave the resident warps a turn each, since a small box needs its
+// particles spread over the chip more than it needs full lanes: 32 warps an SM with FP32
+// packets; 8 with FP64 packets, where a few warps already fill the FP64 pipe and fuller lanes
+// mean fewer of its instructions (the 16^3 sphere's step: 1.79 ms with 32, 1.67 with 8, 1.73 with 4).
 static int send_turn(const DevPtrs &P) {
     long long most = std::max(1, 32 / P.nf);
-    return (int)std::min(most, std::max(1ll, P.n / (152 * 32)));
+    return (int)std::min(most, std::max(1ll, P.n / (152 * (P.fp32 ? 32 : 8))));
 }
 
 // One hop, in six launches and a bookkeeping kernel (k_hop_lens HL_END, launched by the
