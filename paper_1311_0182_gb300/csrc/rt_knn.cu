@@ -252,9 +252,8 @@ __device__ __forceinline__ int cell_box(const DevPtrs &P, long long c) {
 // cell: a cell at offset o >= 2 is at least (o - 1) cs + 1 from it
 __device__ __forceinline__ int cand_radius(long long u2, int cs, int G) {
     if (u2 >= KNN_INF) return G;
-    long long u = (long long)sqrt((double)u2) + 1;
-    long long r = u / cs + 1;
-    return r < G ? (int)r : G;
+    int r = (int)sqrt_up(u2) / cs + 1;   // u2 < 3 * 2^40
+    return r < G ? r : G;
 }
 
 // Calls f(position of the item among the box's items, item) for every particle of box b whose
@@ -263,7 +262,8 @@ __device__ __forceinline__ int cand_radius(long long u2, int cs, int G) {
 // items); the lanes' ranges are then walked together, 32 items at a time, so that a warp reads
 // whole lines and a column of a dense clump does not hold up its lane: with a column a lane the
 // slowest cells of a clump took 13.4 ms of a 300,000-particle build (k_cand_fill), 6.4 ms with
-// the lanes together, and 1.6 ms with the rings in 32-bit arithmetic as well.
+// the lanes together, 1.6 ms with the rings in 32-bit arithmetic as well, and 1.4 ms with the
+// distance test in FP32 (guard band of 1e-6, about five roundings; the exact test inside it).
 template <typename F>
 __device__ __forceinline__ void cand_walk(const DevPtrs &P, int b, int cx, int cy, int cz,
                                           long long u2, F f) {
@@ -274,6 +274,9 @@ __device__ __forceinline__ void cand_walk(const DevPtrs &P, int b, int cx, int c
     int R = cand_radius(u2, cs, G);
     int lx = cx * cs, ly = cy * cs, lz = cz * cs;
     int hx = lx + cs - 1, hy = ly + cs - 1, hz = lz + cs - 1;
+    const float flx = (float)lx, fly = (float)ly, flz = (float)lz, fhx = (float)hx, fhy = (float)hy,
+                fhz = (float)hz;                    // below 2^21: exact
+    const float ulo = (float)u2 * 0.999999f, uhi = (float)u2 * 1.000001f;
     int side = 2 * R + 1;
     long long ncol = (long long)side * side;
     for (long long cb = 0; cb < ncol; cb += 32) {
@@ -311,8 +314,15 @@ __device__ __forceinline__ void cand_walk(const DevPtrs &P, int b, int cx, int c
                 if (__shfl_sync(FULLMASK, incl, own + o - 1) <= c) own += o;
             const int pos = __shfl_sync(FULLMASK, first, own & 31) + c;
             if (c < total) {
-                int4 it = P.grid.items[pos];
-                if (box_d2(it.x, it.y, it.z, lx, ly, lz, hx, hy, hz) <= u2) f(pos - ibase, it);
+                const float4 it = __ldg(P.grid.fitems + pos);
+                const float gx = fmaxf(fmaxf(flx - it.x, it.x - fhx), 0.0f),
+                            gy = fmaxf(fmaxf(fly - it.y, it.y - fhy), 0.0f),
+                            gz = fmaxf(fmaxf(flz - it.z, it.z - fhz), 0.0f);
+                const float d = __fmaf_rn(gx, gx, __fmaf_rn(gy, gy, gz * gz));
+                bool in = d < ulo;
+                if (!in && d <= uhi)
+                    in = box_d2((int)it.x, (int)it.y, (int)it.z, lx, ly, lz, hx, hy, hz) <= u2;
+                if (in) f(pos - ibase, it);
             }
         }
         __syncwarp();
@@ -364,7 +374,7 @@ __global__ void __launch_bounds__(256) k_cand_count(DevPtrs P, long long *u2out,
         int n = 0;
         bool keep = cand_radius(u2, cs, G) <= CAND_R_MAX;   // (always in a box of G <= 8)
         if (keep) {
-            cand_walk(P, b, cx, cy, cz, u2, [&](int, const int4 &) { ++n; });
+            cand_walk(P, b, cx, cy, cz, u2, [&](int, const float4 &) { ++n; });
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(FULLMASK, n, o);
             keep = n <= CAND_MAX;
@@ -391,22 +401,22 @@ __global__ void __launch_bounds__(256) k_cand_fill(DevPtrs P, const long long *u
         int cx = (int)(lc / ((long long)G * G)), cy = (int)((lc / G) % G), cz = (int)(lc % G);
         int mx = cand_centre(cx * cs, cs), my = cand_centre(cy * cs, cs), mz = cand_centre(cz * cs, cs);
         int w = cand_ring_width(cs);
-        const float winv = 1.0f / (float)w;
+        const float winv = 0.999999f / (float)w;
         long long u2 = u2in[c];
         long long a = P.grid.cand_off[c], e = P.grid.cand_off[c + 1];
         if (e == a) continue;   // no list: its queries take the grid walk
-        auto ring_of = [&](const int4 &it) {
-            long long dx = it.x - mx, dy = it.y - my, dz = it.z - mz;
-            // floor(floor(|p - m|) / w) in 32-bit arithmetic (in FP64, at 16 cycles of an SM a warp
-            // instruction, this was most of the kernel); r w <= |p - m| in any case
-            int s = (int)isqrt64(dx * dx + dy * dy + dz * dz);
-            int r = (int)((float)s * winv);
-            if (r * w > s) --r;
-            return min(r, 255);
+        const float fmx = (float)mx, fmy = (float)my, fmz = (float)mz;
+        auto ring_of = [&](const float4 &it) {
+            // |p - m| / w in FP32, shortened by 1e-6 (about six roundings), rounded down: r w <= |p - m|
+            // always, and one ring low at most (in FP64, at 16 cycles of an SM a warp instruction, this
+            // was most of the kernel)
+            const float dx = it.x - fmx, dy = it.y - fmy, dz = it.z - fmz;
+            const float s = sqrtf(__fmaf_rn(dx, dx, __fmaf_rn(dy, dy, dz * dz)));
+            return min((int)(s * winv), 255);
         };
         for (int k = lane; k < 256; k += 32) bin[k] = 0;
         __syncwarp();
-        cand_walk(P, b, cx, cy, cz, u2, [&](int, const int4 &it) { atomicAdd(&bin[ring_of(it)], 1); });
+        cand_walk(P, b, cx, cy, cz, u2, [&](int, const float4 &it) { atomicAdd(&bin[ring_of(it)], 1); });
         __syncwarp();
         // exclusive scan of the 256 bins: 8 per lane
         int loc[8], s = 0;
@@ -423,7 +433,7 @@ __global__ void __launch_bounds__(256) k_cand_fill(DevPtrs P, const long long *u
         for (int k = 0; k < 8; ++k) bin[lane * 8 + k] = incl - s + loc[k];
         __syncwarp();
         bool over = false;
-        cand_walk(P, b, cx, cy, cz, u2, [&](int ipos, const int4 &it) {
+        cand_walk(P, b, cx, cy, cz, u2, [&](int ipos, const float4 &it) {
             int r = ring_of(it);
             long long pos = a + atomicAdd(&bin[r], 1);
             if (pos < e) P.grid.cand[pos] = ((unsigned)r << 24) | (unsigned)ipos;
