@@ -401,16 +401,14 @@ __device__ __forceinline__ int axis_opposite(int nax, int b) {
     return b ^ 3;                           // vertex groups of four: both signs flip
 }
 
-// Recombination emission into the reception cones, deposit reset, frozen n_HI.  Bound by the
-// deposit words it clears and by FP64 (16 cycles of an SM per warp instruction): the words are
-// cleared key by key across the grid (coalesced, and only those the packet precision uses), the
-// rotated axes are computed for one of each opposite pair, and the particles' volumes, which a
-// step does not change, come from the upload.  512,000 particles, 9 bins, no emission: 246 ->
-// 41 us; the 64^3 HII region, 32 cones: 420 -> 203 us.
-template <typename Real, int NRC>
-__global__ void k_emit_rec(DevPtrs P, int *lens, int np) {
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    for (long long key = i; key < P.n * P.nf; key += (long long)gridDim.x * blockDim.x) {
+// The step's deposit words back to zero: key by key across the grid (coalesced), and only those
+// the packet precision uses.  A kernel of its own: in the step graph it runs beside the rotations,
+// which the FP64 pipe bounds, and takes their memory time (2.1 M particles with hardly any packets:
+// the step 0.6% shorter).
+template <typename Real>
+__global__ void k_clear_deposits(DevPtrs P) {
+    for (long long key = (long long)blockIdx.x * blockDim.x + threadIdx.x; key < P.n * P.nf;
+         key += (long long)gridDim.x * blockDim.x) {
         if (sizeof(Real) == 8) {
             P.abs[key] = 0.0; P.absE[key] = 0.0; P.pass[key] = 0.0;
         } else {
@@ -418,6 +416,16 @@ __global__ void k_emit_rec(DevPtrs P, int *lens, int np) {
         }
         P.fx_abs[key] = 0ull; P.fx_lo[key] = 0ull; P.fx_E[key] = 0ull;
     }
+}
+
+// Recombination emission into the reception cones, frozen n_HI.  Bound by FP64 (16 cycles of an
+// SM per warp instruction): the rotated axes are computed for one of each opposite pair, and
+// the particles' volumes, which a step does not change, come from the upload.  The 64^3 HII
+// region, 32 cones, with the deposit words cleared: 420 us with an axis a cone and strided
+// clearing, 203 us in one kernel.
+template <typename Real, int NRC>
+__global__ void k_emit_rec(DevPtrs P, int *lens, int np) {
+    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) {   // the hop loop starts with the step's np emitted packets in free buffer 0
         lens[0] = np;
         P.cnt[CNT_FCUR] = 0;
@@ -2326,6 +2334,10 @@ static rt_status transport_end(rt_ctx *c, bool fp32) {
     return RT_OK;
 }
 
+template <typename Real> static void clear_deposits(rt_ctx *c, cudaStream_t st) {
+    LAUNCH(KT_EMIT_REC, 1, (k_clear_deposits<Real><<<rt_blocks(c->d.n * c->d.nf, 256, 152 * 16), 256, 0, st>>>(c->d)));
+}
+
 template <typename Real, int NRC>
 static rt_status run_parts(rt_ctx *c, int part, long long step, cudaStream_t st) {
     DevPtrs &P = c->d;
@@ -2349,6 +2361,7 @@ static rt_status run_parts(rt_ctx *c, int part, long long step, cudaStream_t st)
         long long np = np_s + np_r;
         if (np > P.F_cap) return rt_fail(c, RT_ERR_CAPACITY, "source packets exceed free_cap");
         if (!c->capturing) set_step(c, step, st);
+        if (!c->capturing) clear_deposits<Real>(c, st);   // (the step graph has it on its other branch)
         LAUNCH(KT_EMIT_REC, 1, (k_emit_rec<Real, NRC><<<(unsigned)((n + tb - 1) / tb), tb, 0, st>>>(P, H.lens, (int)np)));
         c->fcur = 0;
         if (np_s > 0)
@@ -2427,9 +2440,11 @@ static rt_status capture_segment(rt_ctx *c, cudaGraph_t *out, rt_status (*body)(
 template <typename Real, int NRC>
 static rt_status seg_prologue(rt_ctx *c, cudaStream_t st) {
     rt_status s;
-    // the emitted-photon tally beside the rest: it reads what the last step's chemistry left
+    // beside the rest: the deposit words cleared, and the emitted-photon tally (it reads what the
+    // last step's chemistry left)
     cudaEventRecord(c->hev[0], st);
     cudaStreamWaitEvent(c->st2, c->hev[0], 0);
+    clear_deposits<Real>(c, c->st2);
     if ((s = rt_budget_launch(c, 0, c->st2))) return s;
     cudaEventRecord(c->hev[1], c->st2);
     if ((s = run_parts<Real, NRC>(c, 0, 0, st))) return s;
