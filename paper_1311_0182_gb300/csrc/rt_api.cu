@@ -413,8 +413,9 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     c->scan_tmp_n = RT_SCAN_NB;
     if (cudaMalloc(&c->scan_tmp, sizeof(int) * c->scan_tmp_n) != cudaSuccess) ok = false;
     if (cudaMallocHost(&c->cnt_h, sizeof(long long) * CNT_N) != cudaSuccess) ok = false;
-    // the hop loop's second stream, at the highest priority: its receiver-side kernels take
-    // SM slots ahead of the virtual-particle kernel that runs beside them
+    // the hop loop's second stream, at the highest priority: where the host drives the hops, its
+    // receiver-side kernels take SM slots ahead of the virtual-particle kernel beside them (the
+    // step graph keeps only the dependencies: a low priority measured the same)
     int prio_lo = 0, prio_hi = 0;
     cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
     if (cudaStreamCreateWithPriority(&c->st2, cudaStreamNonBlocking, prio_hi) != cudaSuccess)
