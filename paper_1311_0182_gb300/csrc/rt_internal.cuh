@@ -241,7 +241,9 @@ __device__ __forceinline__ unsigned long long gid_of(const DevPtrs &P, long long
     return (unsigned long long)(P.gid0[b] + (i - P.box_off[b]));
 }
 
-// kernel identities for the launch counter and the optional per-kernel timer
+// kernel identities for the launch counter and the optional per-kernel timer (KT_SCAN, KT_EXPAND,
+// KT_FREE_C, KT_SEG_SORT and KT_HOP_COUNT name passes that a hop no longer has; they keep the
+// positions of the others in rt_get_profile)
 enum {
     KT_ROTATE, KT_REBIN, KT_EMIT_REC, KT_EMIT_SRC, KT_PHASE_A, KT_FREE_A, KT_SCAN, KT_EXPAND,
     KT_FREE_C, KT_VIRTUAL, KT_SEG_FILL, KT_SEG_SORT, KT_PHASE_B, KT_HOP_COUNT, KT_HOP_LENS,
@@ -326,8 +328,7 @@ struct rt_ctx {
 // ---- helpers shared by the .cu files (host side) ----
 rt_status rt_fail(rt_ctx *c, rt_status s, const std::string &msg);
 rt_status rt_cuda_check(rt_ctx *c, cudaError_t e, const char *what);
-void rt_scan_exclusive(rt_ctx *c, const int *in, int *out, long long n, const int *d_len,
-                       int *d_total, cudaStream_t st, int *tmp = nullptr);
+void rt_scan_exclusive(rt_ctx *c, const int *in, int *out, long long n, cudaStream_t st);
 void rt_scan_exclusive64(const int *in, long long *out, long long n, long long *tmp,
                          cudaStream_t st);
 rt_status rt_knn_build(rt_ctx *c, cudaStream_t st);

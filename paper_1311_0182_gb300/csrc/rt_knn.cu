@@ -452,7 +452,7 @@ static void cell_lists(rt_ctx *c, cudaStream_t st) {
     cudaMemsetAsync(cnt, 0, sizeof(int) * (P.grid.ncells + 1), st);
     cudaMemsetAsync(fill, 0, sizeof(int) * (P.grid.ncells + 1), st);
     k_cell_count<<<nbk, tb, 0, st>>>(P, cnt);
-    rt_scan_exclusive(c, cnt, P.grid.start, P.grid.ncells + 1, nullptr, nullptr, st);
+    rt_scan_exclusive(c, cnt, P.grid.start, P.grid.ncells + 1, st);
     k_cell_fill<<<nbk, tb, 0, st>>>(P, fill);
 }
 
@@ -554,7 +554,7 @@ rt_status rt_knn_build(rt_ctx *c, cudaStream_t st) {
     long long ne = n * P.kn;
     unsigned nbe = (unsigned)((ne + tb - 1) / tb);
     k_rev_count<<<nbe, tb, 0, st>>>(P, cnt);
-    rt_scan_exclusive(c, cnt, P.rev_off, n + 1, nullptr, nullptr, st);
+    rt_scan_exclusive(c, cnt, P.rev_off, n + 1, st);
     k_rev_fill<<<nbe, tb, 0, st>>>(P, fill);
     k_rev_sort<<<rt_blocks(n * 32, tb, 152 * 32), tb, 0, st>>>(P);
     rt_status s = rt_cuda_check(c, cudaGetLastError(), "neighbour build");

@@ -1,7 +1,5 @@
-// rt_scan.cu -- exclusive prefix sum of int32 counts (cell lists, reverse lists, per-hop
-// requests and receiver segments).  `d_len` (optional) is a device-side element count; the
-// scan covers only the entries before it (the output beyond it is left as it was), so a
-// launch made for a capacity scans the live part without a host round trip.
+// rt_scan.cu -- exclusive prefix sums of int32 counts for the neighbour build (cell lists,
+// reverse lists, candidate lists).
 #include "rt_internal.cuh"
 
 #define SCAN_BLOCK 1024
@@ -35,9 +33,9 @@ __device__ __forceinline__ T block_excl_scan(T v, T *sh, T *total) {
     return r;
 }
 
-// Two kernels on a fixed grid of SCAN_NB blocks: block b owns one contiguous range of the
-// live part; the first kernel sums each range, the second scans it in tiles of SCAN_BLOCK,
-// starting from the sum of the ranges before it.  No launch is sized by the capacity.
+// Two kernels on a fixed grid of SCAN_NB blocks: block b owns one contiguous range; the first
+// kernel sums each range, the second scans it in tiles of SCAN_BLOCK, starting from the sum of
+// the ranges before it.
 #define SCAN_NB RT_SCAN_NB
 
 __device__ __forceinline__ void scan_range(long long len, long long &b0, long long &b1) {
@@ -47,16 +45,10 @@ __device__ __forceinline__ void scan_range(long long len, long long &b0, long lo
     b1 = b0 + per < len ? b0 + per : len;
 }
 
-__device__ __forceinline__ long long scan_len(long long n, const int *d_len) {
-    long long len = d_len ? (long long)*d_len : n;
-    return len < n ? len : n;
-}
-
-__global__ void __launch_bounds__(SCAN_BLOCK) k_scan_sum(const int *in, long long n,
-                                                         const int *d_len, int *btot) {
+__global__ void __launch_bounds__(SCAN_BLOCK) k_scan_sum(const int *in, long long n, int *btot) {
     __shared__ int sh[33];
     long long b0, b1;
-    scan_range(scan_len(n, d_len), b0, b1);
+    scan_range(n, b0, b1);
     int v = 0;
     for (long long i = b0 + threadIdx.x; i < b1; i += SCAN_BLOCK) v += in[i];
     int tot;
@@ -65,22 +57,15 @@ __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_sum(const int *in, long lon
 }
 
 __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_fin(const int *in, int *out, long long n,
-                                                         const int *d_len, const int *btot,
-                                                         int *d_total) {
+                                                         const int *btot) {
     __shared__ int sh[33];
     long long b0, b1;
-    scan_range(scan_len(n, d_len), b0, b1);
-    // the sum of the ranges before this block (and of all of them, for the total)
-    int before = 0, all = 0;
-    for (int k = threadIdx.x; k < SCAN_NB; k += SCAN_BLOCK) {
-        int t = btot[k];
-        all += t;
-        if (k < (int)blockIdx.x) before += t;
-    }
-    int tb, ta;
+    scan_range(n, b0, b1);
+    // the sum of the ranges before this block
+    int before = 0;
+    for (int k = threadIdx.x; k < (int)blockIdx.x; k += SCAN_BLOCK) before += btot[k];
+    int tb;
     block_excl_scan(before, sh, &tb);
-    block_excl_scan(all, sh, &ta);
-    if (blockIdx.x == 0 && threadIdx.x == 0 && d_total) *d_total = ta;
     int carry = tb;
     for (long long base = b0; base < b1; base += SCAN_BLOCK) {
         long long i = base + threadIdx.x;
@@ -92,17 +77,13 @@ __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_fin(const int *in, int *out
     }
 }
 
-// tmp: block-total scratch of at least SCAN_NB ints (default: the context's); two scans in
-// flight at once need two.
-void rt_scan_exclusive(rt_ctx *c, const int *in, int *out, long long n, const int *d_len,
-                       int *d_total, cudaStream_t st, int *tmp) {
-    if (!tmp) tmp = c->scan_tmp;
-    k_scan_sum<<<SCAN_NB, SCAN_BLOCK, 0, st>>>(in, n, d_len, tmp);
-    k_scan_fin<<<SCAN_NB, SCAN_BLOCK, 0, st>>>(in, out, n, d_len, tmp, d_total);
+void rt_scan_exclusive(rt_ctx *c, const int *in, int *out, long long n, cudaStream_t st) {
+    k_scan_sum<<<SCAN_NB, SCAN_BLOCK, 0, st>>>(in, n, c->scan_tmp);
+    k_scan_fin<<<SCAN_NB, SCAN_BLOCK, 0, st>>>(in, out, n, c->scan_tmp);
 }
 
 // The same scan into 64-bit offsets (the per-cell candidate lists, whose total can pass 2^31):
-// counts are int32, sums and offsets int64; no device-side length.
+// counts are int32, sums and offsets int64.
 __global__ void __launch_bounds__(SCAN_BLOCK) k_scan64_sum(const int *in, long long n,
                                                            long long *btot) {
     __shared__ long long sh[33];
