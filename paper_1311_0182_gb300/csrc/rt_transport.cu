@@ -617,9 +617,13 @@ template <typename Real> struct SentPacket {
 // cur: the slot buffer holding the hop's packets.  Receivers of a bitmap word are flagged in
 // `touched` (cleared again by the work-list kernel).
 // SH: the shared frequency bin (a separate instance keeps its code out of the common case)
+// nu0, nfl: a launch serves the frequencies nu0 .. nu0 + nfl - 1 (at most 32, a lane a word); with
+// more than 32 bins a hop takes several launches.  Each bitmap word belongs to one frequency, so
+// it is still written once.
 // lens: the hop's counts (the request list is lens[2] long); null: no requests (inspection)
 template <typename Real, int NRC, bool SH>
-__global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int cur, int per, int *lens) {
+__global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int cur, int per, int nu0,
+                                                                int nfl, int *lens) {
     __shared__ unsigned slist[8][32];
     __shared__ unsigned sreq[8][64];   // requests not yet in the list
     __shared__ int snext, scnt[8];
@@ -628,7 +632,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int c
     int nrq = 0;
     const float cf = 1.0f - 2.0f / (float)P.ntc;
     const long long nrev = P.n * P.kn;
-    const unsigned pmask = P.nf < 32 ? (1u << P.nf) - 1u : FULLMASK;   // a particle's words
+    const unsigned pmask = nfl < 32 ? (1u << nfl) - 1u : FULLMASK;   // a particle's words
     long long ncon = 0;
     int nsend = 0;
     // each block takes one contiguous chunk of particles; its warps pull from it through a
@@ -639,7 +643,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int c
     const long long ib1 = ib0 + chunk < P.n ? ib0 + chunk : P.n;
     if (threadIdx.x == 0) snext = 0;
     __syncthreads();
-    const int lp = lane / P.nf, lnu = lane - lp * P.nf;      // the lane's particle and frequency
+    const int lp = lane / nfl, lnu = nu0 + lane - lp * nfl;  // the lane's particle and frequency
     auto words = [&](long long i) {
         return (i + lp < ib1 && lp < per) ? P.act[cur][(i + lp) * P.nf + lnu] : 0u;
     };
@@ -664,7 +668,10 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int c
         const long long ic = i0 + u * per;
         const unsigned moving = __ballot_sync(FULLMASK, aw != 0u);
         if (moving == 0u) continue;
-        nsend += lane < per && ((moving >> (lane * P.nf)) & pmask) != 0u;
+        bool sends = lane < per && ((moving >> (lane * nfl)) & pmask) != 0u;
+        for (int nu = 0; nu < nu0; ++nu)      // a particle counts once, in its first launch
+            sends = sends && P.act[cur][(ic + lane) * P.nf + nu] == 0u;
+        nsend += sends;
         const unsigned cnt = (unsigned)__popc(aw);
         const unsigned incl = lane_scan(cnt);
         const int total = (int)__shfl_sync(FULLMASK, incl, 31);
@@ -2196,9 +2203,25 @@ static void set_step(rt_ctx *c, long long step, cudaStream_t st) {
 // particles spread over the chip more than it needs full lanes: 32 warps an SM with FP32
 // packets; 8 with FP64 packets, where a few warps already fill the FP64 pipe and fuller lanes
 // mean fewer of its instructions (the 16^3 sphere's step: 1.79 ms with 32, 1.67 with 8, 1.73 with 4).
-static int send_turn(const DevPtrs &P) {
-    long long most = std::max(1, 32 / P.nf);
+// nu0: the launch's first frequency.
+static int send_turn(const DevPtrs &P, int nu0) {
+    long long most = std::max(1, 32 / (P.nf - nu0));
     return (int)std::min(most, std::max(1ll, P.n / (152 * (P.fp32 ? 32 : 8))));
+}
+
+// The sender side of a hop (lens: its counts; null: inspection, no requests), 32 frequencies a launch.
+template <typename Real, int NRC>
+static void launch_senders(rt_ctx *c, cudaStream_t st, int cur, int max_blocks, int *lens) {
+    const DevPtrs &P = c->d;
+    const int tb = 256;
+    for (int nu0 = 0; nu0 < P.nf; nu0 += 32) {
+        const int per = send_turn(P, nu0), nfl = std::min(32, P.nf - nu0);
+        const int nb = rt_blocks((P.n + per - 1) / per * 32, tb, max_blocks);
+        if (P.shared)
+            LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, true><<<nb, tb, 0, st>>>(P, cur, per, nu0, nfl, lens)));
+        else
+            LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, false><<<nb, tb, 0, st>>>(P, cur, per, nu0, nfl, lens)));
+    }
 }
 
 // One hop, in six launches and a bookkeeping kernel (k_hop_lens HL_END, launched by the
@@ -2220,8 +2243,7 @@ static void hop_core(rt_ctx *c, cudaStream_t st, long long nfr, int cur, int fcu
     const int GB = c->grid_hop[2] ? c->grid_hop[2] : GRID_B;
     HopScratch &H = c->hop;
     const int tb = 256;
-    long long n = P.n, nkey = n * P.nf;
-    const int per = send_turn(P);
+    long long nkey = P.n * P.nf;
     cudaStream_t s2 = c->st2;
     cudaEvent_t evFork = c->hev[0], evA = c->hev[1], evFree = c->hev[2], evB = c->hev[3];
     if (nfr < 1) nfr = 1;
@@ -2237,11 +2259,7 @@ static void hop_core(rt_ctx *c, cudaStream_t st, long long nfr, int cur, int fcu
     else
         LAUNCH_ON(s2, KT_FREE_A, 1, (k_free<Real, NRC, false, false><<<nbf, tb, 0, s2>>>(P, fcur, H.lens)));
     cudaEventRecord(evFree, s2);
-    const int nba = rt_blocks((n + per - 1) / per * 32, tb, GA);
-    if (P.shared)
-        LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, true><<<nba, tb, 0, st>>>(P, cur, per, H.lens)));
-    else
-        LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, false><<<nba, tb, 0, st>>>(P, cur, per, H.lens)));
+    launch_senders<Real, NRC>(c, st, cur, GA, H.lens);
     cudaEventRecord(evA, st);
     cudaStreamWaitEvent(s2, evA, 0);
     LAUNCH_ON(s2, KT_WORKLIST, 1, (k_worklist<<<rt_blocks(nkey, 1024, 152 * 8), tb, 0, s2>>>(P, cur, H.lens)));
@@ -2374,11 +2392,7 @@ static rt_status run_parts(rt_ctx *c, int part, long long step, cudaStream_t st)
     if (part == 3) {  // cone masks of the held packets only (inspection)
         clear_cone_bits(c, st);
         c->bm_dirty = true;
-        const int per = send_turn(P);
-        if (P.shared)
-            LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, true><<<rt_blocks((n + per - 1) / per * 32, tb, 152 * 64), tb, 0, st>>>(P, c->cur, per, nullptr)));
-        else
-            LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, false><<<rt_blocks((n + per - 1) / per * 32, tb, 152 * 64), tb, 0, st>>>(P, c->cur, per, nullptr)));
+        launch_senders<Real, NRC>(c, st, c->cur, 152 * 64, nullptr);
         return rt_cuda_check(c, cudaGetLastError(), "cone masks");
     }
     // part 4: the hop loop, driven from the host (one synchronisation per hop)
