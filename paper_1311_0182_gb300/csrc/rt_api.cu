@@ -391,15 +391,15 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     }
     A(P.st_key, int, P.ST_cap);
     A(P.st_bin, int, P.ST_cap);
-    A(P.st_ord, unsigned long long, P.ST_cap);
+    A(P.st_pkt, int, P.ST_cap);
     A(P.st_rank, int, P.ST_cap);
+    P.seg_srt = P.st_rank;
     for (int f = 0; f < 9; ++f) P.st_v[f] = dalloc(c, R * P.ST_cap, &ok);
     if (P.shared) P.st_v[9] = dalloc(c, R * P.ST_cap, &ok);
     long long segn = std::max<long long>(nkey, ncell) + 4;
     A(P.seg_cnt, int, segn);
     A(P.seg_off, int, segn);
     A(P.seg_fill, int, segn);
-    A(P.seg_ent, ulonglong2, P.ST_cap);
     A(P.seg_idx, int, P.ST_cap);
     A(P.abs, double, nkey); A(P.absE, double, nkey); A(P.pass, double, nkey);
     A(P.passf, float, nkey);

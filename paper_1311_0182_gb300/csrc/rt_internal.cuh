@@ -211,14 +211,14 @@ struct DevPtrs {              // plain pointers handed to kernels (by value)
     FreeBuf fr[2];
     // staged free-packet contributions
     int *st_key;              // receiver key j*nf+nu
-    unsigned long long *st_ord;  // the packet's order (one contribution a receiver)
+    int *st_pkt;              // its packet (one contribution a receiver)
     int *st_rank;             // place among the receiver's contributions, in arrival order
     int *st_bin;
     void *st_v[10];           // T, T dx, T dy, T dz, T clock, T eps, A, A eps, w, T sigma (Real;
                               // the last with a shared bin only)
     int *seg_cnt, *seg_off;   // per key: contributions (zero between hops) and first entry
-    ulonglong2 *seg_ent;      // (order of the packet, contribution), in arrival order
-    int *seg_idx;             // contributions in packet order
+    int *seg_idx;             // contributions in arrival order
+    int *seg_srt;             // in packet order (st_rank's memory: ranks are read before)
     int *seg_fill;            // scratch of the neighbour build
     // accumulators
     double *abs, *absE, *pass;                // [n * nf]

@@ -821,7 +821,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int c
 // collects the members of their cones in a list.  32 members at a time (lane = member) become
 // staged contributions, at a position from one counter: a packet has about one member, so a
 // warp of its own computed one contribution with one lane.  The position is arbitrary; a
-// contribution carries its packet's order (st_ord), by which the receiver orders its segment, and its
+// contribution names its packet (st_pkt), by whose order the receiver orders its segment, and its
 // place among the receiver's (st_rank, the count before it).  A packet without a member
 // requests a virtual particle.  Measured per step against two kernels and a prefix sum with a
 // warp a packet: 64^3 HII region 7.4 -> 3.6 ms, the FP64 path at 32^3 4.7 -> 1.8 ms.
@@ -865,7 +865,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_free(DevPtrs P, int fcu
             const long long key = j * P.nf + nu;
             Real **V = (Real **)P.st_v;
             P.st_key[s] = (int)key;
-            P.st_ord[s] = F.okey[f];
+            P.st_pkt[s] = (int)f;
             int bt = -1;
             if (BAR && barrier_crosses_call(P.bar[q.w], fx, fy, fz, q.x, q.y, q.z)) {
                 // the share crosses the barrier: removed (counted escaped); the staged
@@ -1473,13 +1473,13 @@ __global__ void __launch_bounds__(256) k_worklist(DevPtrs P, int cur, int *lens)
     }
 }
 
-// the staged contributions into their receivers' segments, with their packets
+// the staged contributions into their receivers' segments
 __global__ void __launch_bounds__(256) k_seg_fill(DevPtrs P, const int *lens) {
     long long nst = lens[3];
     if (nst > P.ST_cap) nst = P.ST_cap;
     for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < nst;
          s += (long long)gridDim.x * blockDim.x)
-        P.seg_ent[P.seg_off[P.st_key[s]] + P.st_rank[s]] = make_ulonglong2(P.st_ord[s], (unsigned long long)s);
+        P.seg_idx[P.seg_off[P.st_key[s]] + P.st_rank[s]] = (int)s;
 }
 
 // absorptions of one receiver group in one hop.  FP64 path: FP64 sums.  FP32 path: the
@@ -1577,15 +1577,67 @@ __device__ __forceinline__ int staged_contribution(const DevPtrs &P, int s, int 
     return bin;
 }
 
-// A segment of n staged contributions in packet order, by eight lanes: each takes the place
-// given by the number of earlier packets (distinct).  Out of line: few groups have any, and
-// inlined it costs the receiver side registers.
-static __device__ __noinline__ void order_segment(const ulonglong2 *ent, int *idx, int n) {
-    for (int c = threadIdx.x & 7; c < n; c += 8) {
-        const ulonglong2 e = ent[c];
+// A segment of n > 8 contributions from idx into srt in packet order, by the whole warp: blocks of
+// 32 by counting earlier packets (distinct), then sorted runs merged in pairs, an entry's place
+// being its place in its run and the earlier ones of the other (binary search).  The passes
+// alternate between idx and srt and end in srt.  Counting the earlier packets of the whole segment,
+// without the merges, is quadratic: 20,000 sources within one smoothing length give their
+// neighbours segments of 20,000, and a step of a 32^3 box took 2.1 s (FP32), 48 ms now; with 4,096
+// sources 96 and 12 ms.
+__device__ void order_wide(const unsigned long long *okey, const int *pkt, int *idx, int *srt,
+                           unsigned n) {
+    const unsigned lane = threadIdx.x & 31u;
+    bool odd = false;                  // number of merge passes
+    for (unsigned L = 32; L < n; L *= 2) odd = !odd;
+    int *a = odd ? idx : srt, *b = odd ? srt : idx;
+    for (unsigned c = 0; c < n; c += 32) {
+        const bool on = c + lane < n;
+        const int s = on ? idx[c + lane] : 0;
+        const unsigned long long key = on ? okey[pkt[s]] : ~0ull;
         int r = 0;
-        for (int k = 0; k < n; ++k) r += ent[k].x < e.x;
-        idx[r] = (int)e.y;
+        for (int k = 0; k < 32; ++k) r += __shfl_sync(FULLMASK, key, k) < key;
+        if (on) a[c + r] = s;
+    }
+    __syncwarp();
+    for (unsigned L = 32; L < n; L *= 2) {
+        for (unsigned t = lane; t < n; t += 32) {
+            const int s = a[t];
+            const unsigned long long key = okey[pkt[s]];
+            const unsigned run = t & ~(L - 1u), other = run ^ L;
+            unsigned lo = min(other, n), hi = min(other + L, n);
+            const unsigned o0 = lo;
+            while (lo < hi) {
+                const unsigned m = (lo + hi) >> 1;
+                if (okey[pkt[a[m]]] < key) lo = m + 1u;
+                else hi = m;
+            }
+            b[min(run, other) + (t - run) + (lo - o0)] = s;
+        }
+        __syncwarp();
+        int *x = a;
+        a = b;
+        b = x;
+    }
+}
+
+// The four segments of a warp (n contributions each, lanes of eight hold the same) from idx into
+// srt in packet order.  Up to eight: a lane an entry, all four at once.  Out of line: few groups
+// have any, and inlined it costs the receiver side registers.
+static __device__ __noinline__ void order_segments(const unsigned long long *okey, const int *pkt,
+                                                   int *idx, int *srt, int n) {
+    const int lane = threadIdx.x & 31, l = lane & 7;
+    const bool on = n <= 8 && l < n;
+    const int s = on ? idx[l] : 0;
+    const unsigned long long key = on && n > 1 ? okey[pkt[s]] : ~0ull;
+    int r = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) r += __shfl_sync(FULLMASK, key, k, 8) < key;
+    if (on) srt[r] = s;
+    for (unsigned w = __ballot_sync(FULLMASK, n > 8 && l == 0); w; w &= w - 1u) {
+        const int k = __ffs(w) - 1;
+        order_wide(okey, pkt, (int *)__shfl_sync(FULLMASK, (unsigned long long)idx, k),
+                   (int *)__shfl_sync(FULLMASK, (unsigned long long)srt, k),
+                   (unsigned)__shfl_sync(FULLMASK, n, k));
     }
     __syncwarp();
 }
@@ -1706,7 +1758,7 @@ __device__ __forceinline__ void wide_group(const DevPtrs &P, int cur, long long 
     for (int cb = 0; cb < fc; cb += 32) {
         int bin = -1;
         if (cb + lane < fc)
-            bin = staged_contribution<Real, SH>(P, P.seg_idx[so + cb + lane], nu, sv, lane);
+            bin = staged_contribution<Real, SH>(P, P.seg_srt[so + cb + lane], nu, sv, lane);
         merge(bin);
     }
     const Real N = a.photons();
@@ -1754,9 +1806,10 @@ __device__ __forceinline__ void wide_group(const DevPtrs &P, int cur, long long 
 // of n_rc edges, modulo n_rc), then a tree over the lanes.  Results do not depend on how
 // groups meet in a warp.
 // Groups come from the work list; the next buffer's occupancy words were cleared by the
-// work-list kernel.  cur: the slot buffer holding the hop's packets.
+// work-list kernel.  cur, fcur: the slot and free-packet buffers holding the hop's packets.
 template <typename Real, int G, bool BAR, bool SH>
-__global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int cur, const int *lens) {
+__global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int cur, int fcur,
+                                                                const int *lens) {
     __shared__ Pair<Real> svs[8][BV_N][32];
     __shared__ unsigned slist[8][32];
     __shared__ unsigned smask[8][2][32];
@@ -1799,7 +1852,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int c
         const Real sig_nhi = sigma_of<Real>(P, nu) * ((Real *)P.nHIr)[j];
         Slots<Real> So(P, cur), Sn(P, nxt);
         if (__any_sync(FULLMASK, fc > 0)) {
-            order_segment(P.seg_ent + so, P.seg_idx + so, fc);
+            order_segments(P.fr[fcur].okey, P.st_pkt, P.seg_idx + so, P.seg_srt + so, fc);
             if ((lane & 7) == 0 && fc > 0) P.seg_cnt[key] = 0;   // for the next hop
         }
         // a group's values to the lanes that work on it
@@ -1913,7 +1966,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int c
                 const int c = p - (kk == 0 ? 0 : kk == 1 ? f1 : kk == 2 ? f2 : f3);
                 const int sok = of(so, kk), nuk = of(nu, kk);
                 int bin = -1;
-                if (p < ft) bin = staged_contribution<Real, SH>(P, P.seg_idx[sok + c], nuk, sv, lane);
+                if (p < ft) bin = staged_contribution<Real, SH>(P, P.seg_srt[sok + c], nuk, sv, lane);
                 merge(kk, bin, c & 7);
             }
             // the merged packets
@@ -2027,7 +2080,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int c
                     bin = gas_contribution<Real, G, BAR, SH>(P, (long long)e0k + ((code >> 5) & 63u),
                                                              code & 31u, jk, nuk, boxk, uk, snk, sv, lane);
                 else if (lane < n)
-                    bin = staged_contribution<Real, SH>(P, P.seg_idx[sok + ec], nuk, sv, lane);
+                    bin = staged_contribution<Real, SH>(P, P.seg_srt[sok + ec], nuk, sv, lane);
                 __syncwarp();
                 // the lowest lane of each (group, cone) adds its contributions in list order
                 const unsigned live = __ballot_sync(FULLMASK, bin >= 0);
@@ -2267,11 +2320,11 @@ static void hop_core(rt_ctx *c, cudaStream_t st, long long nfr, int cur, int fcu
     cudaStreamWaitEvent(st, evFree, 0);
     const int nbb = rt_blocks(nkey * 8, tb, GB);
     if (P.shared)
-        LAUNCH_ON(s2, KT_PHASE_B, 1, (k_phaseB<Real, NRC, true, true><<<nbb, tb, 0, s2>>>(P, cur, H.lens)));
+        LAUNCH_ON(s2, KT_PHASE_B, 1, (k_phaseB<Real, NRC, true, true><<<nbb, tb, 0, s2>>>(P, cur, fcur, H.lens)));
     else if (P.any_bar)
-        LAUNCH_ON(s2, KT_PHASE_B, 1, (k_phaseB<Real, NRC, true, false><<<nbb, tb, 0, s2>>>(P, cur, H.lens)));
+        LAUNCH_ON(s2, KT_PHASE_B, 1, (k_phaseB<Real, NRC, true, false><<<nbb, tb, 0, s2>>>(P, cur, fcur, H.lens)));
     else
-        LAUNCH_ON(s2, KT_PHASE_B, 1, (k_phaseB<Real, NRC, false, false><<<nbb, tb, 0, s2>>>(P, cur, H.lens)));
+        LAUNCH_ON(s2, KT_PHASE_B, 1, (k_phaseB<Real, NRC, false, false><<<nbb, tb, 0, s2>>>(P, cur, fcur, H.lens)));
     cudaEventRecord(evB, s2);
     const int IS = KNN_IB_SMALL, IL = KNN_IB_LARGE;
     const int nbv = rt_blocks(P.F_cap * 32, tb, GV);
