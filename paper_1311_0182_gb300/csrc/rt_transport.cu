@@ -617,13 +617,14 @@ template <typename Real> struct SentPacket {
 // cur: the slot buffer holding the hop's packets.  Receivers of a bitmap word are flagged in
 // `touched` (cleared again by the work-list kernel).
 // SH: the shared frequency bin (a separate instance keeps its code out of the common case)
-// nu0, nfl: a launch serves the frequencies nu0 .. nu0 + nfl - 1 (at most 32, a lane a word); with
-// more than 32 bins a hop takes several launches.  Each bitmap word belongs to one frequency, so
-// it is still written once.
+// WIDE: more than 32 frequencies, in several launches a hop (an instance of its own likewise): one
+// serves the frequencies nu0 .. nu0 + nfl - 1 (at most 32, a lane a word).  Each bitmap word belongs
+// to one frequency, so it is still written once.
 // lens: the hop's counts (the request list is lens[2] long); null: no requests (inspection)
-template <typename Real, int NRC, bool SH>
-__global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int cur, int per, int nu0,
-                                                                int nfl, int *lens) {
+template <typename Real, int NRC, bool SH, bool WIDE>
+__global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int cur, int per, int nu0w,
+                                                                int nflw, int *lens) {
+    const int nu0 = WIDE ? nu0w : 0, nfl = WIDE ? nflw : P.nf;
     __shared__ unsigned slist[8][32];
     __shared__ unsigned sreq[8][64];   // requests not yet in the list
     __shared__ int snext, scnt[8];
@@ -669,8 +670,9 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int c
         const unsigned moving = __ballot_sync(FULLMASK, aw != 0u);
         if (moving == 0u) continue;
         bool sends = lane < per && ((moving >> (lane * nfl)) & pmask) != 0u;
-        for (int nu = 0; nu < nu0; ++nu)      // a particle counts once, in its first launch
-            sends = sends && P.act[cur][(ic + lane) * P.nf + nu] == 0u;
+        if (WIDE)                             // a particle counts once, in its first launch
+            for (int nu = 0; nu < nu0; ++nu)
+                sends = sends && P.act[cur][(ic + lane) * P.nf + nu] == 0u;
         nsend += sends;
         const unsigned cnt = (unsigned)__popc(aw);
         const unsigned incl = lane_scan(cnt);
@@ -2270,10 +2272,9 @@ static void launch_senders(rt_ctx *c, cudaStream_t st, int cur, int max_blocks, 
     for (int nu0 = 0; nu0 < P.nf; nu0 += 32) {
         const int per = send_turn(P, nu0), nfl = std::min(32, P.nf - nu0);
         const int nb = rt_blocks((P.n + per - 1) / per * 32, tb, max_blocks);
-        if (P.shared)
-            LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, true><<<nb, tb, 0, st>>>(P, cur, per, nu0, nfl, lens)));
-        else
-            LAUNCH(KT_PHASE_A, 1, (k_phaseA<Real, NRC, false><<<nb, tb, 0, st>>>(P, cur, per, nu0, nfl, lens)));
+        auto kernel = P.nf <= 32 ? (P.shared ? k_phaseA<Real, NRC, true, false> : k_phaseA<Real, NRC, false, false>)
+                                 : (P.shared ? k_phaseA<Real, NRC, true, true> : k_phaseA<Real, NRC, false, true>);
+        LAUNCH(KT_PHASE_A, 1, (kernel<<<nb, tb, 0, st>>>(P, cur, per, nu0, nfl, lens)));
     }
 }
 
