@@ -320,14 +320,11 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     A(P.bpart, double, 2 * (long long)P.nbch);
     A(x->src_emit, double, n_boxes);
     A(P.pbox, int, n);
-    A(P.qx, int, n); A(P.qy, int, n); A(P.qz, int, n);
     A(P.q4, int4, n);
     A(P.nH, double, n); A(P.NH, double, n); A(P.xHI, double, n); A(P.T, double, n);
     A(P.Nrec, double, n); A(P.epsrec, double, n); A(P.nHI, double, n); A(P.phot, double, n);
-    P.nHIr = dalloc(c, R * n, &ok);
-    P.Vr = dalloc(c, R * n, &ok);
-    P.dep_s = dalloc(c, R * n, &ok);
-    P.depE_s = dalloc(c, R * n, &ok);
+    P.nHIr = P.nHI;
+    if (P.fp32) P.nHIr = dalloc(c, R * n, &ok);
     P.vpv = dalloc(c, 4 * R * n, &ok);
     A(P.sbox, int, n_src + 1);
     A(P.gid0, long long, n_boxes);
@@ -347,9 +344,7 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     A(P.sgate, int, n_src + 1);
     A(P.bar, Barrier, n_boxes);
     A(P.fwd4, float4, n * P.kn);
-    A(P.revpos, int, n * P.kn);
     A(P.rev_off, int, n + 1);
-    A(P.rev_ent, unsigned, n * P.kn);
     A(P.rev4, float4, n * P.kn);
     A(P.grid.G, int, n_boxes);
     A(P.grid.cs, int, n_boxes);
@@ -372,8 +367,11 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
         A(P.act[b], unsigned, nkey + 4);
     }
     P.rec = dalloc(c, 8 * R * nslot, &ok);
+    P.b_ent = (unsigned *)P.rec;     // 2 * 4 * 32 bytes a particle at most, of 8 * 4 * 8 at least
+    P.b_pos = (int *)P.rec + n * P.kn;
     A(P.bm, unsigned, n * P.kn * P.nf);
-    A(P.worklist, int, nkey);
+    A(P.worklist, int, nkey + 4);
+    P.b_fill = P.worklist;           // cells and particles: ncell <= n <= nkey, and one more
     A(P.touched, unsigned char, nkey + 4);
     A(P.req, unsigned long long, fc);
     for (int b = 0; b < 2; ++b) {
@@ -391,18 +389,20 @@ extern "C" rt_status rt_create(const rt_config *cfg, int n_boxes, const long lon
     }
     A(P.st_key, int, P.ST_cap);
     A(P.st_bin, int, P.ST_cap);
-    A(P.st_pkt, int, P.ST_cap);
-    A(P.st_rank, int, P.ST_cap);
-    P.seg_srt = P.st_rank;
-    for (int f = 0; f < 9; ++f) P.st_v[f] = dalloc(c, R * P.ST_cap, &ok);
-    if (P.shared) P.st_v[9] = dalloc(c, R * P.ST_cap, &ok);
+    A(P.seg_tmp, int2, P.ST_cap);
+    P.st_rank = (int *)P.seg_tmp;
+    P.st_pkt = P.st_rank + P.ST_cap;
+    for (int f = 0; f < 4; ++f) P.st_v[f] = dalloc(c, R * P.ST_cap, &ok);
     long long segn = std::max<long long>(nkey, ncell) + 4;
     A(P.seg_cnt, int, segn);
     A(P.seg_off, int, segn);
-    A(P.seg_fill, int, segn);
-    A(P.seg_idx, int, P.ST_cap);
-    A(P.abs, double, nkey); A(P.absE, double, nkey); A(P.pass, double, nkey);
-    A(P.passf, float, nkey);
+    A(P.seg_ent, int2, P.ST_cap);
+    A(P.seg_key, unsigned long long, P.ST_cap);
+    if (P.fp32) {
+        A(P.passf, float, nkey);
+    } else {
+        A(P.abs, double, nkey); A(P.absE, double, nkey); A(P.pass, double, nkey);
+    }
     A(P.fx_abs, unsigned long long, nkey);
     A(P.fx_E, unsigned long long, nkey);
     A(P.fx_lo, unsigned long long, nkey);
@@ -1053,7 +1053,8 @@ extern "C" rt_status rt_get_neighbours(rt_ctx *c, int *nbr, long long *h2, int *
 __global__ void k_get_q(DevPtrs P, long long *q) {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P.n) return;
-    q[3 * i] = P.qx[i]; q[3 * i + 1] = P.qy[i]; q[3 * i + 2] = P.qz[i];
+    const int4 v = P.q4[i];
+    q[3 * i] = v.x; q[3 * i + 1] = v.y; q[3 * i + 2] = v.z;
 }
 
 template <typename T> static T *dtmp(size_t n) {
@@ -1150,7 +1151,7 @@ __global__ void k_masks(DevPtrs P, int cur, unsigned *out) {
     const unsigned *bmr = P.bm + (long long)nu * P.n * P.kn;
     if ((a >> b) & 1u)
         for (int k = 0; k < P.kn; ++k)
-            m |= ((bmr[P.revpos[i * P.kn + k]] >> b) & 1u) << k;
+            m |= ((bmr[__float_as_int(P.fwd4[i * P.kn + k].w)] >> b) & 1u) << k;
     out[t] = m;
 }
 
@@ -1329,13 +1330,13 @@ __global__ void k_deposits(DevPtrs P, double *a, double *e, double *ps) {
     long long key = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (key >= P.n * P.nf) return;
     long long i = key / P.nf;
-    ps[key] = P.pass[key] + (double)P.passf[key] * P.norm[P.pbox[i]];
+    ps[key] = P.fp32 ? (double)P.passf[key] * P.norm[P.pbox[i]] : P.pass[key];
     // the fixed-point words count in units of the neutral atoms at the start of the step (the
     // n_HI frozen for the transport), not of the x_HI the chemistry has written since
     double NHI = P.nH[i] > 0.0 ? P.nHI[i] / P.nH[i] * P.NH[i] : 0.0;
-    a[key] = P.abs[key] + ((double)P.fx_abs[key] + (double)P.fx_lo[key] / FX_LO_SCALE) *
+    a[key] = (P.fp32 ? 0.0 : P.abs[key]) + ((double)P.fx_abs[key] + (double)P.fx_lo[key] / FX_LO_SCALE) *
                               (NHI / FX_ABS_SCALE);
-    e[key] = P.absE[key] + (double)P.fx_E[key] * (NHI * 1.602176634e-12 / FX_E_SCALE);
+    e[key] = (P.fp32 ? 0.0 : P.absE[key]) + (double)P.fx_E[key] * (NHI * 1.602176634e-12 / FX_E_SCALE);
 }
 
 extern "C" rt_status rt_get_deposits(rt_ctx *c, double *abs_, double *absE, double *pass,

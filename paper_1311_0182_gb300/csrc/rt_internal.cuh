@@ -163,12 +163,11 @@ struct DevPtrs {              // plain pointers handed to kernels (by value)
     long long *bch_lo;        // [nbch + 1] particle ranges
     double *bpart;            // [nbch * 2]
     // particles
-    int *pbox, *qx, *qy, *qz;
+    int *pbox;
     int4 *q4;                 // (qx, qy, qz, box)
     double *nH, *NH, *xHI, *T, *Nrec, *epsrec, *nHI, *phot;
-    void *nHIr, *Vr, *depE_s;  // Real [n]
-    void *dep_s;               // Real [n]: fixed-point scale of photon deposits
-    void *vpv;                 // Real [n * 4]: volume, n_HI and the two deposit scales, together
+    void *nHIr;               // Real [n]: n_HI of the transport (FP64: nHI itself)
+    void *vpv;                // Real [n * 4]: PV_VOL, PV_NHI, PV_DEP, PV_DEPE of each particle
     // sources
     int *sbox, *sqx, *sqy, *sqz;
     // identities in the random streams: particle i of box b draws as gid0[b] + (i - box_off[b]),
@@ -186,11 +185,15 @@ struct DevPtrs {              // plain pointers handed to kernels (by value)
     int any_bar;              // some box has a barrier
     int kwide;                // some box holds more than 2^22 particles (24-bit kNN keys)
     int gated;                // some source has a gate
-    float4 *fwd4;             // [n * kn]: offset q_j - q_i, and the neighbour j (its bits)
-    int *revpos;              // [n * kn]: the entry's position in the reverse lists
+    float4 *fwd4;             // [n * kn]: offset q_j - q_i, and the place in the reverse lists (its bits)
     int *rev_off;
-    unsigned *rev_ent;        // (i << 5) | k
-    float4 *rev4;             // the same order: offset q_j - q_i, and the sender i (its bits)
+    float4 *rev4;             // in reverse order: offset q_j - q_i, and the sender i (its bits)
+    // scratch of the neighbour build, in arrays that hold nothing outside a hop: reverse entries
+    // (i << 5) | k and the places in the reverse lists per edge (in rec), a counter per cell or
+    // particle (in worklist)
+    unsigned *b_ent;
+    int *b_pos;
+    int *b_fill;
     Grid grid;
     // rotations
     double *R, *Rs;
@@ -214,19 +217,28 @@ struct DevPtrs {              // plain pointers handed to kernels (by value)
     int *st_pkt;              // its packet (one contribution a receiver)
     int *st_rank;             // place among the receiver's contributions, in arrival order
     int *st_bin;
-    void *st_v[10];           // T, T dx, T dy, T dz, T clock, T eps, A, A eps, w, T sigma (Real;
-                              // the last with a shared bin only)
+    void *st_v[4];            // T, T clock, A, w (Real); what else a merge takes is a product of T
+                              // or A with a value of the packet
     int *seg_cnt, *seg_off;   // per key: contributions (zero between hops) and first entry
-    int *seg_idx;             // contributions in arrival order
-    int *seg_srt;             // in packet order (st_rank's memory: ranks are read before)
-    int *seg_fill;            // scratch of the neighbour build
+    int2 *seg_ent;            // (contribution, packet), in arrival order, then in packet order
+    unsigned long long *seg_key;  // the order of the packets, in arrival order
+    int2 *seg_tmp;            // scratch of long segments (the memory of st_rank and st_pkt, which
+                              // the segments' filling reads)
     // accumulators
-    double *abs, *absE, *pass;                // [n * nf]
+    double *abs, *absE, *pass;                // [n * nf] (FP64 path only)
     unsigned long long *fx_abs, *fx_lo, *fx_E;  // [n * nf]: photons (2 words), energy
     long long *cnt;                           // CNT_N counters
     int ax_rc, ax_ec;         // index of the reception / emission direction set in c_axes*
     int *worklist;            // (particle, nu) keys a hop's receiver side has to visit
 };
+
+// what a deposit or a virtual particle reads of a particle, in one piece: its volume, n_HI and the
+// fixed-point scales of photon and energy deposits
+enum { PV_VOL, PV_NHI, PV_DEP, PV_DEPE };
+template <typename Real>
+__device__ __forceinline__ Real &pv(const DevPtrs &P, long long i, int k) {
+    return ((Real *)P.vpv)[4 * i + k];
+}
 
 // the low word of a device counter, loaded where it is used (volatile: the load is neither
 // hoisted nor kept in a register across the caller's loops)

@@ -30,11 +30,10 @@ __global__ void k_quantise(DevPtrs P, const double *x, const double *y, const do
         q[a] = (int)qq;
     }
     P.pbox[i] = lo;
-    P.qx[i] = q[0]; P.qy[i] = q[1]; P.qz[i] = q[2];
     P.q4[i] = make_int4(q[0], q[1], q[2], lo);
     double V = P.NH[i] / P.nH[i] / P.vunit[lo];   // volume in the box's volume unit
-    if (P.fp32) ((float *)P.Vr)[i] = (float)V;
-    else ((double *)P.Vr)[i] = V;
+    if (P.fp32) pv<float>(P, i, PV_VOL) = (float)V;
+    else pv<double>(P, i, PV_VOL) = V;
 }
 
 __global__ void k_quantise_src(DevPtrs P, const double *x, const double *y, const double *z) {
@@ -56,10 +55,10 @@ __global__ void k_quantise_src(DevPtrs P, const double *x, const double *y, cons
 }
 
 __device__ __forceinline__ long long cell_of_particle(const DevPtrs &P, long long i) {
-    int b = P.pbox[i];
+    const int4 q = P.q4[i];
+    int b = q.w;
     int G = P.grid.G[b], cs = P.grid.cs[b];
-    int cx = cell_coord(P.qx[i], cs, G), cy = cell_coord(P.qy[i], cs, G),
-        cz = cell_coord(P.qz[i], cs, G);
+    int cx = cell_coord(q.x, cs, G), cy = cell_coord(q.y, cs, G), cz = cell_coord(q.z, cs, G);
     return P.grid.coff[b] + ((long long)cx * G + cy) * G + cz;
 }
 
@@ -74,10 +73,10 @@ __global__ void k_cell_fill(DevPtrs P, int *fill) {
     if (i >= P.n) return;
     long long c = cell_of_particle(P, i);
     int pos = P.grid.start[c] + atomicAdd(&fill[c], 1);
-    int b = P.pbox[i];
-    const int q[3] = {P.qx[i], P.qy[i], P.qz[i]}, idx = (int)(i - P.box_off[b]);
-    P.grid.items[pos] = make_int4(q[0], q[1], q[2], idx);
-    P.grid.fitems[pos] = make_float4((float)q[0], (float)q[1], (float)q[2], __int_as_float(idx));
+    const int4 q = P.q4[i];
+    const int idx = (int)(i - P.box_off[q.w]);
+    P.grid.items[pos] = make_int4(q.x, q.y, q.z, idx);
+    P.grid.fitems[pos] = make_float4((float)q.x, (float)q.y, (float)q.z, __int_as_float(idx));
 }
 
 void knn_offset_table(int *out) {
@@ -111,8 +110,8 @@ __device__ __forceinline__ BoxGrid box_grid(const DevPtrs &P, int b) {
     return g;
 }
 
-// one warp per gas particle (exclude itself) or source
-__global__ void __launch_bounds__(256) k_knn(DevPtrs P, int sources) {
+// one warp per gas particle (exclude itself) or source; rev: senders of each particle, counted
+__global__ void __launch_bounds__(256) k_knn(DevPtrs P, int sources, int *rev) {
     __shared__ int sdelta[8][32];
     int lane = threadIdx.x & 31;
     long long nq = sources ? P.ns : P.n;
@@ -123,7 +122,8 @@ __global__ void __launch_bounds__(256) k_knn(DevPtrs P, int sources) {
         if (sources) {
             b = P.sbox[w]; qx = P.sqx[w]; qy = P.sqy[w]; qz = P.sqz[w]; ex = -1;
         } else {
-            b = P.pbox[w]; qx = P.qx[w]; qy = P.qy[w]; qz = P.qz[w];
+            const int4 q = P.q4[w];
+            b = q.w; qx = q.x; qy = q.y; qz = q.z;
             ex = (int)(w - P.box_off[b]);
         }
         long long d2;
@@ -144,21 +144,13 @@ __global__ void __launch_bounds__(256) k_knn(DevPtrs P, int sources) {
                 P.snbr[w * P.kn + lane] = (int)g;
             } else {
                 P.nbr[w * P.kn + lane] = (int)g;
-                P.fwd4[w * P.kn + lane] = make_float4((float)(P.qx[g] - qx), (float)(P.qy[g] - qy),
-                                                      (float)(P.qz[g] - qz),
-                                                      __int_as_float((int)g));
+                atomicAdd(&rev[g], 1);
             }
         }
         if (lane == 0) {
             if (sources) P.sh2[w] = kd2; else P.h2[w] = kd2;
         }
     }
-}
-
-__global__ void k_rev_count(DevPtrs P, int *cnt) {
-    long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= P.n * P.kn) return;
-    atomicAdd(&cnt[P.nbr[e]], 1);
 }
 
 __global__ void k_rev_fill(DevPtrs P, int *fill) {
@@ -168,14 +160,15 @@ __global__ void k_rev_fill(DevPtrs P, int *fill) {
     int k = (int)(e % P.kn);
     int j = P.nbr[e];
     int pos = P.rev_off[j] + atomicAdd(&fill[j], 1);
-    P.rev_ent[pos] = ((unsigned)i << 5) | (unsigned)k;
+    P.b_ent[pos] = ((unsigned)i << 5) | (unsigned)k;
 }
 
 // Order each receiver's senders by index (the fill order is arbitrary) and write the edges in
 // that order.  A warp a receiver: lanes hold 32 entries each round, and an entry's place is the
 // number of smaller ones (the entries are distinct), counted against all rounds.  Offsets come
 // from the positions (16 bytes a particle, which the L2 holds; reading them from the senders'
-// edges, 154 MB in random order, took 2.5 ms).  A thread a receiver sorted by insertion in
+// edges, 154 MB in random order, took 2.5 ms), and the places go to the edges through a list of
+// words (38 MB, likewise) that k_edges reads in order.  A thread a receiver sorted by insertion in
 // global memory before: 1328 us for 300,000 particles, 143 us now.
 __global__ void __launch_bounds__(256) k_rev_sort(DevPtrs P) {
     const int lane = threadIdx.x & 31;
@@ -185,22 +178,31 @@ __global__ void __launch_bounds__(256) k_rev_sort(DevPtrs P) {
         const int4 q = __ldg(P.q4 + j);
         for (int r0 = a; r0 < b; r0 += 32) {
             const bool on = r0 + lane < b;
-            const unsigned v = on ? P.rev_ent[r0 + lane] : 0u;
+            const unsigned v = on ? P.b_ent[r0 + lane] : 0u;
             int rank = 0;
             for (int c0 = a; c0 < b; c0 += 32) {
-                const unsigned o = c0 == r0 ? v : c0 + lane < b ? P.rev_ent[c0 + lane] : 0u;
+                const unsigned o = c0 == r0 ? v : c0 + lane < b ? P.b_ent[c0 + lane] : 0u;
                 const int m = min(32, b - c0);
                 for (int k = 0; k < m; ++k) rank += __shfl_sync(FULLMASK, o, k) < v;
             }
             if (on) {
                 const int p = a + rank, i = (int)(v >> 5);
                 const int4 s = __ldg(P.q4 + i);
-                P.revpos[(long long)i * P.kn + (v & 31u)] = p;
+                P.b_pos[(long long)i * P.kn + (v & 31u)] = p;
                 P.rev4[p] = make_float4((float)(q.x - s.x), (float)(q.y - s.y), (float)(q.z - s.z),
                                         __int_as_float(i));
             }
         }
     }
+}
+
+// the forward edges: offset and place in the reverse lists, in one piece
+__global__ void k_edges(DevPtrs P) {
+    long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= P.n * P.kn) return;
+    const int4 q = __ldg(P.q4 + P.nbr[e]), s = __ldg(P.q4 + (unsigned)e / (unsigned)P.kn);
+    P.fwd4[e] = make_float4((float)(q.x - s.x), (float)(q.y - s.y), (float)(q.z - s.z),
+                            __int_as_float(P.b_pos[e]));
 }
 
 // Timing probe of the occupancy search: the kNN search of virtual-particle-like points, one
@@ -214,7 +216,8 @@ __global__ void __launch_bounds__(256) k_knn_probe(DevPtrs P, unsigned long long
     unsigned long long acc = 0;
     for (long long w = w0; 4 * w < P.n; w += nw) {
         long long i = 4 * w;
-        int b = P.pbox[i];
+        const int4 q = P.q4[i];
+        int b = q.w;
         long long H = (long long)sqrt((double)P.h2[i]);
         unsigned long long hsh = mix64((unsigned long long)i);
         int o[3];
@@ -222,9 +225,9 @@ __global__ void __launch_bounds__(256) k_knn_probe(DevPtrs P, unsigned long long
             int u = (int)((hsh >> (16 * a)) & 0xffff) - 32768;       // in [-2^15, 2^15)
             o[a] = (int)((long long)u * (H / 4) / 32768);             // |o| < 0.44 H
         }
-        int qx = min(max(P.qx[i] + o[0], 0), RT_Q - 1);
-        int qy = min(max(P.qy[i] + o[1], 0), RT_Q - 1);
-        int qz = min(max(P.qz[i] + o[2], 0), RT_Q - 1);
+        int qx = min(max(q.x + o[0], 0), RT_Q - 1);
+        int qy = min(max(q.y + o[1], 0), RT_Q - 1);
+        int qz = min(max(q.z + o[2], 0), RT_Q - 1);
         long long d2;
         int idx;
         CandQuery Q = cand_query(P.grid, b, qx, qy, qz);
@@ -359,9 +362,10 @@ __global__ void __launch_bounds__(256) k_cand_count(DevPtrs P, long long *u2out,
         long long u2 = 0;
         if (ok && lane < P.kn) {
             long long j = P.box_off[b] + idx;
-            long long ex = max(P.qx[j] - lx, lx + cs - 1 - P.qx[j]);
-            long long ey = max(P.qy[j] - ly, ly + cs - 1 - P.qy[j]);
-            long long ez = max(P.qz[j] - lz, lz + cs - 1 - P.qz[j]);
+            const int4 q = P.q4[j];
+            long long ex = max(q.x - lx, lx + cs - 1 - q.x);
+            long long ey = max(q.y - ly, ly + cs - 1 - q.y);
+            long long ez = max(q.z - lz, lz + cs - 1 - q.z);
             u2 = ex * ex + ey * ey + ez * ez;
         }
 #pragma unroll
@@ -448,7 +452,7 @@ static void cell_lists(rt_ctx *c, cudaStream_t st) {
     DevPtrs &P = c->d;
     int tb = 256;
     unsigned nbk = (unsigned)((P.n + tb - 1) / tb);
-    int *cnt = P.seg_cnt, *fill = P.seg_fill;   // scratch, sized >= max(ncells, n)
+    int *cnt = P.seg_cnt, *fill = P.b_fill;   // scratch, sized >= max(ncells, n)
     cudaMemsetAsync(cnt, 0, sizeof(int) * (P.grid.ncells + 1), st);
     cudaMemsetAsync(fill, 0, sizeof(int) * (P.grid.ncells + 1), st);
     k_cell_count<<<nbk, tb, 0, st>>>(P, cnt);
@@ -541,22 +545,21 @@ rt_status rt_knn_build(rt_ctx *c, cudaStream_t st) {
     DevPtrs &P = c->d;
     long long n = P.n;
     int tb = 256;
-    unsigned nbk = (unsigned)((n + tb - 1) / tb);
-    int *cnt = P.seg_cnt, *fill = P.seg_fill;
+    int *cnt = P.seg_cnt, *fill = P.b_fill;
     // cell lists
     cell_lists(c, st);
     // neighbours of particles and sources
-    k_knn<<<rt_blocks(n * 32, tb, 152 * 64), tb, 0, st>>>(P, 0);
-    if (P.ns > 0) k_knn<<<rt_blocks((long long)P.ns * 32, tb), tb, 0, st>>>(P, 1);
-    // reverse lists
     cudaMemsetAsync(cnt, 0, sizeof(int) * (n + 1), st);
+    k_knn<<<rt_blocks(n * 32, tb, 152 * 64), tb, 0, st>>>(P, 0, cnt);
+    if (P.ns > 0) k_knn<<<rt_blocks((long long)P.ns * 32, tb), tb, 0, st>>>(P, 1, nullptr);
+    // reverse lists
     cudaMemsetAsync(fill, 0, sizeof(int) * (n + 1), st);
     long long ne = n * P.kn;
     unsigned nbe = (unsigned)((ne + tb - 1) / tb);
-    k_rev_count<<<nbe, tb, 0, st>>>(P, cnt);
     rt_scan_exclusive(c, cnt, P.rev_off, n + 1, st);
     k_rev_fill<<<nbe, tb, 0, st>>>(P, fill);
     k_rev_sort<<<rt_blocks(n * 32, tb, 152 * 32), tb, 0, st>>>(P);
+    k_edges<<<nbe, tb, 0, st>>>(P);
     rt_status s = rt_cuda_check(c, cudaGetLastError(), "neighbour build");
     if (s != RT_OK) return s;
     // the virtual particles' candidate lists, on the grid the occupancy search picks (it needs

@@ -432,21 +432,15 @@ __global__ void k_emit_rec(DevPtrs P, int *lens, int np) {
     }
     if (i >= P.n) return;
     int cur = (int)P.cnt[CNT_CUR];
-    int b = P.pbox[i];
-    double nm = P.norm[b];
+    double nm = P.norm[P.pbox[i]];
     double x = P.xHI[i], nH = P.nH[i], NH = P.NH[i];
     double nHI = __dmul_rn(x, nH);
     P.nHI[i] = nHI;
-    ((Real *)P.nHIr)[i] = (Real)nHI;
     double NHI = x * NH;
-    ((Real *)P.dep_s)[i] = NHI > 0.0 ? (Real)(FX_ABS_SCALE * nm / NHI) : Real(0);
-    ((Real *)P.depE_s)[i] = NHI > 0.0 ? (Real)(FX_E_SCALE * nm * P.eunit / (NHI * EV_ERG)) : Real(0);
-    // the four a virtual particle reads of a neighbour, in one piece
-    Real *pv = (Real *)P.vpv + 4 * i;
-    pv[0] = ((Real *)P.Vr)[i];
-    pv[1] = (Real)nHI;
-    pv[2] = ((Real *)P.dep_s)[i];
-    pv[3] = ((Real *)P.depE_s)[i];
+    ((Real *)P.nHIr)[i] = (Real)nHI;
+    pv<Real>(P, i, PV_NHI) = (Real)nHI;
+    pv<Real>(P, i, PV_DEP) = NHI > 0.0 ? (Real)(FX_ABS_SCALE * nm / NHI) : Real(0);
+    pv<Real>(P, i, PV_DEPE) = NHI > 0.0 ? (Real)(FX_E_SCALE * nm * P.eunit / (NHI * EV_ERG)) : Real(0);
     double Nr = P.Nrec[i];
     if (!(Nr > 0.0) || P.rec_mode == RT_REC_EMISSION_CONES) return;
     double e_phys = Nr / (double)NRC;
@@ -555,7 +549,8 @@ __global__ void k_emit_rec_cones(DevPtrs P, long long base) {
     int k = (int)((p % per) / P.nec), e = (int)(p % P.nec);
     FreeBuf F = P.fr[0];
     long long f = base + p;
-    int b = P.pbox[i];
+    const int4 q = P.q4[i];
+    const int b = q.w;
     double Nr = P.Nrec[i];
     double N = Nr > 0.0 ? __ddiv_rn(Nr, (double)per) : 0.0;
     double R[9], d[3];
@@ -563,7 +558,7 @@ __global__ void k_emit_rec_cones(DevPtrs P, long long base) {
     random_rotation(P.seed, 4u, (unsigned)step, (unsigned)k, (unsigned)gi, R);
     rot_apply(R, c_axd[P.ax_ec] + 3 * e, d);
     F.box[f] = b;
-    F.qx[f] = P.qx[i]; F.qy[f] = P.qy[i]; F.qz[f] = P.qz[i];
+    F.qx[f] = q.x; F.qy[f] = q.y; F.qz[f] = q.z;
     for (int a = 0; a < P.kn; ++a) F.nbr[f * P.kn + a] = P.nbr[i * P.kn + a];
     F.h2[f] = P.h2[i];
     ((Real *)F.N)[f] = (Real)(N / P.norm[b]);
@@ -678,8 +673,9 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int c
         const unsigned incl = lane_scan(cnt);
         const int total = (int)__shfl_sync(FULLMASK, incl, 31);
         // the current particle's neighbour of this lane, and the next one's
-        float4 ed = make_float4(0.f, 0.f, 0.f, 0.f), edn = ed;
-        int rp = 0, rpn = 0;
+        float ex = 0.f, ey = 0.f, ez = 0.f;   // offset, place in the reverse lists, index
+        int rp = 0, nb = 0, nbn = 0;
+        float4 edn = make_float4(0.f, 0.f, 0.f, 0.f);
         float ir = 0.f;
         bool valid = false;
         int curp = -1;                    // the current particle (of the turn's)
@@ -689,13 +685,13 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int c
             if (lane < P.kn) {
                 long long f = (ic + p) * P.kn + lane;
                 edn = __ldg(P.fwd4 + f);
-                rpn = __ldg(P.revpos + f);
+                nbn = __ldg(P.nbr + f);
             }
         };
         auto flush = [&]() {
             if (word) {
                 P.bm[(long long)wnu * nrev + rp] = word;
-                P.touched[(long long)__float_as_int(ed.w) * P.nf + wnu] = 1;
+                P.touched[(long long)nb * P.nf + wnu] = 1;
             }
             word = 0u;
         };
@@ -733,26 +729,27 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseA(DevPtrs P, int c
             for (int t = 0; t < nk; ++t) {
                 if ((first >> t) & 1u) {
                     flush();
-                    ed = edn;
-                    rp = rpn;
+                    ex = edn.x; ey = edn.y; ez = edn.z;
+                    rp = __float_as_int(edn.w);
+                    nb = nbn;
                     curp = __shfl_sync(FULLMASK, op, t);
                     wnu = -1;
-                    valid = lane < P.kn && (ed.x != 0.f || ed.y != 0.f || ed.z != 0.f);
-                    ir = rsqrtf(__fmaf_rn(ed.x, ed.x, __fmaf_rn(ed.y, ed.y, ed.z * ed.z)));
+                    valid = lane < P.kn && (ex != 0.f || ey != 0.f || ez != 0.f);
+                    ir = rsqrtf(__fmaf_rn(ex, ex, __fmaf_rn(ey, ey, ez * ez)));
                     unsigned later = first & (0xfffffffeu << t);
                     if (later) fetch(__shfl_sync(FULLMASK, op, __ffs(later) - 1));
                 }
                 const float e0 = __shfl_sync(FULLMASK, f0, t), e1 = __shfl_sync(FULLMASK, f1, t),
                             e2 = __shfl_sync(FULLMASK, f2, t);
                 const int unu = __shfl_sync(FULLMASK, onu, t), ub = __shfl_sync(FULLMASK, ob, t);
-                const float cs = __fmaf_rn(ed.x, e0, __fmaf_rn(ed.y, e1, ed.z * e2)) * ir;
+                const float cs = __fmaf_rn(ex, e0, __fmaf_rn(ey, e1, ez * e2)) * ir;
                 bool in = valid && cs > cf + CONE_BAND;
                 const bool amb = valid && !in && !(cs < cf - CONE_BAND);
                 if (__any_sync(FULLMASK, amb)) {   // inside the guard band: the exact test
                     const Real x0 = __shfl_sync(FULLMASK, K.d0, t), x1 = __shfl_sync(FULLMASK, K.d1, t),
                                x2 = __shfl_sync(FULLMASK, K.d2, t);
                     if (amb)
-                        in = cone_exact((int)ed.x, (int)ed.y, (int)ed.z, (double)x0, (double)x1,
+                        in = cone_exact((int)ex, (int)ey, (int)ez, (double)x0, (double)x1,
                                         (double)x2, P.ntc);
                 }
                 const unsigned m = __ballot_sync(FULLMASK, in);
@@ -857,7 +854,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_free(DevPtrs P, int fcu
             const Real N = ((Real *)F.N)[f];
             const Real w = N / (Real)(int)((mw >> 27) + 1u);
             const Real d0 = ((Real *)F.dx)[f], d1 = ((Real *)F.dy)[f], d2 = ((Real *)F.dz)[f];
-            const Real clk = ((Real *)F.clock)[f], eps = ((Real *)F.eps)[f];
+            const Real clk = ((Real *)F.clock)[f];
             const int nu = F.nu[f];
             // the packet's cross-section: its own mean in a shared bin, else its bin's
             const bool sgs = SH && nu == 0;
@@ -882,15 +879,9 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_free(DevPtrs P, int fcu
                 split_absorbed<Real>(w, tau, A, T);
                 bt = bin_fast<Real>(P.Rf + j * 9, P.R + j * 9, P.ax_rc, NRC, d0, d1, d2);
                 V[0][s] = T;
-                V[1][s] = T * d0;
-                V[2][s] = T * d1;
-                V[3][s] = T * d2;
-                V[4][s] = T * (clk + light_time(l));
-                V[5][s] = T * eps;
-                V[6][s] = A;
-                V[7][s] = A * eps;
-                V[8][s] = w;
-                if (sgs) V[9][s] = T * sg;
+                V[1][s] = T * (clk + light_time(l));
+                V[2][s] = A;
+                V[3][s] = w;
             }
             P.st_bin[s] = bt;
             P.st_rank[s] = atomicAdd(&P.seg_cnt[key], 1);
@@ -1124,8 +1115,9 @@ __global__ void __launch_bounds__(256, VIRT_MINB(Real)) k_virtual(DevPtrs P, int
                 long long i = (unsigned)code / (unsigned)P.S;   // slot codes < 2^31
                 int s = (int)((unsigned)code % (unsigned)P.S);
                 D.nu = s / NRC;
-                D.box = P.pbox[i];
-                D.qx = P.qx[i]; D.qy = P.qy[i]; D.qz = P.qz[i];
+                const int4 q = P.q4[i];
+                D.box = q.w;
+                D.qx = q.x; D.qy = q.y; D.qz = q.z;
                 D.h2 = P.h2[i];
                 D.N = S.N[code];
                 packet_dir(S.X[code], S.Y[code], S.Z[code], D.d0, D.d1, D.d2);
@@ -1475,13 +1467,18 @@ __global__ void __launch_bounds__(256) k_worklist(DevPtrs P, int cur, int *lens)
     }
 }
 
-// the staged contributions into their receivers' segments
-__global__ void __launch_bounds__(256) k_seg_fill(DevPtrs P, const int *lens) {
+// the staged contributions into their receivers' segments, with the order of their packets
+__global__ void __launch_bounds__(256) k_seg_fill(DevPtrs P, int fcur, const int *lens) {
     long long nst = lens[3];
     if (nst > P.ST_cap) nst = P.ST_cap;
     for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < nst;
-         s += (long long)gridDim.x * blockDim.x)
-        P.seg_idx[P.seg_off[P.st_key[s]] + P.st_rank[s]] = (int)s;
+         s += (long long)gridDim.x * blockDim.x) {
+        const int key = P.st_key[s], rank = P.st_rank[s], f = P.st_pkt[s];
+        const unsigned long long order = P.fr[fcur].okey[f];   // (loaded beside the offset)
+        const int pos = P.seg_off[key] + rank;
+        P.seg_ent[pos] = make_int2((int)s, f);
+        P.seg_key[pos] = order;
+    }
 }
 
 // absorptions of one receiver group in one hop.  FP64 path: FP64 sums.  FP32 path: the
@@ -1511,7 +1508,7 @@ __device__ __forceinline__ unsigned long long deposit_group<float>(const DevPtrs
                                                                    float w) {
     // atomics: virtual-particle deposits into the same words may run at the same time
     unsigned long long old = 0ull;
-    float fa = a * ((float *)P.dep_s)[j];
+    float fa = a * pv<float>(P, j, PV_DEP);
     if (fa > 0.0f) {
         unsigned long long qh, ql;
         if (fx_split(fa, qh, ql)) {
@@ -1521,7 +1518,7 @@ __device__ __forceinline__ unsigned long long deposit_group<float>(const DevPtrs
             atomicOr((unsigned long long *)&P.cnt[CNT_ERR], (unsigned long long)ERRB_RANGE);
         }
     }
-    float fe = ae * ((float *)P.depE_s)[j];
+    float fe = ae * pv<float>(P, j, PV_DEPE);
     if (fe > 0.0f) atomicAdd(&P.fx_E[key], f2u64_rz(fe + 0.5f));
     P.passf[key] += w;
     return old;
@@ -1544,9 +1541,9 @@ __device__ __forceinline__ int gas_contribution(const DevPtrs &P, long long e, i
     rec_load(P.rec, (long long)__float_as_int(ed.w) * P.S + (long long)nu * G + b, w, d0, d1, d2,
              clk, eps, sgs, sgc);
     if (BAR) {
-        int jx = P.qx[j], jy = P.qy[j], jz = P.qz[j];
-        if (barrier_crosses_call(P.bar[box], jx - (int)ed.x, jy - (int)ed.y, jz - (int)ed.z, jx,
-                                 jy, jz)) {
+        const int4 q = P.q4[j];
+        if (barrier_crosses_call(P.bar[box], q.x - (int)ed.x, q.y - (int)ed.y, q.z - (int)ed.z, q.x,
+                                 q.y, q.z)) {
             atomicAdd(&P.esc_fx[box], esc_fixed(w, P, box));
             return -1;
         }
@@ -1565,37 +1562,41 @@ __device__ __forceinline__ int gas_contribution(const DevPtrs &P, long long e, i
     return bin_fast<Real>(P.Rf + j * 9, P.R + j * 9, P.ax_rc, G, d0, d1, d2);
 }
 
-// A staged free-packet contribution: its values into sv[.][lane], its cone (-1: removed).
+// A staged contribution (e.x) of a packet (e.y) of free buffer fcur: its values into sv[.][lane], its cone
+// (-1: removed).
 template <typename Real, bool SH>
-__device__ __forceinline__ int staged_contribution(const DevPtrs &P, int s, int nu,
+__device__ __forceinline__ int staged_contribution(const DevPtrs &P, int fcur, int2 e, int nu,
                                                    Pair<Real> (*sv)[32], int lane) {
     Real *const *V = (Real *const *)P.st_v;
-    int bin = P.st_bin[s];
+    const int s = e.x, f = e.y, bin = P.st_bin[s];
     if (bin >= 0) {
-#pragma unroll
-        for (int f = 0; f < 4; ++f) sv[f][lane] = make_pair2(V[2 * f][s], V[2 * f + 1][s]);
-        sv[4][lane] = make_pair2(V[8][s], SH && nu == 0 ? V[9][s] : Real(0));
+        const FreeBuf &F = P.fr[fcur];
+        const Real T = V[0][s], A = V[2][s], eps = ((Real *)F.eps)[f];
+        sv[0][lane] = make_pair2(T, T * ((Real *)F.dx)[f]);
+        sv[1][lane] = make_pair2(T * ((Real *)F.dy)[f], T * ((Real *)F.dz)[f]);
+        sv[2][lane] = make_pair2(V[1][s], T * eps);
+        sv[3][lane] = make_pair2(A, A * eps);
+        sv[4][lane] = make_pair2(V[3][s], SH && nu == 0 ? T * ((Real *)F.sig)[f] : Real(0));
     }
     return bin;
 }
 
-// A segment of n > 8 contributions from idx into srt in packet order, by the whole warp: blocks of
-// 32 by counting earlier packets (distinct), then sorted runs merged in pairs, an entry's place
-// being its place in its run and the earlier ones of the other (binary search).  The passes
-// alternate between idx and srt and end in srt.  Counting the earlier packets of the whole segment,
-// without the merges, is quadratic: 20,000 sources within one smoothing length give their
-// neighbours segments of 20,000, and a step of a 32^3 box took 2.1 s (FP32), 48 ms now; with 4,096
-// sources 96 and 12 ms.
-__device__ void order_wide(const unsigned long long *okey, const int *pkt, int *idx, int *srt,
-                           unsigned n) {
+// A segment of n > 8 contributions brought into packet order by the whole warp: blocks of 32 by
+// counting earlier packets (distinct), then sorted runs merged in pairs, an entry's place being its
+// place in its run and the earlier ones of the other (binary search).  The passes alternate
+// between ent and tmp and end in ent.  Counting the earlier packets of the whole segment, without
+// the merges, is quadratic: 20,000 sources within one smoothing length give their neighbours
+// segments of 20,000, and a step of a 32^3 box took 2.1 s (FP32), 35 ms now; with 4,096 sources 96
+// and 9 ms.
+__device__ void order_wide(const unsigned long long *okey, int2 *ent, int2 *tmp, unsigned n) {
     const unsigned lane = threadIdx.x & 31u;
     bool odd = false;                  // number of merge passes
     for (unsigned L = 32; L < n; L *= 2) odd = !odd;
-    int *a = odd ? idx : srt, *b = odd ? srt : idx;
+    int2 *a = odd ? tmp : ent, *b = odd ? ent : tmp;
     for (unsigned c = 0; c < n; c += 32) {
         const bool on = c + lane < n;
-        const int s = on ? idx[c + lane] : 0;
-        const unsigned long long key = on ? okey[pkt[s]] : ~0ull;
+        const int2 s = on ? ent[c + lane] : make_int2(0, 0);
+        const unsigned long long key = on ? okey[s.y] : ~0ull;
         int r = 0;
         for (int k = 0; k < 32; ++k) r += __shfl_sync(FULLMASK, key, k) < key;
         if (on) a[c + r] = s;
@@ -1603,44 +1604,48 @@ __device__ void order_wide(const unsigned long long *okey, const int *pkt, int *
     __syncwarp();
     for (unsigned L = 32; L < n; L *= 2) {
         for (unsigned t = lane; t < n; t += 32) {
-            const int s = a[t];
-            const unsigned long long key = okey[pkt[s]];
+            const int2 s = a[t];
+            const unsigned long long key = okey[s.y];
             const unsigned run = t & ~(L - 1u), other = run ^ L;
             unsigned lo = min(other, n), hi = min(other + L, n);
             const unsigned o0 = lo;
             while (lo < hi) {
                 const unsigned m = (lo + hi) >> 1;
-                if (okey[pkt[a[m]]] < key) lo = m + 1u;
+                if (okey[a[m].y] < key) lo = m + 1u;
                 else hi = m;
             }
             b[min(run, other) + (t - run) + (lo - o0)] = s;
         }
         __syncwarp();
-        int *x = a;
+        int2 *x = a;
         a = b;
         b = x;
     }
 }
 
-// The four segments of a warp (n contributions each, lanes of eight hold the same) from idx into
-// srt in packet order.  Up to eight: a lane an entry, all four at once.  Out of line: few groups
-// have any, and inlined it costs the receiver side registers.
-static __device__ __noinline__ void order_segments(const unsigned long long *okey, const int *pkt,
-                                                   int *idx, int *srt, int n) {
-    const int lane = threadIdx.x & 31, l = lane & 7;
-    const bool on = n <= 8 && l < n;
-    const int s = on ? idx[l] : 0;
-    const unsigned long long key = on && n > 1 ? okey[pkt[s]] : ~0ull;
-    int r = 0;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) r += __shfl_sync(FULLMASK, key, k, 8) < key;
-    if (on) srt[r] = s;
-    for (unsigned w = __ballot_sync(FULLMASK, n > 8 && l == 0); w; w &= w - 1u) {
+// the four segments of a warp (n contributions each, lanes of eight hold the same): those of more
+// than eight, one after the other
+static __device__ __noinline__ void order_long(const unsigned long long *okey, int2 *ent, int2 *tmp,
+                                               int n) {
+    for (unsigned w = __ballot_sync(FULLMASK, n > 8 && (threadIdx.x & 7) == 0); w; w &= w - 1u) {
         const int k = __ffs(w) - 1;
-        order_wide(okey, pkt, (int *)__shfl_sync(FULLMASK, (unsigned long long)idx, k),
-                   (int *)__shfl_sync(FULLMASK, (unsigned long long)srt, k),
+        order_wide(okey, (int2 *)__shfl_sync(FULLMASK, (unsigned long long)ent, k),
+                   (int2 *)__shfl_sync(FULLMASK, (unsigned long long)tmp, k),
                    (unsigned)__shfl_sync(FULLMASK, n, k));
     }
+}
+
+// those of up to eight, all at once: a lane an entry.  Out of line: few groups have any, and inlined
+// it costs the receiver side registers.
+static __device__ __noinline__ void order_segments(const unsigned long long *key, int2 *ent, int n) {
+    const int l = threadIdx.x & 7;
+    const bool on = n <= 8 && l < n;
+    const int2 s = on ? ent[l] : make_int2(0, 0);
+    const unsigned long long v = on ? key[l] : ~0ull;
+    int r = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) r += __shfl_sync(FULLMASK, v, k, 8) < v;
+    if (on) ent[r] = s;
     __syncwarp();
 }
 
@@ -1696,8 +1701,8 @@ __device__ __forceinline__ unsigned byte_popc(unsigned x) {
 // edges, contributions and waiting packets: edges 32 at a time, contributions 32 at a time,
 // each cone's lane adding its contributions in list order.
 template <typename Real, bool BAR, bool SH>
-__device__ __forceinline__ void wide_group(const DevPtrs &P, int cur, long long key, bool touched,
-                                           int fc, int so, Pair<Real> (*sv)[32], unsigned *list,
+__device__ __forceinline__ void wide_group(const DevPtrs &P, int cur, int fcur, long long key,
+                                           bool touched, int fc, int so, Pair<Real> (*sv)[32], unsigned *list,
                                            unsigned *smask, unsigned long long &pend, bool &bad,
                                            int *stot) {
     const int lane = threadIdx.x & 31;
@@ -1760,7 +1765,7 @@ __device__ __forceinline__ void wide_group(const DevPtrs &P, int cur, long long 
     for (int cb = 0; cb < fc; cb += 32) {
         int bin = -1;
         if (cb + lane < fc)
-            bin = staged_contribution<Real, SH>(P, P.seg_srt[so + cb + lane], nu, sv, lane);
+            bin = staged_contribution<Real, SH>(P, fcur, P.seg_ent[so + cb + lane], nu, sv, lane);
         merge(bin);
     }
     const Real N = a.photons();
@@ -1854,7 +1859,9 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int c
         const Real sig_nhi = sigma_of<Real>(P, nu) * ((Real *)P.nHIr)[j];
         Slots<Real> So(P, cur), Sn(P, nxt);
         if (__any_sync(FULLMASK, fc > 0)) {
-            order_segments(P.fr[fcur].okey, P.st_pkt, P.seg_idx + so, P.seg_srt + so, fc);
+            order_segments(P.seg_key + so, P.seg_ent + so, fc);
+            if (__any_sync(FULLMASK, fc > 8))
+                order_long(P.fr[fcur].okey, P.seg_ent + so, P.seg_tmp + so, fc);
             if ((lane & 7) == 0 && fc > 0) P.seg_cnt[key] = 0;   // for the next hop
         }
         // a group's values to the lanes that work on it
@@ -1968,7 +1975,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int c
                 const int c = p - (kk == 0 ? 0 : kk == 1 ? f1 : kk == 2 ? f2 : f3);
                 const int sok = of(so, kk), nuk = of(nu, kk);
                 int bin = -1;
-                if (p < ft) bin = staged_contribution<Real, SH>(P, P.seg_srt[sok + c], nuk, sv, lane);
+                if (p < ft) bin = staged_contribution<Real, SH>(P, fcur, P.seg_ent[sok + c], nuk, sv, lane);
                 merge(kk, bin, c & 7);
             }
             // the merged packets
@@ -2037,7 +2044,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int c
                         k1 = kk + 1;
                     }
                 if (k1 == k0) {
-                    wide_group<Real, BAR, SH>(P, cur, of(key, k0), of((int)touched, k0) != 0,
+                    wide_group<Real, BAR, SH>(P, cur, fcur, of(key, k0), of((int)touched, k0) != 0,
                                               of(fc, k0), of(so, k0), sv, list, smask[wid][0], pend,
                                               bad, stot);
                     ++k0;
@@ -2082,7 +2089,7 @@ __global__ void __launch_bounds__(256, HOP_MINB(Real)) k_phaseB(DevPtrs P, int c
                     bin = gas_contribution<Real, G, BAR, SH>(P, (long long)e0k + ((code >> 5) & 63u),
                                                              code & 31u, jk, nuk, boxk, uk, snk, sv, lane);
                 else if (lane < n)
-                    bin = staged_contribution<Real, SH>(P, P.seg_srt[sok + ec], nuk, sv, lane);
+                    bin = staged_contribution<Real, SH>(P, fcur, P.seg_ent[sok + ec], nuk, sv, lane);
                 __syncwarp();
                 // the lowest lane of each (group, cone) adds its contributions in list order
                 const unsigned live = __ballot_sync(FULLMASK, bin >= 0);
@@ -2317,7 +2324,7 @@ static void hop_core(rt_ctx *c, cudaStream_t st, long long nfr, int cur, int fcu
     cudaEventRecord(evA, st);
     cudaStreamWaitEvent(s2, evA, 0);
     LAUNCH_ON(s2, KT_WORKLIST, 1, (k_worklist<<<rt_blocks(nkey, 1024, 152 * 8), tb, 0, s2>>>(P, cur, H.lens)));
-    LAUNCH_ON(s2, KT_SEG_FILL, 1, (k_seg_fill<<<rt_blocks(nfr * 2, tb, 152 * 8), tb, 0, s2>>>(P, H.lens)));
+    LAUNCH_ON(s2, KT_SEG_FILL, 1, (k_seg_fill<<<rt_blocks(nfr * 2, tb, 152 * 8), tb, 0, s2>>>(P, fcur, H.lens)));
     cudaStreamWaitEvent(st, evFree, 0);
     const int nbb = rt_blocks(nkey * 8, tb, GB);
     if (P.shared)
