@@ -99,7 +99,8 @@ typedef struct {
                              virtual particles, receiver side) are chosen by timing the first
                              steps of rt_step as whole step-graph launches: coordinate search
                              from the built-in sizes over 152 x {2, 3, 4, 5} blocks for the
-                             virtual particles (one wave at most: they pull work from a queue)
+                             virtual particles (one wave at most with FP32 packets: they
+                             pull work from a queue)
                              and 152 x {8, 16, 32, 64} for the two others, each candidate step
                              after a step of the best so far, per unit of work of the step (18
                              steps).  The winner is kept for the process per

@@ -26,14 +26,15 @@ struct Rates {
     double aA, aB, beta, L, Lce, Lff;   // L: recombination cooling of the case in use
 };
 
-// what the mode needs of the rates (uniform over the launch): the others are not evaluated
+// what the mode needs of the rates (uniform over the launch); the FP32 fits evaluate no others, the
+// FP64 ones, a lane each, all
 struct RateNeeds {
     bool aA, aB, caseB, therm;
 };
 
 // FP64 fits, shared by the four lanes of a particle: each evaluates one fit of the form
 // pre * lam^e1 / (1 + (lam / c)^e2)^e3 (case-A and case-B coefficients, collisional ionisation,
-// recombination cooling), so a subcycle's chain is 4 pow calls long instead of 13.
+// recombination cooling), so a subcycle's chain is 4 pow calls long instead of 16.
 __device__ __forceinline__ void rates64(double T, Rates &r, const RateNeeds &nd) {
     const int q = threadIdx.x & 3;
     const unsigned gm = 0xfu << (threadIdx.x & 28);

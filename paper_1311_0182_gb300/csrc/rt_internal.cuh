@@ -41,7 +41,6 @@ enum {
     CNT_ERR = 4,        // sticky error bits
     CNT_VIRT = 5,       // virtual particles this step
     CNT_VESC = 6,       // escaped virtual particles this step
-    CNT_GAS = 7,        // gas-to-gas contributions this step
     CNT_SUB = 8,        // chemistry subcycles
     CNT_FLOOR = 9,      // subcycle-floor hits
     CNT_CHEMQ = 10,     // the chemistry's work queue: particles taken
@@ -397,9 +396,11 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
     return z ^ (z >> 31);
 }
 
-// a / b, correctly rounded, from y = the correctly rounded 1 / b: quotient estimate, exact
-// remainder, one correction (Markstein 1990, IBM J. Res. Dev. 34, 111).  For operands whose
-// quotient and remainder neither overflow nor underflow.
+// a / b, correctly rounded, from y = the correctly rounded 1 / b: quotient estimate, remainder, one
+// correction (Markstein 1990, IBM J. Res. Dev. 34, 111).  For operands whose quotient and
+// remainder neither overflow nor underflow.  The theorem is stated for an estimate within one unit
+// in the last place; a y can be 1.5 off where a's mantissa is below b's.  The steps give the rounded
+// quotient there too: for every pair of mantissas at 3 to 13 bits, and in all 3e8 random FP64 pairs.
 __device__ __forceinline__ double div_by_rcp(double a, double b, double y) {
     double q = __dmul_rn(a, y);
     return __fma_rn(__fma_rn(-q, b, a), y, q);
@@ -473,21 +474,11 @@ static __device__ __noinline__ bool cone_exact(int dx, int dy, int dz, double d0
     return xmul(t, t) >= xmul(xmul(c, c), (double)r2i);
 }
 
-// Fast FP32 test with a guard band; falls back to the exact test inside the band.  The
-// FP32 cosine estimate is within ~1e-6 of the exact value, far inside the 2e-5 band.
+// Guard band of the hop kernels' cone test.  They estimate the cosine in FP32 (fused products times
+// rsqrtf, within ~1e-6 of the exact value): above cf + band inside the cone, below cf - band
+// outside, between the two cone_exact decides.  Conversions of FP64 directions, which run on the
+// FP64 pipe, happen there only.
 #define CONE_BAND 2e-5f
-// (the direction comes in the packet's own precision; conversions to FP64 run on the FP64
-// pipe, so they happen only inside the band)
-template <typename Real>
-__device__ __forceinline__ bool cone_test(int dx, int dy, int dz, float fx, float fy, float fz,
-                                          Real d0, Real d1, Real d2, float cf, int ntc) {
-    if ((dx | dy | dz) == 0) return false;
-    float r2 = __fmaf_rn(fx, fx, __fmaf_rn(fy, fy, fz * fz));
-    float cs = __fmaf_rn(fx, (float)d0, __fmaf_rn(fy, (float)d1, fz * (float)d2)) * rsqrtf(r2);
-    if (cs > cf + CONE_BAND) return true;
-    if (cs < cf - CONE_BAND) return false;
-    return cone_exact(dx, dy, dz, (double)d0, (double)d1, (double)d2, ntc);
-}
 
 // Reception cone of direction d at a particle with rotation R: argmax_b (R^T d) . D_b,
 // first maximum on ties.  Exact (FP64) form.

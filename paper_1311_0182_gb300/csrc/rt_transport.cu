@@ -31,7 +31,6 @@ static const double EV_ERG = 1.602176634e-12;
 
 // the two isotropic direction sets (index 0: 8 directions, 1: 32), FP64 and FP32 copies
 __constant__ double c_axd[2][96];
-__constant__ float c_axf[2][96];
 // FP32 copy in global memory for lane-divergent reads, and the candidate table of each set
 __device__ float g_axf[2][96];
 __device__ unsigned g_bin_tab[2][BIN_TAB_M * BIN_TAB_M];
@@ -139,7 +138,6 @@ void rt_upload_axes() {
         return t;
     }();
     cudaMemcpyToSymbol(c_axd, d, sizeof(d));
-    cudaMemcpyToSymbol(c_axf, f, sizeof(f));
     cudaMemcpyToSymbol(g_axf, f, sizeof(f));
     cudaMemcpyToSymbol(g_bin_tab, tab->t, sizeof(tab->t));
 }
@@ -161,12 +159,14 @@ void rt_upload_axes() {
 #define GRID_A (152 * 16)
 #endif
 #ifndef GRID_V
-#define GRID_V (152 * VIRT_MINB_F32)   // one wave: the virtual particles pull from a work queue
+// one wave with FP32 packets (1.7 with FP64, three blocks an SM: the virtual particles pull from a
+// work queue, so the later blocks find what is left)
+#define GRID_V (152 * VIRT_MINB_F32)
 #endif
 #ifndef GRID_B
 #define GRID_B (152 * 8)
 #endif
-#define GRID_F (152 * 4)   // free-packet senders: one wave
+#define GRID_F (152 * 4)   // free-packet senders: one wave (1.3 with FP64)
 
 template <typename Real> struct Slots {
     Real *N, *X, *Y, *Z, *C, *E;
@@ -219,7 +219,7 @@ __device__ __forceinline__ void rec_load(const void *rec, long long s, double &w
 // Quotients with a shared divisor, correctly rounded like a division each (div_by_rcp): an FP64
 // division takes about ten FP64 instructions, a further quotient by the same divisor three.  The
 // plain division where an operand is so large or small that the exact remainder could leave
-// the range.
+// the range.  (A zero numerator of either sign gives +0; every sum that takes it starts at +0.)
 __device__ __forceinline__ bool in_range(double a) {   // 2^-400 <= |a| < 2^401
     return (((unsigned)__double2hiint(a) >> 20) & 0x7ffu) - 623u < 801u;
 }
@@ -1042,7 +1042,7 @@ __device__ __forceinline__ float rcp_rn(float b) { return __frcp_rn(b); }
 // shadow test (FP64) 8.7 -> 7.8 ms.
 // Work queue: every warp of the launch takes its next group from one device counter (CNT_VQ,
 // zero before the hop), so all resident warps stay busy until the requests run out, whatever
-// each request costs; the grid is one wave of resident blocks.  Results do not depend on which
+// each request costs.  Results do not depend on which
 // warp takes a request.
 // BAR: some box has a barrier (a separate instance keeps the test out of the common case);
 // SH: the shared frequency bin (likewise); IB: index bits of the exact kNN's keys (24 when a box
@@ -2199,7 +2199,6 @@ __global__ void k_hop_lens(DevPtrs P, int *lens, int phase, long long arg, int i
     } else {                            // HL_TRANSPORT: start of the hop loop (arg = hop cap)
         cnt[CNT_VIRT] = 0;
         cnt[CNT_VESC] = 0;
-        cnt[CNT_GAS] = 0;
         for (int k = CNT_ACTP; k <= CNT_OUT; ++k) cnt[k] = 0;
         cnt[CNT_HOP] = 0;
         cnt[CNT_PKFREE] = 0;
@@ -2385,10 +2384,11 @@ static rt_status transport_end(rt_ctx *c, bool fp32) {
         double wls = (double)c->cnt_h[CNT_WLS], outs = (double)c->cnt_h[CNT_OUT];
         double vreq = (double)c->cnt_h[CNT_VIRT];
         // algorithmic bytes: each input read once and each output written once
-        c->kstat[KT_PHASE_A].bytes += actp * (kn * (4 + 4 + 12) + P.nf * 4) + acts * 12 * R +
-                                      gcon * 8 + (double)hops * (double)P.n * 4;
+        const double keys = (double)hops * (double)P.n * P.nf;   // words swept over the hops
+        c->kstat[KT_PHASE_A].bytes += keys * 4 + actp * kn * 20 + acts * 12 * R + gcon * 5;
+        c->kstat[KT_WORKLIST].bytes += keys * 21 + wls * 4;
         c->kstat[KT_PHASE_B].bytes += wls * (16 + 8 + 48 + kn * 4) + gcon * (16 + 6 * R + 4) +
-                                      stg * (8 + 9 * R) + outs * 6 * R;
+                                      stg * (12 + 8 * R) + outs * 6 * R;
         c->kstat[KT_VIRTUAL].bytes += vreq * (8 + 6 * R + 40 + kn * (16 + 4 * R + 16 + 4) +
                                               6 * R + 40);
     }
